@@ -120,7 +120,11 @@ static Lattice make_lattice() {
     }
     f.theta0 = (float)th0;
     f.inv_3theta0 = (float)(1.0 / (3.0 * th0));
-    for (int i = 0; i < kQ; ++i) L.lc.w41.w[i] = w41[i];
+    for (int i = 0; i < kQ; ++i) {
+        L.lc.w41.w[i] = w41[i];
+        L.lc.w41.chi[i] = (float)(1.0 / w41[i]);
+        L.lc.w41.clo[i] = (float)(1.0 / w41[i] - (double)L.lc.w41.chi[i]);
+    }
     L.lc.theta0 = th0;
     return L;
 }

@@ -1,5 +1,7 @@
 // Launchers of the non-step kernels: initialisation from fields, node
 // moments, global conservation sums and population format conversion.
+#include <algorithm>
+
 #include "lb_kernels.cuh"
 
 namespace gblb {
@@ -53,11 +55,11 @@ cudaError_t launch_init(int prec, int eq, void* dst, const Dims& d, const Launch
         const unsigned nb = blocks_for(count, 256);
         T* o = static_cast<T*>(dst);
         if (eq >= 2)  // the exact entropic equilibrium (kind 3 adds only the path length)
-            k_init<C, 2><<<nb, 256, 0, st>>>(o, d, consts_for<C>(c), c.theta0, q0, count, rho, u, ustride, theta, err);
+            k_init<C, 2><<<nb, 256, 0, st>>>(o, d, consts_for<C>(c), c.theta0, 1.0 / c.theta0, q0, count, rho, u, ustride, theta, err);
         else if (eq == 1)
-            k_init<C, 1><<<nb, 256, 0, st>>>(o, d, consts_for<C>(c), c.theta0, q0, count, rho, u, ustride, theta, err);
+            k_init<C, 1><<<nb, 256, 0, st>>>(o, d, consts_for<C>(c), c.theta0, 1.0 / c.theta0, q0, count, rho, u, ustride, theta, err);
         else
-            k_init<C, 0><<<nb, 256, 0, st>>>(o, d, consts_for<C>(c), c.theta0, q0, count, rho, u, ustride, theta, err);
+            k_init<C, 0><<<nb, 256, 0, st>>>(o, d, consts_for<C>(c), c.theta0, 1.0 / c.theta0, q0, count, rho, u, ustride, theta, err);
         return cudaGetLastError();
     });
 }
@@ -74,24 +76,10 @@ cudaError_t launch_moments(int prec, const void* src, const Dims& d, const Launc
     });
 }
 
-// Sum of the per-block partials in a fixed order: thread t adds blocks
-// t, t + 256, ... then a shared-memory tree.
 __global__ void __launch_bounds__(kRedThreads) k_reduce_partials(const double* __restrict__ partials, int nblocks,
                                                                   double* __restrict__ out5) {
     __shared__ double sh[5][kRedThreads];
-    double acc[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-    for (int b = threadIdx.x; b < nblocks; b += kRedThreads)
-#pragma unroll
-        for (int k = 0; k < 5; ++k) acc[k] += partials[(int64_t)b * 5 + k];
-#pragma unroll
-    for (int k = 0; k < 5; ++k) sh[k][threadIdx.x] = acc[k];
-    __syncthreads();
-    for (int w = kRedThreads / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w)
-#pragma unroll
-            for (int k = 0; k < 5; ++k) sh[k][threadIdx.x] += sh[k][threadIdx.x + w];
-        __syncthreads();
-    }
+    reduce_partials(partials, nblocks, sh);
     if (threadIdx.x == 0)
 #pragma unroll
         for (int k = 0; k < 5; ++k) out5[k] = sh[k][0];
@@ -100,15 +88,20 @@ __global__ void __launch_bounds__(kRedThreads) k_reduce_partials(const double* _
 cudaError_t launch_conserved(int prec, const void* src, const Dims& d, const LaunchConsts& c, double* partials,
                              int nblocks, double* out5, cudaStream_t st, int64_t z0, int64_t nzr) {
     if (nzr < 0) nzr = d.nz;
+    int nb = nblocks;  // room for four blocks per SM: one wave of this codec's kernel
     cudaError_t e = dispatch(prec, [&](auto codec) {
         using C = decltype(codec);
         using T = typename C::raw_t;
-        k_conserved<C><<<nblocks, kRedThreads, 0, st>>>(static_cast<const T*>(src), d, consts_for<C>(c), partials, z0,
-                                                         nzr);
+        const T* f = static_cast<const T*>(src);
+        nb = std::max(1, nblocks / 4 * sum_blocks_per_sm<C>());
+        if (sum_vector_ok<C>(src, d))
+            k_conserved<C, sum_width<C>()><<<nb, kRedThreads, 0, st>>>(f, d, consts_for<C>(c), partials, z0, nzr);
+        else
+            k_conserved<C, 1><<<nb, kRedThreads, 0, st>>>(f, d, consts_for<C>(c), partials, z0, nzr);
         return cudaGetLastError();
     });
     if (e != cudaSuccess) return e;
-    k_reduce_partials<<<1, kRedThreads, 0, st>>>(partials, nblocks, out5);
+    k_reduce_partials<<<1, kRedThreads, 0, st>>>(partials, nb, out5);
     return cudaGetLastError();
 }
 
@@ -142,13 +135,19 @@ cudaError_t launch_halo_copy(int prec, void* f, const Dims& d, const HaloList& l
     return cudaGetLastError();
 }
 
+// Blocks of k_to_f64 / k_from_f64: one row of blocks for each plane that [e0, e0 + count) touches.
+static dim3 plane_grid(int64_t plane, int64_t e0, int64_t count) {
+    return dim3(blocks_for(plane, kConvPer * 256), (unsigned)((e0 + count - 1) / plane - e0 / plane + 1));
+}
+
 cudaError_t launch_to_f64(int prec, const void* src, const Dims& d, const LaunchConsts& c, int64_t e0, int64_t count,
                           double* f, cudaStream_t st) {
     if (count <= 0) return cudaSuccess;
     return dispatch(prec, [&](auto codec) {
         using C = decltype(codec);
         using T = typename C::raw_t;
-        k_to_f64<C><<<blocks_for(count, 256), 256, 0, st>>>(static_cast<const T*>(src), d.plane, c.w41, e0, count, f);
+        k_to_f64<C><<<plane_grid(d.plane, e0, count), 256, 0, st>>>(static_cast<const T*>(src), d.plane, c.w41, e0,
+                                                                   count, f);
         return cudaGetLastError();
     });
 }
@@ -159,7 +158,8 @@ cudaError_t launch_from_f64(int prec, const double* f, void* dst, const Dims& d,
     return dispatch(prec, [&](auto codec) {
         using C = decltype(codec);
         using T = typename C::raw_t;
-        k_from_f64<C><<<blocks_for(count, 256), 256, 0, st>>>(f, d.plane, c.w41, e0, count, static_cast<T*>(dst));
+        k_from_f64<C><<<plane_grid(d.plane, e0, count), 256, 0, st>>>(f, d.plane, c.w41, e0, count,
+                                                                     static_cast<T*>(dst));
         return cudaGetLastError();
     });
 }

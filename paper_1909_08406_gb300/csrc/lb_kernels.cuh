@@ -413,9 +413,10 @@ __global__ void __launch_bounds__(kStepThreads, MINB) k_step2x(const typename Co
 // pointers are indexed by q - q0 (u component c at c * ustride + q - q0).
 template <class Codec, int EQ>
 __global__ void __launch_bounds__(256) k_init(typename Codec::raw_t* __restrict__ dst, Dims d, Consts<typename Codec::R> K,
-                                              double theta0, int64_t q0, int64_t count, const double* __restrict__ rho,
-                                              const double* __restrict__ u, int64_t ustride,
-                                              const double* __restrict__ theta, int* __restrict__ err) {
+                                              double theta0, double inv_theta0, int64_t q0, int64_t count,
+                                              const double* __restrict__ rho, const double* __restrict__ u,
+                                              int64_t ustride, const double* __restrict__ theta,
+                                              int* __restrict__ err) {
     using R = typename Codec::R;
     const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= count) return;
@@ -428,7 +429,7 @@ __global__ void __launch_bounds__(256) k_init(typename Codec::raw_t* __restrict_
     st.ux = (R)u[k];
     st.uy = (R)u[ustride + k];
     st.uz = (R)u[2 * ustride + k];
-    st.eta = (R)(theta[k] / theta0 - 1.0);
+    st.eta = (R)((theta[k] - theta0) * inv_theta0);
     bool ok = state_ok(st);
     R zero[kQ];
 #pragma unroll
@@ -477,29 +478,69 @@ __global__ void __launch_bounds__(256) k_moments(const typename Codec::raw_t* __
 
 constexpr int kRedThreads = 256;
 
-// Per-block FP64 partial sums of (drho, jx, jy, jz, dk) over all nodes, in a
-// fixed order (grid-stride loop, then a shared-memory tree): deterministic
-// for a given grid size.
-template <class Codec>
-// Over the planes [z0, z0 + nzr) of both sub-lattices (all of them: z0 = 0, nzr = nz).
-__global__ void __launch_bounds__(kRedThreads) k_conserved(const typename Codec::raw_t* __restrict__ src, Dims d,
-                                                           Consts<typename Codec::R> K, double* __restrict__ partials,
-                                                           int64_t z0, int64_t nzr) {
-    using R = typename Codec::R;
-    double acc[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-    const int64_t nxy = (int64_t)d.nx * d.ny, span = nzr * nxy, n = 2 * span;
-    for (int64_t j = (int64_t)blockIdx.x * kRedThreads + threadIdx.x; j < n; j += (int64_t)gridDim.x * kRedThreads) {
-        int64_t q = j;
-        if (nzr != d.nz) {
-            const int64_t s = j / span;
-            q = s * d.plane + z0 * nxy + (j - s * span);
-        }
-        const NodeMoments<R> m = node_moments_at<Codec>(src, d, q, K);
+// The five sums (drho, jx, jy, jz, dk) of the V consecutive nodes that start at node q, as FP64
+// additions to acc.  V = 2 (FP32 arithmetic): one aligned two-element load per population, packed
+// FP32x2 arithmetic; each node's five values are the ones V = 1 forms.
+template <class Codec, int V>
+__device__ __forceinline__ void add_node_sums(const typename Codec::raw_t* __restrict__ src, const Dims& d, int64_t q,
+                                              const Consts<typename Codec::R>& K, double (&acc)[5]) {
+    if constexpr (V == 1) {
+        const NodeMoments<typename Codec::R> m = node_moments_at<Codec>(src, d, q, K);
         acc[0] += (double)m.drho;
         acc[1] += (double)m.jx;
         acc[2] += (double)m.jy;
         acc[3] += (double)m.jz;
         acc[4] += (double)m.dk;
+    } else {
+        using P = typename Codec::pair_t;
+        const int s = q >= d.plane;
+        const typename Codec::raw_t* base = src + (int64_t)s * (kQ - 1) * d.plane + q;
+        P v[kQ];
+        static_for<kQ>([&](auto I) { v[I] = __ldg(reinterpret_cast<const P*>(base + (int64_t)I * d.plane)); });
+        constexpr float inv_scale = (float)(1.0 / Codec::kScale);
+        const NodeMoments<F2> m = moments_from<F2>(
+            [&](auto I) { return F2(K.w[vel(I).shell] * inv_scale) * F2(Codec::unpack2(v[I])); });
+        const F2 part[5] = {m.drho, m.jx, m.jy, m.jz, m.dk};
+#pragma unroll
+        for (int k = 0; k < 5; ++k) {
+            acc[k] += (double)part[k].v.x;
+            acc[k] += (double)part[k].v.y;
+        }
+    }
+}
+
+template <class Codec>
+constexpr int sum_width() {
+    return sizeof(typename Codec::R) == 4 ? 2 : 1;
+}
+// Resident blocks per SM that the summing kernel's registers are sized for (80 and up to 128 a
+// thread, so that a node's 41 loads are in flight together); its grid is one wave of them.
+template <class Codec>
+constexpr int sum_blocks_per_sm() {
+    return sizeof(typename Codec::raw_t) == 2 ? 3 : 2;
+}
+// The paired loads need an even number of nodes in every plane and an aligned base.
+template <class Codec>
+inline bool sum_vector_ok(const void* src, const Dims& d) {
+    constexpr int V = sum_width<Codec>();
+    return V > 1 && ((int64_t)d.nx * d.ny) % V == 0 &&
+           reinterpret_cast<uintptr_t>(src) % (V * sizeof(typename Codec::raw_t)) == 0;
+}
+
+// Per-block FP64 partial sums of (drho, jx, jy, jz, dk) over all nodes, in a
+// fixed order (grid-stride loop, then a shared-memory tree): deterministic
+// for a given grid size.
+// Over the planes [z0, z0 + nzr) of both sub-lattices (all of them: z0 = 0, nzr = nz).
+template <class Codec, int V>
+__global__ void __launch_bounds__(kRedThreads, sum_blocks_per_sm<Codec>())
+    k_conserved(const typename Codec::raw_t* __restrict__ src, Dims d, Consts<typename Codec::R> K,
+                double* __restrict__ partials, int64_t z0, int64_t nzr) {
+    double acc[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+    const int64_t nxy = (int64_t)d.nx * d.ny, span = nzr * nxy, n = 2 * span;
+    for (int64_t j = ((int64_t)blockIdx.x * kRedThreads + threadIdx.x) * V; j < n;
+         j += (int64_t)gridDim.x * kRedThreads * V) {
+        const int64_t q = j < span ? z0 * nxy + j : d.plane + z0 * nxy + (j - span);
+        add_node_sums<Codec, V>(src, d, q, K, acc);
     }
     __shared__ double sh[5][kRedThreads];
 #pragma unroll
@@ -516,35 +557,109 @@ __global__ void __launch_bounds__(kRedThreads) k_conserved(const typename Codec:
         for (int k = 0; k < 5; ++k) partials[(int64_t)blockIdx.x * 5 + k] = sh[k][0];
 }
 
+// Sum of the per-block partials in a fixed order: thread t adds blocks t, t + 256, ..., then a
+// shared-memory tree; sh[k][0] holds the five sums.
+__device__ __forceinline__ void reduce_partials(const double* __restrict__ partials, int nblocks,
+                                                double (&sh)[5][kRedThreads]) {
+    double acc[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+    for (int b = threadIdx.x; b < nblocks; b += kRedThreads)
+#pragma unroll
+        for (int k = 0; k < 5; ++k) acc[k] += partials[(int64_t)b * 5 + k];
+#pragma unroll
+    for (int k = 0; k < 5; ++k) sh[k][threadIdx.x] = acc[k];
+    __syncthreads();
+    for (int w = kRedThreads / 2; w > 0; w >>= 1) {
+        if (threadIdx.x < w)
+#pragma unroll
+            for (int k = 0; k < 5; ++k) sh[k][threadIdx.x] += sh[k][threadIdx.x + w];
+        __syncthreads();
+    }
+}
+
+// Bits of an FP32 number as the FP64 number of the same value, formed with integer operations where
+// the number is normal or zero (GB300 converts and adds FP64 at 1/64 of its FP32 rate).
+__device__ __forceinline__ double widen(float v) {
+    const uint32_t u = __float_as_uint(v), e = (u >> 23) & 0xffu;
+    if (e - 1u < 254u) return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(u << 29));
+    return (double)v;
+}
+
+// c d of an FP64 number d and c = chi + clo as an FP32 number, |error| below (1/2 + 2^-20) ulp:
+// d splits exactly into its upper 24 and lower 29 bits (integer operations), the product is formed
+// in two FP32 terms.  Exponents outside [-70, 60] (and zero, infinities, NaN) take FP64 arithmetic.
+__device__ __forceinline__ float scale_to_float(double d, float chi, float clo) {
+    const uint32_t h = (uint32_t)__double2hiint(d), l = (uint32_t)__double2loint(d);
+    const uint32_t e = (h >> 20) & 0x7ffu;
+    if (e - 953u > 130u) return (float)(d * ((double)chi + (double)clo));
+    const uint32_t sign = h & 0x80000000u;
+    const float hi = __uint_as_float(sign | ((e - 896u) << 23) | ((h & 0xfffffu) << 3) | (l >> 29));
+    // the lower 29 bits in units of 2^(e - 1023 - 52)
+    const float unit = __uint_as_float(sign | ((e - 896u - 52u) << 23));
+    const float lo = __uint2float_rn(l & 0x1fffffffu) * unit;
+    const float p = hi * chi;
+    float r = fmaf(hi, chi, -p);
+    r = fmaf(hi, clo, r);
+    r = fmaf(lo, chi, r);
+    return p + r;
+}
+
 // Raw storage <-> float64 populations for elements e in [e0, e0 + count) of the
-// [s][41][nz][ny][nx] array; the float64 side is indexed by e - e0.
+// [s][41][nz][ny][nx] array; the float64 side is indexed by e - e0.  blockIdx.y counts the
+// (sub-lattice, population) planes from the one that holds e0, so that the weight is uniform in a
+// block and no element index is divided; a block covers kConvPer x 256 elements of its plane, each
+// thread kConvPer of them 256 apart.
+constexpr int kConvPer = 4;
+
+template <class F>
+__device__ __forceinline__ void for_plane_elements(int64_t plane, int64_t e0, int64_t count, F&& body) {
+    const int64_t p = e0 / plane + blockIdx.y, first = p * plane;
+    const int i = (int)(p % kQ);
+    const int64_t lo = max(first, e0), hi = min(first + plane, e0 + count);
+    const int64_t e = first + (int64_t)blockIdx.x * (kConvPer * 256) + threadIdx.x;
+    body(i, e, lo, hi);
+}
+
+// FP64 work per element: one fused multiply-add (from storage), one subtraction (to storage); the
+// conversions and the scaling are FP32 and integer operations.
 template <class Codec>
 __global__ void __launch_bounds__(256) k_to_f64(const typename Codec::raw_t* __restrict__ src, int64_t plane, W41 w,
                                                 int64_t e0, int64_t count, double* __restrict__ f) {
-    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= count) return;
-    const int64_t e = e0 + k;
-    const int i = (int)((e / plane) % kQ);
-    const double v = (double)Codec::value(src[e]);
-    if constexpr (Codec::stores_f)
-        f[k] = v;
-    else
-        f[k] = w.w[i] * (1.0 + v * (1.0 / Codec::kScale));
+    for_plane_elements(plane, e0, count, [&](int i, int64_t e, int64_t lo, int64_t hi) {
+        const double wi = w.w[i], ws = wi * (1.0 / Codec::kScale);
+        typename Codec::raw_t r[kConvPer];
+#pragma unroll
+        for (int k = 0; k < kConvPer; ++k)
+            if (e + 256 * k >= lo && e + 256 * k < hi) r[k] = src[e + 256 * k];
+#pragma unroll
+        for (int k = 0; k < kConvPer; ++k) {
+            if (e + 256 * k < lo || e + 256 * k >= hi) continue;
+            if constexpr (Codec::stores_f)
+                f[e + 256 * k - e0] = r[k];
+            else
+                f[e + 256 * k - e0] = fma(widen(Codec::value(r[k])), ws, wi);
+        }
+    });
 }
 
 template <class Codec>
 __global__ void __launch_bounds__(256) k_from_f64(const double* __restrict__ f, int64_t plane, W41 w, int64_t e0,
                                                   int64_t count, typename Codec::raw_t* __restrict__ dst) {
-    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= count) return;
-    const int64_t e = e0 + k;
-    const int i = (int)((e / plane) % kQ);
-    double h;
-    if constexpr (Codec::stores_f)
-        h = f[k];
-    else
-        h = (f[k] - w.w[i]) / w.w[i] * Codec::kScale;
-    dst[e] = Codec::to_raw((typename Codec::R)h);
+    for_plane_elements(plane, e0, count, [&](int i, int64_t e, int64_t lo, int64_t hi) {
+        const double wi = w.w[i];
+        const float chi = w.chi[i] * (float)Codec::kScale, clo = w.clo[i] * (float)Codec::kScale;
+        double v[kConvPer];
+#pragma unroll
+        for (int k = 0; k < kConvPer; ++k)
+            if (e + 256 * k >= lo && e + 256 * k < hi) v[k] = f[e + 256 * k - e0];
+#pragma unroll
+        for (int k = 0; k < kConvPer; ++k) {
+            if (e + 256 * k < lo || e + 256 * k >= hi) continue;
+            if constexpr (Codec::stores_f)
+                dst[e + 256 * k] = v[k];
+            else
+                dst[e + 256 * k] = Codec::to_raw(scale_to_float(v[k] - wi, chi, clo));
+        }
+    });
 }
 
 }  // namespace gblb

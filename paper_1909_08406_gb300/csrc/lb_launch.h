@@ -10,6 +10,7 @@ namespace gblb {
 
 struct W41 {
     double w[kQ];  // per-population weights, library order
+    float chi[kQ], clo[kQ];  // 1 / w as the sum of two FP32 numbers
 };
 
 struct LaunchConsts {
