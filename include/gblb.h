@@ -228,7 +228,7 @@ lb_status lb_set_state(lb_ctx *ctx, const void *raw, int on_device);
  *   LB_KERNEL_DIRECT1  one node per thread, direct global loads
  *   LB_KERNEL_DIRECT2  two rows per thread, packed FP32x2 arithmetic (not FP64;
  *                      ny even, nx*ny*nz < 2^32)
- *   LB_KERNEL_DIRECT2R the same with a register budget for 4 CTAs per SM
+ *   LB_KERNEL_DIRECT2R the same with a register budget for 3 CTAs per SM instead of 4
  *   LB_KERNEL_STAGED   tiles of 128/256 x fetched by TMA bulk copies into a
  *                      shared-memory ring (not FP64; nx a multiple of 128 and
  *                      of 16 bytes)

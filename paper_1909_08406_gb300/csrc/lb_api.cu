@@ -67,19 +67,20 @@ static Lattice make_lattice() {
         pk[s][1] = k.p1[s];
         pk[s][2] = k.p2[s];
         pk[s][3] = k.p3[s];
+        double n2 = 0, n4 = 0, n22 = 0;
         for (int i = 0; i < kQ; ++i) {
             if (vel(i).shell != s) continue;
             const double cx = 0.5 * vel(i).x, cy = 0.5 * vel(i).y;
-            k.n2[s] += cx * cx;
-            k.n4[s] += cx * cx * cx * cx;
-            k.n22[s] += cx * cx * cy * cy;
+            n2 += cx * cx;
+            n4 += cx * cx * cx * cx;
+            n22 += cx * cx * cy * cy;
         }
         // the projection's shell sums folded into cubics in eta
         for (int p = 0; p < 4; ++p) {
-            k.pj[0][p] += k.w[s] * k.n2[s] * pk[s][p];
-            k.pj[1][p] += k.w[s] * k.n2[s] * csq * pk[s][p];
-            k.pj[2][p] += k.w[s] * k.n4[s] * pk[s][p];
-            k.pj[3][p] += k.w[s] * k.n22[s] * pk[s][p];
+            k.pj[0][p] += k.w[s] * n2 * pk[s][p];
+            k.pj[1][p] += k.w[s] * n2 * csq * pk[s][p];
+            k.pj[2][p] += k.w[s] * n4 * pk[s][p];
+            k.pj[3][p] += k.w[s] * n22 * pk[s][p];
         }
     }
     double A[4] = {0, 0, 0, 0}, B[4] = {0, 0, 0, 0};
@@ -108,9 +109,6 @@ static Lattice make_lattice() {
         f.p1[s] = (float)k.p1[s];
         f.p2[s] = (float)k.p2[s];
         f.p3[s] = (float)k.p3[s];
-        f.n2[s] = (float)k.n2[s];
-        f.n4[s] = (float)k.n4[s];
-        f.n22[s] = (float)k.n22[s];
     }
     for (int j = 0; j < 4; ++j)
         for (int p = 0; p < 4; ++p) f.pj[j][p] = (float)k.pj[j][p];
@@ -120,6 +118,43 @@ static Lattice make_lattice() {
     }
     f.theta0 = (float)th0;
     f.inv_3theta0 = (float)(1.0 / (3.0 * th0));
+    auto step = [&](double scale, bool stores_f) {
+        StepConsts<double> q;
+        memset(&q, 0, sizeof q);
+        for (int s = 0; s < kShells; ++s) {
+            const double e = k.c2[s] - 3.0 * th0;
+            q.w[s] = stores_f ? (s ? 2.0 : 1.0) * k.w[s] : k.w[s] / scale;
+            q.de[s] = stores_f ? e : k.w[s] * e / scale;
+            q.c2[s] = k.c2[s];
+            for (int p = 0; p < 4; ++p) q.rp[s][p] = (stores_f ? k.w[s] : 1.0) * pk[s][p];
+        }
+        q.j2 = 2.0 * k.w[2] / scale;
+        q.j5 = 0.5 * k.w[5] / scale;
+        for (int p = 0; p < 4; ++p) {
+            q.m2[p] = k.m2[p];
+            q.m2p[p] = k.m2p[p];
+            q.pj0[p] = k.pj[0][p];
+            q.pj1[p] = k.pj[1][p];
+            q.pj3[p] = k.pj[3][p];
+            q.pq[p] = k.pj[2][p] - 3.0 * k.pj[3][p];
+        }
+        q.inv_theta0 = 1.0 / th0;
+        q.inv_3theta0 = 1.0 / (3.0 * th0);
+        return q;
+    };
+    L.lc.sd = step(1.0, true);
+    for (int h = 0; h < 2; ++h) {
+        const StepConsts<double> q = step(h ? CodecF16::kScale : 1.0, false);
+        constexpr size_t n = sizeof q / sizeof(double);
+        static_assert(sizeof(StepConsts<float2>) == n * sizeof(float2), "plain arrays of constants");
+        const double* from = reinterpret_cast<const double*>(&q);
+        float* one = reinterpret_cast<float*>(&L.lc.sf[h]);
+        float2* two = reinterpret_cast<float2*>(&L.lc.sp[h]);
+        for (size_t i = 0; i < n; ++i) {
+            one[i] = (float)from[i];
+            two[i] = make_float2(one[i], one[i]);
+        }
+    }
     for (int i = 0; i < kQ; ++i) {
         L.lc.w41.w[i] = w41[i];
         L.lc.w41.chi[i] = (float)(1.0 / w41[i]);

@@ -16,14 +16,6 @@ size_t storage_bytes(int prec) {
     }
 }
 
-template <class Codec>
-static const Consts<typename Codec::R>& consts_for(const LaunchConsts& c) {
-    if constexpr (std::is_same<typename Codec::R, double>::value)
-        return c.kd;
-    else
-        return c.kf;
-}
-
 // Calls f.template operator()<Codec>() for the codec of prec.
 template <class F>
 static cudaError_t dispatch(int prec, F&& f) {
@@ -55,11 +47,11 @@ cudaError_t launch_init(int prec, int eq, void* dst, const Dims& d, const Launch
         const unsigned nb = blocks_for(count, 256);
         T* o = static_cast<T*>(dst);
         if (eq >= 2)  // the exact entropic equilibrium (kind 3 adds only the path length)
-            k_init<C, 2><<<nb, 256, 0, st>>>(o, d, consts_for<C>(c), c.theta0, 1.0 / c.theta0, q0, count, rho, u, ustride, theta, err);
+            k_init<C, 2><<<nb, 256, 0, st>>>(o, d, consts_of<C>(c), c.theta0, 1.0 / c.theta0, q0, count, rho, u, ustride, theta, err);
         else if (eq == 1)
-            k_init<C, 1><<<nb, 256, 0, st>>>(o, d, consts_for<C>(c), c.theta0, 1.0 / c.theta0, q0, count, rho, u, ustride, theta, err);
+            k_init<C, 1><<<nb, 256, 0, st>>>(o, d, consts_of<C>(c), c.theta0, 1.0 / c.theta0, q0, count, rho, u, ustride, theta, err);
         else
-            k_init<C, 0><<<nb, 256, 0, st>>>(o, d, consts_for<C>(c), c.theta0, 1.0 / c.theta0, q0, count, rho, u, ustride, theta, err);
+            k_init<C, 0><<<nb, 256, 0, st>>>(o, d, consts_of<C>(c), c.theta0, 1.0 / c.theta0, q0, count, rho, u, ustride, theta, err);
         return cudaGetLastError();
     });
 }
@@ -70,7 +62,7 @@ cudaError_t launch_moments(int prec, const void* src, const Dims& d, const Launc
     return dispatch(prec, [&](auto codec) {
         using C = decltype(codec);
         using T = typename C::raw_t;
-        k_moments<C><<<blocks_for(count, 256), 256, 0, st>>>(static_cast<const T*>(src), d, consts_for<C>(c), c.theta0,
+        k_moments<C><<<blocks_for(count, 256), 256, 0, st>>>(static_cast<const T*>(src), d, consts_of<C>(c), c.theta0,
                                                               q0, count, rho, u, ustride, theta);
         return cudaGetLastError();
     });
@@ -95,9 +87,9 @@ cudaError_t launch_conserved(int prec, const void* src, const Dims& d, const Lau
         const T* f = static_cast<const T*>(src);
         nb = std::max(1, nblocks / 4 * sum_blocks_per_sm<C>());
         if (sum_vector_ok<C>(src, d))
-            k_conserved<C, sum_width<C>()><<<nb, kRedThreads, 0, st>>>(f, d, consts_for<C>(c), partials, z0, nzr);
+            k_conserved<C, sum_width<C>()><<<nb, kRedThreads, 0, st>>>(f, d, consts_of<C>(c), partials, z0, nzr);
         else
-            k_conserved<C, 1><<<nb, kRedThreads, 0, st>>>(f, d, consts_for<C>(c), partials, z0, nzr);
+            k_conserved<C, 1><<<nb, kRedThreads, 0, st>>>(f, d, consts_of<C>(c), partials, z0, nzr);
         return cudaGetLastError();
     });
     if (e != cudaSuccess) return e;

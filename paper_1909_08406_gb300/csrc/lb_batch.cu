@@ -123,7 +123,7 @@ __device__ __forceinline__ double tb_of<double>(const BatchSim& s) {
 // read, in step k + 1, lines another CTA wrote in step k).
 template <class Codec, bool PROJECT, class Ld>
 __device__ __forceinline__ void batch_tile(const BatchSim* __restrict__ sims, int nsims, int64_t t, int parity,
-                                           const Consts<typename Codec::R>& K, int tx, int txs, int ry, int* err) {
+                                           const StepConsts<typename Codec::R>& K, int tx, int txs, int ry, int* err) {
     using R = typename Codec::R;
     using T = typename Codec::raw_t;
     const BatchSim& S = sims[find_sim(sims, nsims, t)];
@@ -138,7 +138,7 @@ __device__ __forceinline__ void batch_tile(const BatchSim* __restrict__ sims, in
 // (y + 1, x) with packed FP32x2 arithmetic.
 template <class Codec, bool PROJECT, class Ld>
 __device__ __forceinline__ void batch_tile2(const BatchSim* __restrict__ sims, int nsims, int64_t t, int parity,
-                                            const Consts<float>& K, int tx, int txs, int ry, int* err) {
+                                            const StepConsts<float2>& K, int tx, int txs, int ry, int* err) {
     using T = typename Codec::raw_t;
     const BatchSim& S = sims[find_sim(sims, nsims, t)];
     int s, z, y, x;
@@ -156,9 +156,13 @@ constexpr int batch_min_blocks(bool persistent) {
     return (TWO || sizeof(typename Codec::R) == 8) ? 3 : (persistent ? 6 : 6);
 }
 
+// Constants of the one-node and of the packed two-node update.
+template <class Codec, bool TWO>
+using BatchK = StepConsts<std::conditional_t<TWO, float2, typename Codec::R>>;
+
 template <class Codec, bool PROJECT, bool TWO>
 __global__ void __launch_bounds__(128, batch_min_blocks<Codec, TWO>(false)) k_batch_step(const BatchSim* __restrict__ sims, int nsims, int parity,
-                                                    Consts<typename Codec::KS> K, int tx, int txs, int ry, int* err) {
+                                                    BatchK<Codec, TWO> K, int tx, int txs, int ry, int* err) {
     if constexpr (TWO)
         batch_tile2<Codec, PROJECT, LoadNC>(sims, nsims, blockIdx.x, parity, K, tx, txs, ry, err);
     else
@@ -204,7 +208,7 @@ __device__ __forceinline__ bool grid_sync(GridBar* bar, unsigned expected, long 
 template <class Codec, bool PROJECT, bool TWO>
 __global__ void __launch_bounds__(128, batch_min_blocks<Codec, TWO>(true))
     k_batch_persistent(const BatchSim* __restrict__ sims, int nsims, int64_t ntiles, int64_t nsteps, int parity0,
-                       Consts<typename Codec::KS> K, int tx, int txs, int ry, int* err, GridBar* bar,
+                       BatchK<Codec, TWO> K, int tx, int txs, int ry, int* err, GridBar* bar,
                        unsigned expected, long long limit) {
     const int nt = (int)ntiles;  // < 2^31 (the work list is checked when it is laid out)
     for (int64_t step = 0; step < nsteps; ++step) {
@@ -231,14 +235,6 @@ static cudaError_t dispatch_codec(int prec, F&& f) {
         case kBF16: return f(CodecBF16{});
         default: return cudaErrorInvalidValue;
     }
-}
-
-template <class Codec>
-static const Consts<typename Codec::KS>& consts_of(const LaunchConsts& c) {
-    if constexpr (std::is_same<typename Codec::KS, double>::value)
-        return c.kd;
-    else
-        return c.kf;
 }
 
 }  // namespace gblb
@@ -354,19 +350,20 @@ static cudaError_t launch_batch_step(lb_batch* b, int parity, cudaStream_t st) {
         if constexpr (std::is_same<typename C::R, float>::value) {
             if (P.two_rows) {
                 if (b->project)
-                    k_batch_step<C, true, true><<<grid, block, 0, st>>>(P.d_sims, b->n, parity, consts_of<C>(lc),
+                    k_batch_step<C, true, true><<<grid, block, 0, st>>>(P.d_sims, b->n, parity, pair_consts<C>(lc),
                                                                         P.tx, log2i(P.tx), P.ry, b->d_err);
                 else
-                    k_batch_step<C, false, true><<<grid, block, 0, st>>>(P.d_sims, b->n, parity, consts_of<C>(lc),
+                    k_batch_step<C, false, true><<<grid, block, 0, st>>>(P.d_sims, b->n, parity, pair_consts<C>(lc),
                                                                          P.tx, log2i(P.tx), P.ry, b->d_err);
                 return cudaGetLastError();
             }
         }
+        const StepConsts<typename C::R>& one = step_consts<C, 1>(lc);
         if (b->project)
-            k_batch_step<C, true, false><<<grid, block, 0, st>>>(P.d_sims, b->n, parity, consts_of<C>(lc), P.tx,
+            k_batch_step<C, true, false><<<grid, block, 0, st>>>(P.d_sims, b->n, parity, one, P.tx,
                                                                  log2i(P.tx), P.ry, b->d_err);
         else
-            k_batch_step<C, false, false><<<grid, block, 0, st>>>(P.d_sims, b->n, parity, consts_of<C>(lc), P.tx,
+            k_batch_step<C, false, false><<<grid, block, 0, st>>>(P.d_sims, b->n, parity, one, P.tx,
                                                                   log2i(P.tx), P.ry, b->d_err);
         return cudaGetLastError();
     });
@@ -376,12 +373,15 @@ static cudaError_t launch_persistent(lb_batch* b, int64_t nsteps, int parity, cu
     const LaunchConsts& lc = lattice_consts();
     return dispatch_codec(b->prec, [&](auto codec) -> cudaError_t {
         using C = decltype(codec);
-        void (*kern)(const BatchSim*, int, int64_t, int64_t, int, Consts<typename C::KS>, int, int, int, int*,
-                     GridBar*, unsigned, long long) =
-            b->project ? k_batch_persistent<C, true, false> : k_batch_persistent<C, false, false>;
+        const void* kern = b->project ? (const void*)k_batch_persistent<C, true, false>
+                                      : (const void*)k_batch_persistent<C, false, false>;
+        const void* K = &step_consts<C, 1>(lc);
         if constexpr (std::is_same<typename C::R, float>::value) {
-            if (b->pp.two_rows)
-                kern = b->project ? k_batch_persistent<C, true, true> : k_batch_persistent<C, false, true>;
+            if (b->pp.two_rows) {
+                kern = b->project ? (const void*)k_batch_persistent<C, true, true>
+                                  : (const void*)k_batch_persistent<C, false, true>;
+                K = &pair_consts<C>(lc);
+            }
         }
         int per_sm = 0;
         const lb_batch::Plan& P = b->pp;
@@ -397,12 +397,11 @@ static cudaError_t launch_persistent(lb_batch* b, int64_t nsteps, int parity, cu
         const BatchSim* sims = P.d_sims;
         int nsims = b->n;
         int64_t ntiles = P.ntiles;
-        Consts<typename C::KS> K = consts_of<C>(lc);
         int tx = P.tx, txs = log2i(P.tx), ry = P.ry;
         int* err = b->d_err;
         GridBar* bar = b->d_bar;
         long long limit = b->wait_limit;
-        void* args[] = {(void*)&sims, (void*)&nsims, (void*)&ntiles, (void*)&nsteps, (void*)&parity, (void*)&K,
+        void* args[] = {(void*)&sims, (void*)&nsims, (void*)&ntiles, (void*)&nsteps, (void*)&parity, const_cast<void*>(K),
                         (void*)&tx, (void*)&txs, (void*)&ry, (void*)&err, (void*)&bar, (void*)&expected,
                         (void*)&limit};
         cudaLaunchConfig_t cfg = {};
@@ -415,7 +414,7 @@ static cudaError_t launch_persistent(lb_batch* b, int64_t nsteps, int parity, cu
         attr[0].val.cooperative = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        return cudaLaunchKernelExC(&cfg, (const void*)kern, args);
+        return cudaLaunchKernelExC(&cfg, kern, args);
     });
 }
 

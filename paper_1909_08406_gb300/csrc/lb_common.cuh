@@ -78,13 +78,27 @@ struct Consts {
     //   pj[2](eta) = sum_s w_s n4_s R_s,       pj[3](eta) = sum_s w_s n22_s R_s,
     // pj[j](eta) = pj[j][0] + eta (pj[j][1] + eta (pj[j][2] + eta pj[j][3])).
     R pj[4][4];
-    R n2[kShells];   // sum over the shell of c_x^2 (the packed two-node path sums the shells directly)
-    R n4[kShells];   // sum over the shell of c_x^4
-    R n22[kShells];  // sum over the shell of c_x^2 c_y^2
     R m2[4];         // M_2  (1+eta)^2 = m2[0] + m2[1] eta + m2[2] eta^2 + m2[3] eta^3
     R m2p[4];        // M_2' (1+eta)^2 likewise
     R theta0;
     R inv_3theta0;
+};
+
+// What the series step needs, in the type it is used in: S = float or double, or float2 with each
+// constant twice, so that the packed two-node kernels read a constant pair in one load.
+// Deviation codecs (FP32 arithmetic), with the stored scale folded in:
+//   w = w_s / kScale, de = w_s (c_s^2 - 3 theta_0) / kScale, j2 = 2 w[2], j5 = w[5] / 2,
+//   rp = (unused, p1, p2, p3)
+// FP64, which stores f:
+//   w = 2 w_s (w[0] = w_0), de = c_s^2 - 3 theta_0, rp = w_s (1, p1, p2, p3): w_s R_s as a cubic
+template <class S>
+struct StepConsts {
+    S w[kShells], de[kShells], c2[kShells], j2, j5;
+    S rp[kShells][4];
+    S m2[4], m2p[4];                // as in Consts
+    S pj0[4], pj1[4], pj3[4];       // Consts::pj
+    S pq[4];                        // pj[2] - 3 pj[3]
+    S inv_theta0, inv_3theta0;
 };
 
 template <int... Is, class F>
@@ -188,8 +202,8 @@ struct F2 {
     __device__ __forceinline__ F2(float2 x) : v(x) {}
 };
 __device__ __forceinline__ F2 operator+(F2 a, F2 b) { return F2(__fadd2_rn(a.v, b.v)); }
-__device__ __forceinline__ F2 operator-(F2 a, F2 b) { return F2(__ffma2_rn(b.v, make_float2(-1.f, -1.f), a.v)); }
-__device__ __forceinline__ F2 operator-(F2 a) { return F2(__fmul2_rn(a.v, make_float2(-1.f, -1.f))); }
+__device__ __forceinline__ F2 operator-(F2 a) { return F2(make_float2(-a.v.x, -a.v.y)); }
+__device__ __forceinline__ F2 operator-(F2 a, F2 b) { return F2(__fadd2_rn(a.v, (-b).v)); }
 __device__ __forceinline__ F2 operator*(F2 a, F2 b) { return F2(__fmul2_rn(a.v, b.v)); }
 __device__ __forceinline__ F2 operator/(F2 a, F2 b) { return F2(a.v.x / b.v.x, a.v.y / b.v.y); }
 __device__ __forceinline__ F2& operator+=(F2& a, F2 b) {
@@ -211,11 +225,9 @@ template <class Base>
 struct Codec2 {
     using raw_t = typename Base::raw_t;
     using R = F2;
-    using KS = float;
+    using KS = float2;
     static constexpr bool stores_f = Base::stores_f;
     static constexpr double kScale = Base::kScale;
-    static __device__ __forceinline__ F2 dev(F2 v, F2 w) { return w * v; }
-    static __device__ __forceinline__ F2 relax(F2 v, F2 omb, F2 x, F2, F2) { return fma(omb, v, x); }
 };
 
 // Moments of one node from the deviations d_i = f_i - w_i (Sec. II):
@@ -295,6 +307,283 @@ __device__ __forceinline__ bool state_ok(const NodeState<F2>& st) {
            mb < 1e30f;
 }
 
+// Moments of one node as the fused step uses them: drho = rho - 1, j = rho u and
+// de = <f, c^2 - 3 theta_0>, summed by shells.
+template <class R>
+struct NodeSums {
+    R drho, jx, jy, jz, de;
+};
+
+// Sums of the working values v = vget(I).  Per +-c pair one sum and one difference; the pair sums are
+// added up by shell and weighted once per shell, and the differences are combined along the axes of
+// the fcc and bcc shells first (the four diagonals give all three components in seven additions):
+// about 100 operations a node, 115 in FP64, against 163 when every deviation is weighted and enters
+// drho, j and dk by itself.  FP64 stores f: its pair sums are deviations, (f+ - 2w) + f-, both steps
+// exact or within the rounding of f.  Every multiply-add is written as one, so that the scalar and the
+// packed two-node forms round alike.
+template <class Codec, class VGet>
+__device__ __forceinline__ NodeSums<typename Codec::R> node_sums(const StepConsts<typename Codec::KS>& K, VGet&& vget) {
+    using R = typename Codec::R;
+    constexpr bool kF = Codec::stores_f;
+    // sum and difference of the pair ip, ip + 1
+    auto pair = [&](auto IP, R& S, R& D) {
+        constexpr int ip = decltype(IP)::value;
+        const R vp = vget(std::integral_constant<int, ip>{}), vm = vget(std::integral_constant<int, ip + 1>{});
+        if constexpr (kF)
+            S = (vp - R(K.w[vel(ip).shell])) + vm;
+        else
+            S = vp + vm;
+        D = vp - vm;
+    };
+    NodeSums<R> m;
+    {
+        const R v0 = vget(std::integral_constant<int, 0>{});
+        if constexpr (kF) {
+            m.drho = v0 - R(K.w[0]);
+            m.de = m.drho * R(K.de[0]);
+        } else {
+            m.drho = R(K.w[0]) * v0;
+            m.de = R(K.de[0]) * v0;
+        }
+    }
+    // a finished shell's sum H enters drho and de
+    auto shell = [&](int s, R H) {
+        if constexpr (kF) {
+            m.drho = m.drho + H;
+            m.de = fma(H, R(K.de[s]), m.de);
+        } else {
+            m.drho = fma(R(K.w[s]), H, m.drho);
+            m.de = fma(R(K.de[s]), H, m.de);
+        }
+    };
+    {  // sc-1 (pairs 1, 3, 5) and sc-2 (7, 9, 11), axis by axis
+        R H1, H2;
+        auto axis = [&](auto A, R& j) {
+            constexpr int k = decltype(A)::value;
+            R S1, D1, S2, D2;
+            pair(std::integral_constant<int, 1 + 2 * k>{}, S1, D1);
+            pair(std::integral_constant<int, 7 + 2 * k>{}, S2, D2);
+            if constexpr (kF)
+                j = fma(R(2), D2, D1);
+            else
+                j = fma(R(K.w[1]), D1, R(K.j2) * D2);
+            H1 = k == 0 ? S1 : H1 + S1;
+            H2 = k == 0 ? S2 : H2 + S2;
+        };
+        axis(std::integral_constant<int, 0>{}, m.jx);
+        axis(std::integral_constant<int, 1>{}, m.jy);
+        axis(std::integral_constant<int, 2>{}, m.jz);
+        shell(1, H1);
+        shell(2, H2);
+    }
+    {  // fcc-1: (1, 1, 0), (1, -1, 0) and likewise in the xz and yz planes
+        R H;
+        auto plane = [&](auto IP, R& ja, R& jb) {
+            constexpr int ip = decltype(IP)::value;
+            R S1, D1, S2, D2;
+            pair(std::integral_constant<int, ip>{}, S1, D1);
+            pair(std::integral_constant<int, ip + 2>{}, S2, D2);
+            const R p = D1 + D2, n = D1 - D2, S = S1 + S2;
+            ja = kF ? ja + p : fma(R(K.w[3]), p, ja);
+            jb = kF ? jb + n : fma(R(K.w[3]), n, jb);
+            H = ip == 13 ? S : H + S;
+        };
+        plane(std::integral_constant<int, 13>{}, m.jx, m.jy);
+        plane(std::integral_constant<int, 17>{}, m.jx, m.jz);
+        plane(std::integral_constant<int, 21>{}, m.jy, m.jz);
+        shell(3, H);
+    }
+    {  // bcc-1 (pairs 25 ..) and bcc-1/2 (33 ..) along the diagonals (1,1,1) (1,1,-1) (1,-1,1) (-1,1,1)
+        R H4, H5;
+        auto diag = [&](auto KD) {
+            constexpr int k = decltype(KD)::value;
+            R S4, D4, S5, D5;
+            pair(std::integral_constant<int, 25 + 2 * k>{}, S4, D4);
+            pair(std::integral_constant<int, 33 + 2 * k>{}, S5, D5);
+            H4 = k == 0 ? S4 : H4 + S4;
+            H5 = k == 0 ? S5 : H5 + S5;
+            return kF ? fma(R(0.5), D5, D4) : fma(R(K.j5), D5, R(K.w[4]) * D4);
+        };
+        const R E0 = diag(std::integral_constant<int, 0>{}), E1 = diag(std::integral_constant<int, 1>{});
+        const R p = E0 + E1, r = E0 - E1;
+        m.jx = m.jx + p;
+        m.jy = m.jy + p;
+        m.jz = m.jz + r;
+        const R E2 = diag(std::integral_constant<int, 2>{}), E3 = diag(std::integral_constant<int, 3>{});
+        const R q = E2 - E3, t = E2 + E3;
+        m.jx = m.jx + q;
+        m.jy = m.jy - q;
+        m.jz = m.jz + t;
+        shell(4, H4);
+        shell(5, H5);
+    }
+    return m;
+}
+
+// Primitive variables from the shell sums: eta = (de / rho - u^2) / (3 theta_0).
+template <class R, class KS>
+__device__ __forceinline__ NodeState<R> state_from_sums(const NodeSums<R>& m, const StepConsts<KS>& K) {
+    NodeState<R> st;
+    st.drho = m.drho;
+    st.rho = R(1) + m.drho;
+    const R inv_rho = recip(st.rho);
+    st.ux = m.jx * inv_rho;
+    st.uy = m.jy * inv_rho;
+    st.uz = m.jz * inv_rho;
+    const R usq = fma(st.ux, st.ux, fma(st.uy, st.uy, st.uz * st.uz));
+    st.eta = fma(m.de, inv_rho, -usq) * R(K.inv_3theta0);
+    return st;
+}
+
+template <class Codec, class VGet>
+__device__ __forceinline__ NodeState<typename Codec::R> node_state(const StepConsts<typename Codec::KS>& K, VGet&& vget) {
+    return state_from_sums(node_sums<Codec>(K, vget), K);
+}
+
+// Equilibrium (Eq. feqGenU3, with the optional momentum projection) and BGK relaxation of one node, in
+// the fewest operations: v[i] the working values, tb = 2 beta kScale, omb = 1 - 2 beta; sink(I, value)
+// receives the new working value of population I.
+//
+// With up = u / theta, a = up.c and per shell R_s = f~_s / (w_s rho), C_s, D_s (see
+// equilibrium_relax_g), a pair's relaxation is
+//   v'_+- = omb v_+- + T +- P (a (D_s + a^2 / 6) + c.v),  T = B_s + P a^2 / 2,
+//   P = tb rho R_s,  B_s = tb (rho R_s - 1) + P C_s      (deviation codecs)
+//   P = tb w_s rho R_s,  B_s = P (1 + C_s)               (FP64, which stores f)
+// i.e. four multiply-adds for the pair's common terms and two for each population.  Pairs of one
+// direction in two shells (sc-1 and sc-2, bcc-1 and bcc-1/2) share a and a^2: with a = k a_1 the factors
+// k and k^2 go into the shell constants.  The projection v = dj / (rho theta) is odd in u along each
+// axis: v_a = -up_a (K0 + K1 up_a^2).  About 300 operations a node, against 520 for the direct form.
+// RELAX false: sink receives tb h^eq_i (f^eq_i for FP64), no relaxation.
+template <class Codec, bool PROJECT, bool RELAX = true, class VGet, class Sink>
+__device__ __forceinline__ void collide(const NodeState<typename Codec::R>& st,
+                                        const StepConsts<typename Codec::KS>& K, typename Codec::R tb,
+                                        typename Codec::R omb, VGet&& vget, Sink&& sink) {
+    using R = typename Codec::R;
+    constexpr bool kF = Codec::stores_f;
+    const R eta = st.eta;
+    const R it1 = recip(R(1) + eta);           // theta_0 / theta
+    const R it = it1 * R(K.inv_theta0);        // 1 / theta
+    const R usq = fma(st.ux, st.ux, fma(st.uy, st.uy, st.uz * st.uz));
+    const R g = usq * it;
+    const R r2 = it1 * it1;
+    auto cubic = [&](const typename Codec::KS(&c)[4]) {
+        return fma(eta, fma(eta, fma(eta, R(c[3]), R(c[2])), R(c[1])), R(c[0]));
+    };
+    const R M2 = cubic(K.m2) * r2, M2p = cubic(K.m2p) * r2;
+    const R M52 = R(2.5) * M2;
+    const R A1 = M52 * recip(R(1) + M52);
+    // A2 = 5 A1 (1 - M2) - (3 + M2' - 5 M2)
+    const R A2 = fma(fma(R(-5), M2, R(5)), A1, fma(R(5), M2, R(-3) - M2p));
+    const R nga = (g * A1) * (it * R(-1.0 / 6.0));  // -g A1 / (6 theta)
+    const R hg = R(-0.5) * g;
+    const R cg = fma(-hg, A1, hg);                  // -g (1 - A1) / 2
+    const R dg = (g * A2) * R(1.0 / 6.0);
+    const R upx = st.ux * it, upy = st.uy * it, upz = st.uz * it;
+    const R x2 = upx * upx, y2 = upy * upy, z2 = upz * upz;
+    R vx = R(0), vy = R(0), vz = R(0);
+    if constexpr (PROJECT) {
+        const R Sp = fma(dg, cubic(K.pj0), nga * cubic(K.pj1));
+        const R nit = -it;
+        const R K0 = nit * fma((it * g) * R(0.5), cubic(K.pj3), Sp);
+        const R K1 = (nit * R(1.0 / 6.0)) * cubic(K.pq);
+        vx = upx * fma(K1, x2, K0);
+        vy = upy * fma(K1, y2, K0);
+        vz = upz * fma(K1, z2, K0);
+    }
+    const R tbr = tb * st.rho, tbd = tb * st.drho, one_cg = R(1) + cg, one_dg = R(1) + dg;
+    // P and B of shell s
+    auto shell = [&](int s, R& P, R& B) {
+        if constexpr (kF) {
+            P = tbr * cubic(K.rp[s]);
+            B = P * fma(nga, R(K.c2[s]), one_cg);
+        } else {
+            const R rm1 = eta * fma(eta, fma(eta, R(K.rp[s][3]), R(K.rp[s][2])), R(K.rp[s][1]));
+            const R tr = fma(tbr, rm1, tbd);  // tb (rho R_s - 1)
+            P = fma(tbr, rm1, tbr);
+            B = fma(P, fma(nga, R(K.c2[s]), cg), tr);
+        }
+    };
+    auto Dof = [&](int s) { return fma(nga, R(K.c2[s]), one_dg); };
+    {
+        R P, B;
+        shell(0, P, B);
+        if constexpr (RELAX)
+            sink(std::integral_constant<int, 0>{}, fma(omb, vget(std::integral_constant<int, 0>{}), B));
+        else
+            sink(std::integral_constant<int, 0>{}, B);
+    }
+    // pair ip, ip + 1 along a_1 (its square sq, projection cv = c_1.v): half = k^2 P / 2, odd = k P
+    auto pair = [&](auto IP, R a, R sq, R cv, R B, R half, R odd, R sixth, R Ds) {
+        const R T = fma(half, sq, B);
+        const R m = fma(a, fma(sq, sixth, Ds), cv);
+        constexpr std::integral_constant<int, decltype(IP)::value> p{};
+        constexpr std::integral_constant<int, decltype(IP)::value + 1> n{};
+        if constexpr (RELAX) {
+            sink(p, fma(odd, m, fma(omb, vget(p), T)));
+            sink(n, fma(odd, -m, fma(omb, vget(n), T)));
+        } else {
+            sink(p, fma(odd, m, T));
+            sink(n, fma(odd, -m, T));
+        }
+    };
+    {
+        R P1, B1, P2, B2;
+        shell(1, P1, B1);
+        shell(2, P2, B2);
+        const R h1 = R(0.5) * P1, o2 = R(2) * P2, D1 = Dof(1), D2 = Dof(2);
+        const R s1 = R(1.0 / 6.0), s2 = R(4.0 / 6.0);
+        pair(std::integral_constant<int, 1>{}, upx, x2, vx, B1, h1, P1, s1, D1);
+        pair(std::integral_constant<int, 3>{}, upy, y2, vy, B1, h1, P1, s1, D1);
+        pair(std::integral_constant<int, 5>{}, upz, z2, vz, B1, h1, P1, s1, D1);
+        pair(std::integral_constant<int, 7>{}, upx, x2, vx, B2, o2, o2, s2, D2);
+        pair(std::integral_constant<int, 9>{}, upy, y2, vy, B2, o2, o2, s2, D2);
+        pair(std::integral_constant<int, 11>{}, upz, z2, vz, B2, o2, o2, s2, D2);
+    }
+    const R axy = upx + upy, dxy = upx - upy, cxy = vx + vy, exy = vx - vy;
+    {
+        R P, B;
+        shell(3, P, B);
+        const R h = R(0.5) * P, Ds = Dof(3), s6 = R(1.0 / 6.0);
+        auto fcc = [&](auto IP, R a, R cv) { pair(IP, a, a * a, cv, B, h, P, s6, Ds); };
+        fcc(std::integral_constant<int, 13>{}, axy, cxy);
+        fcc(std::integral_constant<int, 15>{}, dxy, exy);
+        fcc(std::integral_constant<int, 17>{}, upx + upz, vx + vz);
+        fcc(std::integral_constant<int, 19>{}, upx - upz, vx - vz);
+        fcc(std::integral_constant<int, 21>{}, upy + upz, vy + vz);
+        fcc(std::integral_constant<int, 23>{}, upy - upz, vy - vz);
+    }
+    {
+        R P4, B4, P5, B5;
+        shell(4, P4, B4);
+        shell(5, P5, B5);
+        const R h4 = R(0.5) * P4, h5 = R(0.125) * P5, o5 = R(0.5) * P5;
+        const R D4 = Dof(4), D5 = Dof(5), s4 = R(1.0 / 6.0), s5 = R(1.0 / 24.0);
+        // the two shells' pairs along the diagonals (1,1,1) (1,1,-1) (1,-1,1) (-1,1,1)
+        auto diagonals = [&](auto&& f) {
+            f(std::integral_constant<int, 0>{}, axy + upz, cxy + vz);
+            f(std::integral_constant<int, 2>{}, axy - upz, cxy - vz);
+            f(std::integral_constant<int, 4>{}, dxy + upz, exy + vz);
+            f(std::integral_constant<int, 6>{}, upz - dxy, vz - exy);
+        };
+        auto bcc = [&](auto KD, R a, R sq, R cv) {
+            pair(std::integral_constant<int, 25 + decltype(KD)::value>{}, a, sq, cv, B4, h4, P4, s4, D4);
+        };
+        auto half = [&](auto KD, R a, R sq, R cv) {
+            pair(std::integral_constant<int, 33 + decltype(KD)::value>{}, a, sq, cv, B5, h5, o5, s5, D5);
+        };
+        if constexpr (kF) {  // bound by its operations: a, a^2 and c.v serve both shells
+            diagonals([&](auto KD, R a, R cv) {
+                const R sq = a * a;
+                bcc(KD, a, sq, cv);
+                half(KD, a, sq, cv);
+            });
+        } else {  // bound by registers: one shell's constants at a time
+            diagonals([&](auto KD, R a, R cv) { bcc(KD, a, a * a, cv); });
+            diagonals([&](auto KD, R a, R cv) { half(KD, a, a * a, cv); });
+        }
+    }
+}
+
 // Equilibrium (Eq. feqGenU3, with the optional momentum projection) and BGK
 // relaxation of one node.  v[i] are the working values of the node's incoming
 // populations (f or h, see the codec), tb = 2 beta, omb = 1 - 2 beta.
@@ -334,20 +623,7 @@ __device__ __forceinline__ void equilibrium_relax_g(const NodeState<typename Cod
     R vx = R(0), vy = R(0), vz = R(0);
     if constexpr (PROJECT) {
         R S, S4, S22;
-        if constexpr (std::is_same<R, F2>::value) {
-            // packed two-node arithmetic: the shell sums term by term (measured faster here than the
-            // cubics, which lengthen the packed path's dependency chains)
-            S = R(0);
-            S4 = R(0);
-            S22 = R(0);
-#pragma unroll
-            for (int s = 1; s < kShells; ++s) {
-                const R ft = K.w[s] * (rho + rho * rest_m1(s));
-                S = fma(ft * K.n2[s], dm1(s), S);
-                S4 = fma(ft, K.n4[s], S4);
-                S22 = fma(ft, K.n22[s], S22);
-            }
-        } else {
+        {
             auto pj = [&](int j) { return K.pj[j][0] + eta * (K.pj[j][1] + eta * (K.pj[j][2] + eta * K.pj[j][3])); };
             S = rho * (dg * pj(0) - gA1_6t * pj(1));
             S4 = rho * pj(2);
@@ -662,15 +938,46 @@ __device__ __forceinline__ void entropic_relax(const NodeState<typename Codec::R
 // Equilibrium kinds: 0 = Eq. (feqGenU3) as printed, 1 = with the momentum
 // projection, 2 = the exact entropic equilibrium (clears `ok` if Newton fails),
 // 3 = that equilibrium with the entropic path length (entropic_path).
+// The step of one node: StepK is Consts for the entropic kinds, else StepConsts.
+template <class R, int EQ>
+using StepK = std::conditional_t<(EQ >= 2), Consts<R>, StepConsts<R>>;
+
+template <class Codec, int EQ>
+__device__ __forceinline__ NodeState<typename Codec::R> step_state(const StepK<typename Codec::R, EQ>& K,
+                                                                   const typename Codec::R (&v)[kQ]) {
+    using R = typename Codec::R;
+    if constexpr (EQ >= 2) {
+        constexpr R inv_scale = R(1.0 / Codec::kScale);
+        return state_from_moments(
+            moments_from<R>([&](auto I) { return Codec::dev(v[I], K.w[vel(I).shell] * inv_scale); }), K);
+    } else {
+        return node_state<Codec>(K, [&](auto I) { return v[I]; });
+    }
+}
+
 template <class Codec, int EQ, class Sink>
-__device__ __forceinline__ void equilibrium_relax(const NodeState<typename Codec::R>& st,
-                                                  const Consts<typename Codec::KS>& K, typename Codec::R tb,
-                                                  typename Codec::R omb, const typename Codec::R (&v)[kQ], Sink&& sink,
-                                                  bool& ok) {
-    if constexpr (EQ == 2 || EQ == 3)
+__device__ __forceinline__ void step_relax(const NodeState<typename Codec::R>& st,
+                                           const StepK<typename Codec::R, EQ>& K, typename Codec::R tb,
+                                           typename Codec::R omb, const typename Codec::R (&v)[kQ], Sink&& sink,
+                                           bool& ok) {
+    if constexpr (EQ >= 2)
         entropic_relax<Codec, EQ == 3>(st, K, tb, omb, [&](auto I) { return v[I]; }, sink, ok);
     else
-        equilibrium_relax_g<Codec, EQ == 1>(st, K, tb, omb, [&](auto I) { return v[I]; }, sink);
+        collide<Codec, EQ == 1>(st, K, tb, omb, [&](auto I) { return v[I]; }, sink);
+}
+
+// Equilibrium of a node's fields (initial states, wall columns), term by term: sink receives
+// tb h^eq_i (f^eq_i for FP64).
+template <class Codec, int EQ, class Sink>
+__device__ __forceinline__ void equilibrium_of(const NodeState<typename Codec::R>& st,
+                                               const Consts<typename Codec::KS>& K, typename Codec::R tb, Sink&& sink,
+                                               bool& ok) {
+    using R = typename Codec::R;
+    auto zero = [](auto) { return R(0); };
+    if constexpr (EQ >= 2)
+        entropic_relax<Codec, EQ == 3>(st, K, tb, R(0), zero, sink, ok);
+    else
+        equilibrium_relax_g<Codec, EQ == 1>(st, K, tb, R(0), zero, sink);
 }
 
 // ---------------------------------------------------------------------------

@@ -35,7 +35,7 @@ struct LoadCG {
 template <class Codec, int EQ, class Ld = LoadNC, bool SR = false>
 __device__ __forceinline__ void step_node(const typename Codec::raw_t* __restrict__ src,
                                           typename Codec::raw_t* __restrict__ dst, const Dims& d,
-                                          const Consts<typename Codec::R>& K, typename Codec::R tb,
+                                          const StepK<typename Codec::R, EQ>& K, typename Codec::R tb,
                                           int* __restrict__ err, int s, int z, int y, int x, uint32_t sr_key = 0) {
     using R = typename Codec::R;
     using T = typename Codec::raw_t;
@@ -70,11 +70,7 @@ __device__ __forceinline__ void step_node(const typename Codec::raw_t* __restric
         }
     });
 
-    R dv[kQ];
-    constexpr R inv_scale = R(1.0 / Codec::kScale);
-    static_for<kQ>([&](auto I) { dv[I] = Codec::dev(v[I], K.w[vel(I).shell] * inv_scale); });
-    const NodeMoments<R> m = moments_from_dev(dv);
-    const NodeState<R> st = state_from_moments(m, K);
+    const NodeState<R> st = step_state<Codec, EQ>(K, v);
     bool ok = state_ok(st);
 
     const int64_t qn = (int64_t)z * nxy + (int64_t)y * d.nx + x;
@@ -82,14 +78,14 @@ __device__ __forceinline__ void step_node(const typename Codec::raw_t* __restric
     if constexpr (SR) {
         const uint32_t q = (uint32_t)((int64_t)s * d.plane + qn);
         const uint32_t s0 = pcg_hash(sr_key ^ (q >> 1));
-        equilibrium_relax<Codec, EQ>(st, K, tb * R(Codec::kScale), R(1) - tb, v,
+        step_relax<Codec, EQ>(st, K, tb * R(Codec::kScale), R(1) - tb, v,
                                      [&](auto I, R val) {
                                          const uint32_t w = sr_word<decltype(I)::value>(s0);
                                          out[(int64_t)I * d.plane] = sr_bf16(val, (q & 1u) ? (w >> 16) : (w & 0xFFFFu));
                                      },
                                      ok);
     } else {
-        equilibrium_relax<Codec, EQ>(st, K, tb * R(Codec::kScale), R(1) - tb, v,
+        step_relax<Codec, EQ>(st, K, tb * R(Codec::kScale), R(1) - tb, v,
                                      [&](auto I, R val) { out[(int64_t)I * d.plane] = Codec::to_raw(val); }, ok);
     }
     if (!ok) atomicOr(err, 1);
@@ -97,11 +93,11 @@ __device__ __forceinline__ void step_node(const typename Codec::raw_t* __restric
 
 // Direct-load step kernel.  Grid: blockIdx.x = row (s, z, y),
 // blockIdx.y * blockDim.x + threadIdx.x = x.  EQ: equilibrium kind (see
-// equilibrium_relax).
+// step_relax).
 template <class Codec, int EQ>
 __global__ void __launch_bounds__(kStepThreads) k_step(const typename Codec::raw_t* __restrict__ src,
                                                        typename Codec::raw_t* __restrict__ dst, Dims d,
-                                                       Consts<typename Codec::R> K, typename Codec::R tb,
+                                                       StepK<typename Codec::R, EQ> K, typename Codec::R tb,
                                                        int* __restrict__ err) {
     const int x = blockIdx.y * blockDim.x + threadIdx.x;
     if (x >= d.nx) return;
@@ -116,14 +112,14 @@ __global__ void __launch_bounds__(kStepThreads) k_step(const typename Codec::raw
 template <class Codec, bool PROJECT, class Ld>
 __device__ __forceinline__ void step_node2(const typename Codec::raw_t* __restrict__ src,
                                            typename Codec::raw_t* __restrict__ dst, const Dims& d,
-                                           const Consts<float>& K, float tb, int* __restrict__ err, int s, int z,
+                                           const StepConsts<float2>& K, float tb, int* __restrict__ err, int s, int z,
                                            int y, int x);
 
 // k_step with the stochastic BF16 store (series equilibrium with the momentum projection).
 template <class Codec>
 __global__ void __launch_bounds__(kStepThreads) k_step_sr(const typename Codec::raw_t* __restrict__ src,
                                                           typename Codec::raw_t* __restrict__ dst, Dims d,
-                                                          Consts<typename Codec::R> K, typename Codec::R tb,
+                                                          StepConsts<typename Codec::R> K, typename Codec::R tb,
                                                           int* __restrict__ err, uint32_t sr_key) {
     const int x = blockIdx.y * blockDim.x + threadIdx.x;
     if (x >= d.nx) return;
@@ -145,7 +141,7 @@ __global__ void __launch_bounds__(kStepThreads) k_step_sr(const typename Codec::
 template <class Codec, bool PROJECT, int MINB>
 __global__ void __launch_bounds__(kStepThreads, MINB) k_step2(const typename Codec::raw_t* __restrict__ src,
                                                         typename Codec::raw_t* __restrict__ dst, Dims d,
-                                                        Consts<float> K, float tb, int* __restrict__ err,
+                                                        StepConsts<float2> K, float tb, int* __restrict__ err,
                                                         int chunks) {
     const int64_t t = blockIdx.x;
     const int64_t rp = t / chunks;
@@ -163,7 +159,7 @@ __global__ void __launch_bounds__(kStepThreads, MINB) k_step2(const typename Cod
 template <class Codec, bool PROJECT, class Ld>
 __device__ __forceinline__ void step_node2(const typename Codec::raw_t* __restrict__ src,
                                            typename Codec::raw_t* __restrict__ dst, const Dims& d,
-                                           const Consts<float>& K, float tb, int* __restrict__ err, int s, int z,
+                                           const StepConsts<float2>& K, float tb, int* __restrict__ err, int s, int z,
                                            int y, int x) {
     using T = typename Codec::raw_t;
     using C2 = Codec2<Codec>;
@@ -212,13 +208,11 @@ __device__ __forceinline__ void step_node2(const typename Codec::raw_t* __restri
     });
     auto vget = [&](auto I) { return F2(Codec::unpack2(pv[I])); };
 
-    constexpr float inv_scale = (float)(1.0 / Codec::kScale);
-    const NodeMoments<F2> m = moments_from<F2>([&](auto I) { return C2::dev(vget(I), F2(K.w[vel(I).shell] * inv_scale)); });
-    const NodeState<F2> st = state_from_moments(m, K);
+    const NodeState<F2> st = node_state<C2>(K, vget);
     if (!state_ok(st)) atomicOr(err, 1);
 
     T* outa = dst + (size_t)s * kQ * d.plane + ((uint32_t)z * nxy + (uint32_t)y * nx + (uint32_t)x);
-    equilibrium_relax_g<C2, PROJECT>(st, K, F2(tb * (float)Codec::kScale), F2(1.f - tb), vget,
+    collide<C2, PROJECT>(st, K, F2(tb * (float)Codec::kScale), F2(1.f - tb), vget,
                                      [&](auto I, F2 val) {
                                          T* p = outa + (size_t)I * plane;
                                          p[0] = Codec::to_raw(val.v.x);
@@ -330,7 +324,7 @@ __device__ __forceinline__ void prefetch_row_l2(const typename Codec::raw_t* src
 template <class Codec, bool PROJECT, int MINB, int MODE, bool SR = false>
 __global__ void __launch_bounds__(kStepThreads, MINB) k_step2x(const typename Codec::raw_t* __restrict__ src,
                                                          typename Codec::raw_t* __restrict__ dst, Dims d,
-                                                         Consts<float> K, float tb, int* __restrict__ err,
+                                                         StepConsts<float2> K, float tb, int* __restrict__ err,
                                                          int chunks, int rpb, uint32_t sr_key) {
     using T = typename Codec::raw_t;
     using P = typename Codec::pair_t;
@@ -356,7 +350,6 @@ __global__ void __launch_bounds__(kStepThreads, MINB) k_step2x(const typename Co
 
     P pv[kQ];
     auto vget = [&](auto I) { return F2(Codec::unpack2(pv[I])); };
-    constexpr float inv_scale = (float)(1.0 / Codec::kScale);
 
     for (uint32_t r = r0; r < r1; ++r) {
         // the next row, in (s, z, y) order
@@ -384,22 +377,28 @@ __global__ void __launch_bounds__(kStepThreads, MINB) k_step2x(const typename Co
             static_for<kQ>([&](auto I) { pv[I] = load_pair2x<Codec, I>(a, plane, xm, x0, xq); });
         }
 
-        const NodeMoments<F2> m =
-            moments_from<F2>([&](auto I) { return C2::dev(vget(I), F2(K.w[vel(I).shell] * inv_scale)); });
-        const NodeState<F2> st = state_from_moments(m, K);
+        const NodeState<F2> st = node_state<C2>(K, vget);
         if (!state_ok(st)) atomicOr(err, 1);
+        // The values stay packed from here to their relaxation: without the barrier the compiler keeps
+        // the 82 widened numbers of the sums alive and spills at 128 registers.
+        static_for<kQ>([&](auto I) {
+            uint32_t w;
+            memcpy(&w, &pv[I], sizeof w);
+            asm volatile("" : "+r"(w));
+            memcpy(&pv[I], &w, sizeof w);
+        });
 
         P* outp = reinterpret_cast<P*>(dst + (size_t)s * kQ * d.plane + ((uint32_t)z * nxy + (uint32_t)y * nx + x0));
         if constexpr (SR) {
             const uint32_t q = (uint32_t)s * plane + (uint32_t)z * nxy + (uint32_t)y * nx + x0;
             const uint32_t s0 = pcg_hash(sr_key ^ (q >> 1));
-            equilibrium_relax_g<C2, PROJECT>(st, K, F2(tb * (float)Codec::kScale), F2(1.f - tb), vget,
+            collide<C2, PROJECT>(st, K, F2(tb * (float)Codec::kScale), F2(1.f - tb), vget,
                                              [&](auto I, F2 val) {
                                                  outp[(size_t)I * (plane / 2)] =
                                                      sr_bf16x2(val.v, sr_word<decltype(I)::value>(s0));
                                              });
         } else {
-            equilibrium_relax_g<C2, PROJECT>(st, K, F2(tb * (float)Codec::kScale), F2(1.f - tb), vget,
+            collide<C2, PROJECT>(st, K, F2(tb * (float)Codec::kScale), F2(1.f - tb), vget,
                                              [&](auto I, F2 val) { outp[(size_t)I * (plane / 2)] = Codec::to_raw2(val.v); });
         }
         s = sn;
@@ -431,12 +430,9 @@ __global__ void __launch_bounds__(256) k_init(typename Codec::raw_t* __restrict_
     st.uz = (R)u[2 * ustride + k];
     st.eta = (R)((theta[k] - theta0) * inv_theta0);
     bool ok = state_ok(st);
-    R zero[kQ];
-#pragma unroll
-    for (int i = 0; i < kQ; ++i) zero[i] = R(0);
     typename Codec::raw_t* out = dst + (int64_t)s * kQ * d.plane + node;
-    equilibrium_relax<Codec, EQ>(st, K, R(Codec::kScale), R(0), zero,
-                                 [&](auto I, R val) { out[(int64_t)I * d.plane] = Codec::to_raw(val); }, ok);
+    equilibrium_of<Codec, EQ>(st, K, R(Codec::kScale),
+                              [&](auto I, R val) { out[(int64_t)I * d.plane] = Codec::to_raw(val); }, ok);
     if (!ok) atomicOr(err, 1);
 }
 

@@ -16,9 +16,34 @@ struct W41 {
 struct LaunchConsts {
     Consts<float> kf;
     Consts<double> kd;
+    StepConsts<double> sd;
+    StepConsts<float> sf[2];   // [1]: FP16 storage (its scale folded in), [0]: scale 1
+    StepConsts<float2> sp[2];  // the same, each constant twice
     W41 w41;
     double theta0;
 };
+
+template <class Codec>
+inline const Consts<typename Codec::R>& consts_of(const LaunchConsts& c) {
+    if constexpr (sizeof(typename Codec::R) == 8)
+        return c.kd;
+    else
+        return c.kf;
+}
+// Constants of the series step (EQ < 2) or of the entropic one.
+template <class Codec, int EQ>
+inline const StepK<typename Codec::R, EQ>& step_consts(const LaunchConsts& c) {
+    if constexpr (EQ >= 2)
+        return consts_of<Codec>(c);
+    else if constexpr (sizeof(typename Codec::R) == 8)
+        return c.sd;
+    else
+        return c.sf[Codec::kScale != 1.0];
+}
+template <class Codec>
+inline const StepConsts<float2>& pair_consts(const LaunchConsts& c) {
+    return c.sp[Codec::kScale != 1.0];
+}
 
 // Storage precision codes (match lb_precision in gblb.h).
 enum Prec { kF64 = 0, kF32 = 1, kF16 = 2, kBF16 = 3 };

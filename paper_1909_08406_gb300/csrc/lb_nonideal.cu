@@ -499,7 +499,7 @@ __global__ void __launch_bounds__(kNiThreads, 6) k_ni_force2x(Dims d, int chunks
 template <class Codec>
 __global__ void __launch_bounds__(kNiThreads) k_ni_step(const typename Codec::raw_t* __restrict__ src,
                                                         typename Codec::raw_t* __restrict__ dst, Dims d, int chunks,
-                                                        Consts<typename Codec::R> K, typename Codec::R tb,
+                                                        StepConsts<typename Codec::R> K, typename Codec::R tb,
                                                         typename Codec::R inv_theta0,
                                                         const typename Codec::R* __restrict__ G,
                                                         int* __restrict__ err) {
@@ -512,10 +512,7 @@ __global__ void __launch_bounds__(kNiThreads) k_ni_step(const typename Codec::ra
     const R gf[3] = {G[q], G[n + q], G[2 * n + q]};
     R v[kQ];
     ni_gather<Codec>(src, d, s, z, y, x, v);
-    R dv[kQ];
-    constexpr R inv_scale = R(1.0 / Codec::kScale);
-    static_for<kQ>([&](auto I) { dv[I] = Codec::dev(v[I], K.w[vel(I).shell] * inv_scale); });
-    const NodeMoments<R> m = moments_from_dev(dv);
+    const NodeSums<R> m = node_sums<Codec>(K, [&](auto I) { return v[I]; });
     NodeState<R> st;
     st.drho = m.drho;
     st.rho = R(1) + m.drho;
@@ -525,12 +522,11 @@ __global__ void __launch_bounds__(kNiThreads) k_ni_step(const typename Codec::ra
     st.uy = m.jy * inv_rho + R(0.5) * gy;
     st.uz = m.jz * inv_rho + R(0.5) * gz;
     st.eta = R(0);  // isothermal: the equilibrium at theta_0
-    bool ok = state_ok(st);
+    const bool ok = state_ok(st);
     // f^eq in the working representation: f (FP64 codec) or scale * h^eq (deviation codecs)
-    R veq[kQ], zero[kQ];
-#pragma unroll
-    for (int i = 0; i < kQ; ++i) zero[i] = R(0);
-    equilibrium_relax<Codec, 1>(st, K, R(Codec::kScale), R(0), zero, [&](auto I, R val) { veq[I] = val; }, ok);
+    R veq[kQ];
+    collide<Codec, true, false>(st, K, R(Codec::kScale), R(0), [](auto) { return R(0); },
+                                [&](auto I, R val) { veq[I] = val; });
     T* out = dst + (int64_t)s * kQ * d.plane + ((int64_t)z * d.ny + y) * d.nx + x;
     const R half_f = R(1) - R(0.5) * tb;  // 1 - beta
     static_for<kQ>([&](auto I) {
@@ -647,7 +643,7 @@ __global__ void __launch_bounds__(kStepThreads) k_ni_density2x(const typename Co
 template <class Codec>
 __global__ void __launch_bounds__(kStepThreads, 3) k_ni_step2x(const typename Codec::raw_t* __restrict__ src,
                                                                typename Codec::raw_t* __restrict__ dst, Dims d,
-                                                               int chunks, int rpb, Consts<float> K, float tb,
+                                                               int chunks, int rpb, StepConsts<float2> K, float tb,
                                                                float inv_theta0, const float* __restrict__ G,
                                                                int* __restrict__ err) {
     using P = typename Codec::pair_t;
@@ -666,9 +662,7 @@ __global__ void __launch_bounds__(kStepThreads, 3) k_ni_step2x(const typename Co
     auto vget = [&](auto I) { return F2(Codec::unpack2(pv[I])); };
     const F2 gx(*reinterpret_cast<const float2*>(G + q)), gy(*reinterpret_cast<const float2*>(G + n + q)),
         gz(*reinterpret_cast<const float2*>(G + 2 * n + q));
-    constexpr float inv_scale = (float)(1.0 / Codec::kScale);
-    const NodeMoments<F2> m =
-        moments_from<F2>([&](auto I) { return C2::dev(vget(I), F2(K.w[vel(I).shell] * inv_scale)); });
+    const NodeSums<F2> m = node_sums<C2>(K, vget);
     NodeState<F2> st;
     st.drho = m.drho;
     st.rho = F2(1.f) + m.drho;
@@ -685,7 +679,7 @@ __global__ void __launch_bounds__(kStepThreads, 3) k_ni_step2x(const typename Co
     const F2 tbv(tb), half_f(1.f - 0.5f * tb), scale((float)Codec::kScale);
     P* outp = reinterpret_cast<P*>(dst + (size_t)s * kQ * d.plane + (q - (uint32_t)s * (uint32_t)d.plane));
     const size_t pstride = (size_t)d.plane / 2;
-    equilibrium_relax_g<C2, true>(st, K, scale, F2(0.f), vget, [&](auto I, F2 veq) {
+    collide<C2, true, false>(st, K, scale, F2(0.f), vget, [&](auto I, F2 veq) {
         constexpr Vel c = vel(I);
         F2 gc = F2(0.f) - hu;
         if constexpr (c.x != 0) gc = fma(F2(0.5f * c.x), hx, gc);
@@ -726,11 +720,7 @@ cudaError_t launch_nonideal_step(int prec, const void* src, void* dst, const Dim
     return ni_codec(prec, [&](auto codec) {
         using C = decltype(codec);
         using R = typename C::R;
-        const Consts<R>* K;
-        if constexpr (sizeof(R) == 8)
-            K = &c.kd;
-        else
-            K = &c.kf;
+        const Consts<R>* K = &consts_of<C>(c);
         const NiEosT<R> e = ni_eos_in<R>(e64);
         // field arrays in the compute type: RF, A, B, C (2 values per node each; 16-byte aligned, n
         // is even), then MU, D (1) and G (3)
@@ -773,11 +763,11 @@ cudaError_t launch_nonideal_step(int prec, const void* src, void* dst, const Dim
         }
         if constexpr (kPairs) {
             if (pairs)
-                k_ni_step2x<C><<<blocks2, th2, 0, st>>>(in, out, d, chunks2, kRpb, *K, (float)twobeta,
+                k_ni_step2x<C><<<blocks2, th2, 0, st>>>(in, out, d, chunks2, kRpb, pair_consts<C>(c), (float)twobeta,
                                                          (float)(1.0 / c.theta0), fl.G, err);
         }
         if (!pairs)
-            k_ni_step<C><<<blocks, kNiThreads, 0, st>>>(in, out, d, chunks, *K, (R)twobeta, (R)(1.0 / c.theta0), fl.G,
+            k_ni_step<C><<<blocks, kNiThreads, 0, st>>>(in, out, d, chunks, (step_consts<C, 1>(c)), (R)twobeta, (R)(1.0 / c.theta0), fl.G,
                                                          err);
         return cudaGetLastError();
     });

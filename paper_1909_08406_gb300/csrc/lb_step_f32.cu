@@ -1,7 +1,7 @@
 // FP32-arithmetic step kernels (FP32, FP16 and BF16 storage).  Variants:
 //   kKernelDirect1   k_step:        one node per thread, direct global loads
-//   kKernelDirect2   k_step2<.,.,3>: two rows per thread, packed FP32x2 math
-//   kKernelDirect2R  k_step2<.,.,4>: the same, register budget for 4 CTAs/SM
+//   kKernelDirect2   k_step2<.,.,4>: two rows per thread, packed FP32x2 math, 4 CTAs/SM
+//   kKernelDirect2R  k_step2<.,.,3>: the same, register budget for 3 CTAs/SM
 //   kKernelStaged    k_step_tma:    rows fetched by TMA bulk copies into a
 //                                   shared-memory ring
 //   kKernelWarpSpec  k_step_ws:     the same staging with a dedicated producer
@@ -20,7 +20,7 @@ static cudaError_t run_direct1(const void* src, void* dst, const Dims& d, const 
                                int* err, cudaStream_t st) {
     using T = typename Codec::raw_t;
     const int th = step_threads(d);
-    k_step<Codec, P><<<step_grid(d, th), th, 0, st>>>(static_cast<const T*>(src), static_cast<T*>(dst), d, c.kf,
+    k_step<Codec, P><<<step_grid(d, th), th, 0, st>>>(static_cast<const T*>(src), static_cast<T*>(dst), d, (step_consts<Codec, 0>(c)),
                                                       (float)twobeta, err);
     return cudaGetLastError();
 }
@@ -33,7 +33,7 @@ static cudaError_t run_direct2(const void* src, void* dst, const Dims& d, const 
     const int chunks = (d.nx + th - 1) / th;
     const int64_t blocks = d.rows / 2 * chunks;
     k_step2<Codec, P, MINB><<<(unsigned)blocks, th, 0, st>>>(static_cast<const T*>(src), static_cast<T*>(dst), d,
-                                                             c.kf, (float)twobeta, err, chunks);
+                                                             pair_consts<Codec>(c), (float)twobeta, err, chunks);
     return cudaGetLastError();
 }
 
@@ -49,7 +49,7 @@ static cudaError_t run_direct2x(const void* src, void* dst, const Dims& d, const
         const int chunks = (half + th - 1) / th;
         const int64_t blocks = ((d.rows + rpb - 1) / rpb) * chunks;
         auto kern = k_step2x<Codec, P, MINB, MODE, SR>;
-        kern<<<(unsigned)blocks, th, 0, st>>>(static_cast<const T*>(src), static_cast<T*>(dst), d, c.kf,
+        kern<<<(unsigned)blocks, th, 0, st>>>(static_cast<const T*>(src), static_cast<T*>(dst), d, pair_consts<Codec>(c),
                                                  (float)twobeta, err, chunks, rpb, sr_key);
         return cudaGetLastError();
     }
@@ -85,7 +85,7 @@ static cudaError_t run_tma(const void* src, void* dst, const Dims& d, const Laun
     const int64_t ntiles = d.rows * (d.nx / Cfg::TX);
     const int grid = (int)(ntiles < info.grid ? ntiles : info.grid);
     const long long wait_limit = 4000000000LL;  // ~2 s of SM clock
-    kern<<<grid, Cfg::THREADS, Cfg::SMEM, st>>>(static_cast<const T*>(src), static_cast<T*>(dst), d, c.kf,
+    kern<<<grid, Cfg::THREADS, Cfg::SMEM, st>>>(static_cast<const T*>(src), static_cast<T*>(dst), d, (step_consts<Codec, 0>(c)),
                                                  (float)twobeta, err, wait_limit);
     return cudaGetLastError();
 }
@@ -114,7 +114,7 @@ static cudaError_t run_ws(const void* src, void* dst, const Dims& d, const Launc
     const int64_t ntiles = d.rows / 2 * (d.nx / Cfg::TX);
     const int grid = (int)(ntiles < info.grid ? ntiles : info.grid);
     const long long wait_limit = 4000000000LL;  // ~2 s of SM clock
-    kern<<<grid, Cfg::THREADS, Cfg::SMEM, st>>>(static_cast<const T*>(src), static_cast<T*>(dst), d, c.kf,
+    kern<<<grid, Cfg::THREADS, Cfg::SMEM, st>>>(static_cast<const T*>(src), static_cast<T*>(dst), d, pair_consts<Codec>(c),
                                                  (float)twobeta, err, wait_limit);
     return cudaGetLastError();
 }
@@ -185,11 +185,11 @@ static cudaError_t step_codec(int prec, int kernel, const void* src, void* dst, 
                 return run_tma<Codec, P, typename TmaShape<Codec, 256>::Cfg>(src, dst, d, c, twobeta, err, st);
             return run_tma<Codec, P, typename TmaShape<Codec, 128>::Cfg>(src, dst, d, c, twobeta, err, st);
         case kKernelWarpSpec: return run_ws<Codec, P, typename WsShape<Codec>::Cfg>(src, dst, d, c, twobeta, err, st);
-        case kKernelDirect2X: return run_direct2x<Codec, P, 3, 0>(src, dst, d, c, twobeta, err, st, 1);
-        case kKernelDirect2XL: return run_direct2x<Codec, P, 3, 2>(src, dst, d, c, twobeta, err, st, 2);
+        case kKernelDirect2X: return run_direct2x<Codec, P, 4, 0>(src, dst, d, c, twobeta, err, st, 1);
+        case kKernelDirect2XL: return run_direct2x<Codec, P, 4, 2>(src, dst, d, c, twobeta, err, st, 2);
 
-        case kKernelDirect2: return run_direct2<Codec, P, 3>(src, dst, d, c, twobeta, err, st);
-        case kKernelDirect2R: return run_direct2<Codec, P, 4>(src, dst, d, c, twobeta, err, st);
+        case kKernelDirect2: return run_direct2<Codec, P, 4>(src, dst, d, c, twobeta, err, st);
+        case kKernelDirect2R: return run_direct2<Codec, P, 3>(src, dst, d, c, twobeta, err, st);
         default: return run_direct1<Codec, P>(src, dst, d, c, twobeta, err, st);
     }
 }
@@ -216,10 +216,10 @@ cudaError_t launch_step_sr(const void* src, void* dst, const Dims& d, const Laun
                            cudaStream_t st, uint32_t sr_key) {
     using T = CodecBF16::raw_t;
     if (resolve_kernel(kBF16, d, kKernelDirect2XL) == kKernelDirect2XL)
-        return run_direct2x<CodecBF16, true, 3, 2, true>(src, dst, d, c, twobeta, err, st, 2, sr_key);
+        return run_direct2x<CodecBF16, true, 4, 2, true>(src, dst, d, c, twobeta, err, st, 2, sr_key);
     const int th = step_threads(d);
-    k_step_sr<CodecBF16><<<step_grid(d, th), th, 0, st>>>(static_cast<const T*>(src), static_cast<T*>(dst), d, c.kf,
-                                                         (float)twobeta, err, sr_key);
+    k_step_sr<CodecBF16><<<step_grid(d, th), th, 0, st>>>(static_cast<const T*>(src), static_cast<T*>(dst), d,
+                                                         c.sf[0], (float)twobeta, err, sr_key);
     return cudaGetLastError();
 }
 

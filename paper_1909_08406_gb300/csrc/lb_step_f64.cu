@@ -13,9 +13,9 @@ cudaError_t launch_step_f64(int eq, const void* src, void* dst, const Dims& d, c
     else if (eq == 2)
         k_step<CodecF64, 2><<<step_grid(d, th), th, 0, st>>>(s, o, d, c.kd, twobeta, err);
     else if (eq == 1)
-        k_step<CodecF64, 1><<<step_grid(d, th), th, 0, st>>>(s, o, d, c.kd, twobeta, err);
+        k_step<CodecF64, 1><<<step_grid(d, th), th, 0, st>>>(s, o, d, c.sd, twobeta, err);
     else
-        k_step<CodecF64, 0><<<step_grid(d, th), th, 0, st>>>(s, o, d, c.kd, twobeta, err);
+        k_step<CodecF64, 0><<<step_grid(d, th), th, 0, st>>>(s, o, d, c.sd, twobeta, err);
     return cudaGetLastError();
 }
 

@@ -99,7 +99,7 @@ __device__ __forceinline__ TileCoord tile_coord(int64_t t, int tiles_per_row, in
 template <class Codec, bool PROJECT, class Cfg>
 __global__ void __launch_bounds__(Cfg::THREADS, Cfg::MINB) k_step_tma(const typename Codec::raw_t* __restrict__ src,
                                                            typename Codec::raw_t* __restrict__ dst, Dims d,
-                                                           Consts<typename Codec::R> K, typename Codec::R tb,
+                                                           StepConsts<typename Codec::R> K, typename Codec::R tb,
                                                            int* __restrict__ err, long long wait_limit) {
     using R = typename Codec::R;
     using T = typename Codec::raw_t;
@@ -198,11 +198,10 @@ __global__ void __launch_bounds__(Cfg::THREADS, Cfg::MINB) k_step_tma(const type
                     return Codec::value(sb[I * ROW + xl + H - c.x / 2]);
                 }
             };
-            const NodeMoments<R> m = moments_from<R>([&](auto I) { return Codec::dev(vget(I), K.w[vel(I).shell] * inv_scale); });
-            const NodeState<R> ns = state_from_moments(m, K);
+            const NodeState<R> ns = node_state<Codec>(K, vget);
             if (!state_ok(ns)) atomicOr(err, 1);
             T* out = outrow + xl;
-            equilibrium_relax_g<Codec, PROJECT>(ns, K, tbs, omb, vget,
+            collide<Codec, PROJECT>(ns, K, tbs, omb, vget,
                                                 [&](auto I, R val) { out[(int64_t)I * d.plane] = Codec::to_raw(val); });
         }
     }

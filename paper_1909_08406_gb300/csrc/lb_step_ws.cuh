@@ -68,7 +68,7 @@ struct WsCfg {
 template <class Codec, bool PROJECT, class Cfg>
 __global__ void __launch_bounds__(Cfg::THREADS, Cfg::MINB) k_step_ws(const typename Codec::raw_t* __restrict__ src,
                                                                     typename Codec::raw_t* __restrict__ dst, Dims d,
-                                                                    Consts<float> K, float tb, int* __restrict__ err,
+                                                                    StepConsts<float2> K, float tb, int* __restrict__ err,
                                                                     long long wait_limit) {
     using T = typename Codec::raw_t;
     using C2 = Codec2<Codec>;
@@ -200,12 +200,10 @@ __global__ void __launch_bounds__(Cfg::THREADS, Cfg::MINB) k_step_ws(const typen
                 const uint32_t a = sbu + (uint32_t)(((2 * I) * ROW + off) * (int)sizeof(T));
                 return F2(Codec::value(lds_keep<T>(a)), Codec::value(lds_keep<T>(a + ROW * (int)sizeof(T))));
             };
-            const NodeMoments<F2> m =
-                moments_from<F2>([&](auto I) { return C2::dev(vget(I), F2(K.w[vel(I).shell] * inv_scale)); });
-            const NodeState<F2> ns = state_from_moments(m, K);
+            const NodeState<F2> ns = node_state<C2>(K, vget);
             if (!state_ok(ns)) atomicOr(err, 1);
             T* outa = dst + (size_t)s * kQ * d.plane + ((uint32_t)z * nxy + (uint32_t)y * nx + (uint32_t)(x0 + xl));
-            equilibrium_relax_g<C2, PROJECT>(ns, K, tbs, omb, vget, [&](auto I, F2 val) {
+            collide<C2, PROJECT>(ns, K, tbs, omb, vget, [&](auto I, F2 val) {
                 T* p = outa + (size_t)I * plane;
                 p[0] = Codec::to_raw(val.v.x);
                 p[nx] = Codec::to_raw(val.v.y);

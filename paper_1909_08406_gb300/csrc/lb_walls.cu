@@ -103,11 +103,9 @@ __global__ void k_wall_setup(WallPtrs w, Dims d, Consts<double> K, double theta0
     st.uy = pr[ncol + col];
     st.uz = 0.0;
     st.eta = pr[2 * ncol + col] / theta0 - 1.0;
-    double zero[kQ], e[kQ];
-#pragma unroll
-    for (int i = 0; i < kQ; ++i) zero[i] = 0.0;
+    double e[kQ];
     bool ok = state_ok(st);
-    equilibrium_relax<CodecF64, EQ>(st, K, 1.0, 0.0, zero, [&](auto I, double val) { e[I] = val; }, ok);
+    equilibrium_of<CodecF64, EQ>(st, K, 1.0, [&](auto I, double val) { e[I] = val; }, ok);
     double emit = 0.0;
     R* ec = static_cast<R*>(w.e) + (int64_t)side * kQ * ncol + col;
 #pragma unroll
@@ -177,7 +175,7 @@ __global__ void __launch_bounds__(128) k_wall_columns(const typename Codec::raw_
 template <class Codec, int EQ>
 __global__ void __launch_bounds__(kStepThreads) k_step_walls(const typename Codec::raw_t* __restrict__ src,
                                                              typename Codec::raw_t* __restrict__ dst, Dims d,
-                                                             Consts<typename Codec::R> K, typename Codec::R tb,
+                                                             StepK<typename Codec::R, EQ> K, typename Codec::R tb,
                                                              WallPtrs w, int* __restrict__ err) {
     using R = typename Codec::R;
     using T = typename Codec::raw_t;
@@ -233,14 +231,11 @@ __global__ void __launch_bounds__(kStepThreads) k_step_walls(const typename Code
         }
     });
 
-    R dv[kQ];
-    constexpr R inv_scale = R(1.0 / Codec::kScale);
-    static_for<kQ>([&](auto I) { dv[I] = Codec::dev(v[I], K.w[vel(I).shell] * inv_scale); });
-    const NodeState<R> st = state_from_moments(moments_from_dev(dv), K);
+    const NodeState<R> st = step_state<Codec, EQ>(K, v);
     bool ok = state_ok(st);
     T* out = dst + (int64_t)s * kQ * d.plane + (int64_t)z * nxy + (int64_t)y * d.nx + x;
-    equilibrium_relax<Codec, EQ>(st, K, tb * R(Codec::kScale), R(1) - tb, v,
-                                 [&](auto I, R val) { out[(int64_t)I * d.plane] = Codec::to_raw(val); }, ok);
+    step_relax<Codec, EQ>(st, K, tb * R(Codec::kScale), R(1) - tb, v,
+                          [&](auto I, R val) { out[(int64_t)I * d.plane] = Codec::to_raw(val); }, ok);
     if (!ok) atomicOr(err, 1);
 }
 
@@ -265,14 +260,6 @@ static cudaError_t with_eq(int eq, F&& f) {
     }
 }
 
-template <class C>
-static const Consts<typename C::R>& consts_for(const LaunchConsts& c) {
-    if constexpr (sizeof(typename C::R) == 8)
-        return c.kd;
-    else
-        return c.kf;
-}
-
 cudaError_t launch_wall_setup(int prec, int eq, void* blk, const Dims& d, const LaunchConsts& c, cudaStream_t st) {
     const int64_t ncol = (int64_t)d.nx * d.ny;
     return with_codec(prec, [&](auto codec) {
@@ -295,7 +282,7 @@ cudaError_t launch_wall_step(int prec, int eq, int variant, const void* src, voi
         using C = decltype(codec);
         const WallPtrs w = wall_ptrs(blk, ncol, sizeof(typename C::R));
         k_wall_columns<C><<<(unsigned)((2 * ncol + 127) / 128), 128, 0, st>>>(
-            static_cast<const typename C::raw_t*>(src), d, consts_for<C>(c), w);
+            static_cast<const typename C::raw_t*>(src), d, consts_of<C>(c), w);
         return cudaGetLastError();
     });
     if (e != cudaSuccess) return e;
@@ -310,7 +297,7 @@ cudaError_t launch_wall_step(int prec, int eq, int variant, const void* src, voi
         return with_eq(eq, [&](auto E) {
             k_step_walls<C, decltype(E)::value><<<grid, th, 0, st>>>(
                 static_cast<const typename C::raw_t*>(src), static_cast<typename C::raw_t*>(dst), d,
-                consts_for<C>(c), (R)twobeta, w, err);
+                (step_consts<C, decltype(E)::value>(c)), (R)twobeta, w, err);
             return cudaGetLastError();
         });
     });
