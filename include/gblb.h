@@ -237,10 +237,11 @@ lb_status lb_set_state(lb_ctx *ctx, const void *raw, int on_device);
  *                      per thread (not FP64; nx a multiple of 128, ny even)
  *   LB_KERNEL_DIRECT2X two x-adjacent nodes per thread, FP32x2 arithmetic,
  *                      32-bit paired loads and stores (FP16/BF16 storage; nx even)
- *   LB_KERNEL_DIRECT2XL the same over 2 rows per block, the next row's source
- *                      rows prefetched into L2 by bulk prefetches
+ *   LB_KERNEL_DIRECT2XL the same kernel (it once prefetched rows into L2)
  *   LB_KERNEL_AUTO     DIRECT2XL for 16-bit storage with nx even, else DIRECT2 where
  *                      it applies, else DIRECT1 (the default)
+ * The direct kernels give the same bits; a grid too small to fill the SMs with two
+ * nodes per thread runs one node per thread under any of their names.
  * A request that does not apply to the grid falls back to one that does. */
 #define LB_KERNEL_AUTO (-1)
 #define LB_KERNEL_DIRECT1 0

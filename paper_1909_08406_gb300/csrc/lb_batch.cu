@@ -31,29 +31,6 @@
 
 namespace gblb {
 
-// Division of n < 2^31 by a run-time constant d >= 1 as one multiply and shift
-// (Granlund and Montgomery, division by invariant integers using
-// multiplication, 1994): with 2^k >= d and m = ceil(2^(31+k) / d),
-// floor(n / d) = (n m) >> (31 + k).  Proof: write n = q d + r and
-// m d = 2^(31+k) + e with 0 <= e < d <= 2^k; then
-// n m / 2^(31+k) = q + (r + n e / 2^(31+k)) / d, and n e / 2^(31+k) < 1,
-// so the bracket stays below d.  m < 2^32 because d > 2^(k-1) for the
-// smallest such k.
-struct FastDiv {
-    uint32_t m, sh;
-};
-
-static FastDiv make_fastdiv(uint32_t d) {
-    uint32_t k = 0;
-    while ((1ull << k) < d) ++k;
-    FastDiv f;
-    f.m = (uint32_t)(((1ull << (31 + k)) + d - 1) / d);
-    f.sh = 31 + k;
-    return f;
-}
-
-__device__ __forceinline__ uint32_t fdiv(uint32_t n, FastDiv f) { return (uint32_t)(((uint64_t)n * f.m) >> f.sh); }
-
 struct BatchSim {
     void* buf[2];
     Dims d;
@@ -153,7 +130,7 @@ __device__ __forceinline__ void batch_tile2(const BatchSim* __restrict__ sims, i
 // FP64 arithmetic need about 168 (3 CTAs).
 template <class Codec, bool TWO>
 constexpr int batch_min_blocks(bool persistent) {
-    return (TWO || sizeof(typename Codec::R) == 8) ? 3 : (persistent ? 6 : 6);
+    return sizeof(typename Codec::R) == 8 ? 3 : TWO ? 4 : 6;
 }
 
 // Constants of the one-node and of the packed two-node update.

@@ -220,6 +220,11 @@ __device__ __forceinline__ double recip(double x) { return 1.0 / x; }
 __device__ __forceinline__ float recip(float x) { return __fdividef(1.0f, x); }
 __device__ __forceinline__ F2 recip(F2 x) { return F2(__fdividef(1.0f, x.v.x), __fdividef(1.0f, x.v.y)); }
 
+// A product rounded by itself (not contracted into a following addition).
+__device__ __forceinline__ double mul(double a, double b) { return a * b; }
+__device__ __forceinline__ float mul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ F2 mul(F2 a, F2 b) { return a * b; }
+
 // Two-node codec over a one-node storage codec: same storage, F2 arithmetic.
 template <class Base>
 struct Codec2 {
@@ -469,28 +474,28 @@ __device__ __forceinline__ void collide(const NodeState<typename Codec::R>& st,
     auto cubic = [&](const typename Codec::KS(&c)[4]) {
         return fma(eta, fma(eta, fma(eta, R(c[3]), R(c[2])), R(c[1])), R(c[0]));
     };
-    const R M2 = cubic(K.m2) * r2, M2p = cubic(K.m2p) * r2;
-    const R M52 = R(2.5) * M2;
-    const R A1 = M52 * recip(R(1) + M52);
+    const R M2 = mul(cubic(K.m2), r2);
+    const R A1 = (R(2.5) * M2) * recip(fma(R(2.5), M2, R(1)));
     // A2 = 5 A1 (1 - M2) - (3 + M2' - 5 M2)
-    const R A2 = fma(fma(R(-5), M2, R(5)), A1, fma(R(5), M2, R(-3) - M2p));
+    const R A2 = fma(fma(R(-5), M2, R(5)), A1, fma(R(5), M2, fma(-cubic(K.m2p), r2, R(-3))));
     const R nga = (g * A1) * (it * R(-1.0 / 6.0));  // -g A1 / (6 theta)
     const R hg = R(-0.5) * g;
     const R cg = fma(-hg, A1, hg);                  // -g (1 - A1) / 2
-    const R dg = (g * A2) * R(1.0 / 6.0);
-    const R upx = st.ux * it, upy = st.uy * it, upz = st.uz * it;
+    const R gA2 = g * A2;
+    const R upx = mul(st.ux, it), upy = mul(st.uy, it), upz = mul(st.uz, it);
     const R x2 = upx * upx, y2 = upy * upy, z2 = upz * upz;
     R vx = R(0), vy = R(0), vz = R(0);
     if constexpr (PROJECT) {
-        const R Sp = fma(dg, cubic(K.pj0), nga * cubic(K.pj1));
+        const R Sp = fma(gA2 * R(1.0 / 6.0), cubic(K.pj0), nga * cubic(K.pj1));
         const R nit = -it;
         const R K0 = nit * fma((it * g) * R(0.5), cubic(K.pj3), Sp);
         const R K1 = (nit * R(1.0 / 6.0)) * cubic(K.pq);
-        vx = upx * fma(K1, x2, K0);
-        vy = upy * fma(K1, y2, K0);
-        vz = upz * fma(K1, z2, K0);
+        vx = mul(upx, fma(K1, x2, K0));
+        vy = mul(upy, fma(K1, y2, K0));
+        vz = mul(upz, fma(K1, z2, K0));
     }
-    const R tbr = tb * st.rho, tbd = tb * st.drho, one_cg = R(1) + cg, one_dg = R(1) + dg;
+    const R tbr = tb * st.rho, tbd = tb * st.drho, one_cg = R(1) + cg,
+            one_dg = fma(gA2, R(1.0 / 6.0), R(1));
     // P and B of shell s
     auto shell = [&](int s, R& P, R& B) {
         if constexpr (kF) {
@@ -1042,6 +1047,29 @@ struct Dims {
     int64_t plane;  // nx * ny * nz
     int64_t rows;   // 2 * ny * nz
 };
+
+// Division of n < 2^31 by a run-time constant d >= 1 as one multiply and shift
+// (Granlund and Montgomery, division by invariant integers using
+// multiplication, 1994): with 2^k >= d and m = ceil(2^(31+k) / d),
+// floor(n / d) = (n m) >> (31 + k).  Proof: write n = q d + r and
+// m d = 2^(31+k) + e with 0 <= e < d <= 2^k; then
+// n m / 2^(31+k) = q + (r + n e / 2^(31+k)) / d, and n e / 2^(31+k) < 1,
+// so the bracket stays below d.  m < 2^32 because d > 2^(k-1) for the
+// smallest such k.
+struct FastDiv {
+    uint32_t m, sh;
+};
+
+inline FastDiv make_fastdiv(uint32_t d) {
+    uint32_t k = 0;
+    while ((1ull << k) < d) ++k;
+    FastDiv f;
+    f.m = (uint32_t)(((1ull << (31 + k)) + d - 1) / d);
+    f.sh = 31 + k;
+    return f;
+}
+
+__device__ __forceinline__ uint32_t fdiv(uint32_t n, FastDiv f) { return (uint32_t)(((uint64_t)n * f.m) >> f.sh); }
 
 // coordinate of (a) wrapped into [0, n) for a in [-2, n + 1]
 __device__ __forceinline__ int wrap(int a, int n) {

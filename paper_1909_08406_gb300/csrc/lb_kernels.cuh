@@ -25,6 +25,79 @@ struct LoadCG {
         return __ldcg(p);
     }
 };
+template <class T>
+struct SameTypeOf {
+    using type = T;
+};
+template <class T>
+using SameType = typename SameTypeOf<T>::type;  // a parameter that takes no part in deduction
+
+
+// Entries of the direct step kernels.  Thread p takes entry p of the grid's x-fastest order, so only
+// the last block has idle threads whatever nx is (a block per row chunk left 22% of them idle at
+// nx = 150 or 200 and ran 24.9 and 27.4 GMLUPS there with 16-bit storage, against 30.7 and 32.2).
+// An entry is a node (kNode), the nodes (y, x) and (y + 1, x) of two rows, y even (kRows; ny even),
+// or the nodes x and x + 1, x even (kPair; nx even).
+enum EntryKind { kNode, kRows, kPair };
+
+struct EntryGrid {
+    uint32_t entries;  // of both sub-lattices, < 2^31
+    FastDiv fx, fy;    // by the entries per row, by the rows (row pairs) per plane
+};
+
+template <int KIND>
+inline EntryGrid entry_grid(const Dims& d) {
+    const uint32_t wx = (uint32_t)(KIND == kPair ? d.nx / 2 : d.nx), wy = (uint32_t)(KIND == kRows ? d.ny / 2 : d.ny);
+    return EntryGrid{2u * wx * wy * (uint32_t)d.nz, make_fastdiv(wx), make_fastdiv(wy)};
+}
+
+template <int KIND>
+__device__ __forceinline__ bool entry_node(const Dims& d, const EntryGrid& g, int& s, int& z, int& y, int& x) {
+    const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= g.entries) return false;
+    const uint32_t wx = KIND == kPair ? (uint32_t)d.nx >> 1 : (uint32_t)d.nx;
+    const uint32_t wy = KIND == kRows ? (uint32_t)d.ny >> 1 : (uint32_t)d.ny;
+    const uint32_t row = fdiv(p, g.fx), zs = fdiv(row, g.fy);
+    x = (int)(p - row * wx) * (KIND == kPair ? 2 : 1);
+    y = (int)(row - zs * wy) * (KIND == kRows ? 2 : 1);
+    s = zs >= (uint32_t)d.nz;
+    z = (int)zs - (s ? d.nz : 0);
+    return true;
+}
+
+// Base pointers and offsets of the two sub-lattices' populations.  Offsets into a population buffer are
+// 32-bit and hold the sub-lattice's start (one add forms a load's offset, one multiply-add its address);
+// with WIDE, for grids of 42 nx ny nz >= 2^32 elements, the start is in the base pointers.
+template <class T, bool WIDE>
+struct SubBases {
+    const T *own, *oth;
+    uint32_t o_own, o_oth;
+    __device__ __forceinline__ SubBases(const T* src, const Dims& d, int s) {
+        if constexpr (WIDE) {
+            own = src + (size_t)s * kQ * d.plane;
+            oth = src + (size_t)(1 - s) * kQ * d.plane;
+            o_own = o_oth = 0;
+        } else {
+            own = oth = src;
+            o_own = s ? (uint32_t)kQ * (uint32_t)d.plane : 0u;
+            o_oth = s ? 0u : (uint32_t)kQ * (uint32_t)d.plane;
+        }
+    }
+};
+template <class T, bool WIDE>
+__device__ __forceinline__ T* dst_base(T* dst, const Dims& d, int s) {
+    return WIDE ? dst + (size_t)s * kQ * d.plane : dst;
+}
+inline bool wide_offsets(const Dims& d) { return (uint64_t)(kQ + 1) * (uint64_t)d.plane >= ((uint64_t)1 << 32); }
+
+// Waits for the previous kernel's results.  Launched with the programmatic attribute (launch_entries), a
+// step's launch overlaps the previous step's tail: 33 x 18 x 20 nodes, FP32, 100 steps in a row, 2.7 us a
+// step against 5.1 without.  Steps do not trigger their successors early (launch_dependents at the start
+// of the kernel: 4.4 us, the waiting blocks of later steps take the SMs' slots).
+__device__ __forceinline__ void pdl_begin() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // Fused pull update (Sec. II) of one node (s, z, y, x): gather f*_i(x - c_i, t)
 // for all 41 velocities, compute the moments, the equilibrium and the BGK
 // relaxation, and write the 41 post-collision values.  Integer links stay on
@@ -32,131 +105,77 @@ struct LoadCG {
 // other sub-lattice: for A (s = 0) a component +1/2 reads cell r - 1 and -1/2
 // reads cell r; for B (s = 1) +1/2 reads cell r and -1/2 reads cell r + 1.
 // SR: BF16 storage with the stochastic store of lb_common.cuh, step key sr_key.
-template <class Codec, int EQ, class Ld = LoadNC, bool SR = false>
+template <class Codec, int EQ, class Ld = LoadNC, bool SR = false, bool WIDE = true>
 __device__ __forceinline__ void step_node(const typename Codec::raw_t* __restrict__ src,
                                           typename Codec::raw_t* __restrict__ dst, const Dims& d,
                                           const StepK<typename Codec::R, EQ>& K, typename Codec::R tb,
                                           int* __restrict__ err, int s, int z, int y, int x, uint32_t sr_key = 0) {
     using R = typename Codec::R;
     using T = typename Codec::raw_t;
-    const int64_t nxy = (int64_t)d.nx * d.ny;
+    const uint32_t nx = (uint32_t)d.nx, nxy = nx * (uint32_t)d.ny, plane = (uint32_t)d.plane;
+    const SubBases<T, WIDE> b(src, d, s);
 
     // coordinate / offset of the upwind cell for a shift delta = k - 2 (source = x - delta)
-    int xs[5];
-    int64_t yo[5], zo[5];
+    uint32_t xs[5], yo[5], zo[5];
 #pragma unroll
     for (int k = 0; k < 5; ++k) {
-        xs[k] = wrap(x - (k - 2), d.nx);
-        yo[k] = (int64_t)wrap(y - (k - 2), d.ny) * d.nx;
-        zo[k] = (int64_t)wrap(z - (k - 2), d.nz) * nxy;
+        xs[k] = (uint32_t)wrap(x - (k - 2), d.nx);
+        yo[k] = (uint32_t)wrap(y - (k - 2), d.ny) * nx;
+        zo[k] = (uint32_t)wrap(z - (k - 2), d.nz) * nxy + b.o_own;
     }
     // half links: component +1/2 has delta = 1 - s, component -1/2 has delta = -s
-    const int hxp = s ? xs[2] : xs[3], hxm = s ? xs[1] : xs[2];
-    const int64_t hyp = s ? yo[2] : yo[3], hym = s ? yo[1] : yo[2];
-    const int64_t hzp = s ? zo[2] : zo[3], hzm = s ? zo[1] : zo[2];
-
-    const T* same = src + (int64_t)s * kQ * d.plane;
-    const T* other = src + (int64_t)(1 - s) * kQ * d.plane;
+    const uint32_t hxp = s ? xs[2] : xs[3], hxm = s ? xs[1] : xs[2];
+    const uint32_t hyp = s ? yo[2] : yo[3], hym = s ? yo[1] : yo[2];
+    const uint32_t sub = b.o_oth - b.o_own;
+    const uint32_t hzp = (s ? zo[2] : zo[3]) + sub, hzm = (s ? zo[1] : zo[2]) + sub;
 
     R v[kQ];
     static_for<kQ>([&](auto I) {
         constexpr Vel c = vel(I);
         if constexpr (c.shell == 5) {
-            const int64_t off = (c.z > 0 ? hzp : hzm) + (c.y > 0 ? hyp : hym) + (c.x > 0 ? hxp : hxm);
-            v[I] = Codec::value(Ld::load(other + (int64_t)I * d.plane + off));
+            const uint32_t off = (c.z > 0 ? hzp : hzm) + (c.y > 0 ? hyp : hym) + (c.x > 0 ? hxp : hxm);
+            v[I] = Codec::value(Ld::load(b.oth + (size_t)I * plane + off));
         } else {
-            const int64_t off = zo[c.z / 2 + 2] + yo[c.y / 2 + 2] + xs[c.x / 2 + 2];
-            v[I] = Codec::value(Ld::load(same + (int64_t)I * d.plane + off));
+            const uint32_t off = zo[c.z / 2 + 2] + yo[c.y / 2 + 2] + xs[c.x / 2 + 2];
+            v[I] = Codec::value(Ld::load(b.own + (size_t)I * plane + off));
         }
     });
 
     const NodeState<R> st = step_state<Codec, EQ>(K, v);
     bool ok = state_ok(st);
 
-    const int64_t qn = (int64_t)z * nxy + (int64_t)y * d.nx + x;
-    T* out = dst + (int64_t)s * kQ * d.plane + qn;
+    const uint32_t qn = (uint32_t)z * nxy + (uint32_t)y * nx + (uint32_t)x;
+    T* out = dst_base<T, WIDE>(dst, d, s) + (b.o_own + qn);
     if constexpr (SR) {
-        const uint32_t q = (uint32_t)((int64_t)s * d.plane + qn);
+        const uint32_t q = (s ? plane : 0u) + qn;
         const uint32_t s0 = pcg_hash(sr_key ^ (q >> 1));
         step_relax<Codec, EQ>(st, K, tb * R(Codec::kScale), R(1) - tb, v,
-                                     [&](auto I, R val) {
-                                         const uint32_t w = sr_word<decltype(I)::value>(s0);
-                                         out[(int64_t)I * d.plane] = sr_bf16(val, (q & 1u) ? (w >> 16) : (w & 0xFFFFu));
-                                     },
-                                     ok);
+                              [&](auto I, R val) {
+                                  const uint32_t w = sr_word<decltype(I)::value>(s0);
+                                  out[(size_t)I * plane] = sr_bf16(val, (q & 1u) ? (w >> 16) : (w & 0xFFFFu));
+                              },
+                              ok);
     } else {
         step_relax<Codec, EQ>(st, K, tb * R(Codec::kScale), R(1) - tb, v,
-                                     [&](auto I, R val) { out[(int64_t)I * d.plane] = Codec::to_raw(val); }, ok);
+                              [&](auto I, R val) { out[(size_t)I * plane] = Codec::to_raw(val); }, ok);
     }
     if (!ok) atomicOr(err, 1);
 }
 
-// Direct-load step kernel.  Grid: blockIdx.x = row (s, z, y),
-// blockIdx.y * blockDim.x + threadIdx.x = x.  EQ: equilibrium kind (see
-// step_relax).
-template <class Codec, int EQ>
-__global__ void __launch_bounds__(kStepThreads) k_step(const typename Codec::raw_t* __restrict__ src,
-                                                       typename Codec::raw_t* __restrict__ dst, Dims d,
+// One node per thread.  EQ: equilibrium kind (see step_relax).
+template <class Codec, int EQ, bool WIDE, bool SR = false>
+__global__ void __launch_bounds__(kStepThreads, sizeof(typename Codec::R) == 8 && EQ < 2 ? 4 : 1) k_step(const typename Codec::raw_t* __restrict__ src,
+                                                       typename Codec::raw_t* __restrict__ dst, Dims d, EntryGrid g,
                                                        StepK<typename Codec::R, EQ> K, typename Codec::R tb,
-                                                       int* __restrict__ err) {
-    const int x = blockIdx.y * blockDim.x + threadIdx.x;
-    if (x >= d.nx) return;
-    const int64_t row = blockIdx.x;
-    const int y = (int)(row % d.ny);
-    const int64_t zr = row / d.ny;
-    const int z = (int)(zr % d.nz);
-    const int s = (int)(zr / d.nz);
-    step_node<Codec, EQ>(src, dst, d, K, tb, err, s, z, y, x);
+                                                       int* __restrict__ err, uint32_t sr_key) {
+    int s, z, y, x;
+    const bool active = entry_node<kNode>(d, g, s, z, y, x);
+    pdl_begin();
+    if (active) step_node<Codec, EQ, LoadNC, SR, WIDE>(src, dst, d, K, tb, err, s, z, y, x, sr_key);
 }
 
-template <class Codec, bool PROJECT, class Ld>
-__device__ __forceinline__ void step_node2(const typename Codec::raw_t* __restrict__ src,
-                                           typename Codec::raw_t* __restrict__ dst, const Dims& d,
-                                           const StepConsts<float2>& K, float tb, int* __restrict__ err, int s, int z,
-                                           int y, int x);
-
-// k_step with the stochastic BF16 store (series equilibrium with the momentum projection).
-template <class Codec>
-__global__ void __launch_bounds__(kStepThreads) k_step_sr(const typename Codec::raw_t* __restrict__ src,
-                                                          typename Codec::raw_t* __restrict__ dst, Dims d,
-                                                          StepConsts<typename Codec::R> K, typename Codec::R tb,
-                                                          int* __restrict__ err, uint32_t sr_key) {
-    const int x = blockIdx.y * blockDim.x + threadIdx.x;
-    if (x >= d.nx) return;
-    const int64_t row = blockIdx.x;
-    const int y = (int)(row % d.ny);
-    const int64_t zr = row / d.ny;
-    const int z = (int)(zr % d.nz);
-    const int s = (int)(zr / d.nz);
-    step_node<Codec, 1, LoadNC, true>(src, dst, d, K, tb, err, s, z, y, x, sr_key);
-}
-
-// Two-rows-per-thread direct-load step kernel (FP32 arithmetic, any storage
-// except FP64): each thread updates nodes (s, z, y, x) and (s, z, y + 1, x)
-// with packed FP32x2 arithmetic.  Addresses are formed from 32-bit in-plane
-// offsets (the host guarantees nx * ny * nz < 2^32) plus plane * I.  Blocks
-// are numbered chunk-fastest, so the CTAs covering one row segment run
-// together and the sectors they share at chunk and wrap boundaries stay in
-// L2.  Requires ny even.  Grid: (nz * ny / 2 * 2 sub-lattices) * chunks blocks.
-template <class Codec, bool PROJECT, int MINB>
-__global__ void __launch_bounds__(kStepThreads, MINB) k_step2(const typename Codec::raw_t* __restrict__ src,
-                                                        typename Codec::raw_t* __restrict__ dst, Dims d,
-                                                        StepConsts<float2> K, float tb, int* __restrict__ err,
-                                                        int chunks) {
-    const int64_t t = blockIdx.x;
-    const int64_t rp = t / chunks;
-    const int x = (int)(t - rp * chunks) * blockDim.x + threadIdx.x;
-    if (x >= d.nx) return;
-    const int nyh = d.ny >> 1;
-    const int y = 2 * (int)(rp % nyh);
-    const int64_t zr = rp / nyh;
-    const int z = (int)(zr % d.nz);
-    const int s = (int)(zr / d.nz);
-    step_node2<Codec, PROJECT, LoadNC>(src, dst, d, K, tb, err, s, z, y, x);
-}
-
-// Nodes (s, z, y, x) and (s, z, y + 1, x) (y even), packed FP32x2 arithmetic; see k_step2.
-template <class Codec, bool PROJECT, class Ld>
+// Nodes (s, z, y, x) and (s, z, y + 1, x) (y even), packed FP32x2 arithmetic.
+template <class Codec, bool PROJECT, class Ld, bool WIDE = true>
 __device__ __forceinline__ void step_node2(const typename Codec::raw_t* __restrict__ src,
                                            typename Codec::raw_t* __restrict__ dst, const Dims& d,
                                            const StepConsts<float2>& K, float tb, int* __restrict__ err, int s, int z,
@@ -165,6 +184,7 @@ __device__ __forceinline__ void step_node2(const typename Codec::raw_t* __restri
     using C2 = Codec2<Codec>;
     const uint32_t nx = (uint32_t)d.nx, nxy = (uint32_t)d.nx * (uint32_t)d.ny;
     const uint32_t plane = (uint32_t)d.plane;
+    const SubBases<T, WIDE> b(src, d, s);
 
     // source coordinates: x - delta for delta = k - 2; rows y + k - 2 for k = 0..5 (covers
     // y - delta for the first node and y + 1 - delta for the second); planes z - delta
@@ -172,17 +192,16 @@ __device__ __forceinline__ void step_node2(const typename Codec::raw_t* __restri
 #pragma unroll
     for (int k = 0; k < 5; ++k) {
         xs[k] = (uint32_t)wrap(x - (k - 2), d.nx);
-        zo[k] = (uint32_t)wrap(z - (k - 2), d.nz) * nxy;
+        zo[k] = (uint32_t)wrap(z - (k - 2), d.nz) * nxy + b.o_own;
     }
 #pragma unroll
     for (int k = 0; k < 6; ++k) yo[k] = (uint32_t)wrap(y + k - 2, d.ny) * nx;
     // half links: delta = 1 - s for a +1/2 component, -s for -1/2; the row index is 2 - delta
     const uint32_t hxp = s ? xs[2] : xs[3], hxm = s ? xs[1] : xs[2];
-    const uint32_t hzp = s ? zo[2] : zo[3], hzm = s ? zo[1] : zo[2];
-    const int kyp = 1 + s, kym = 2 + s;  // 2 - delta for +1/2 and -1/2
-
-    const T* same = src + (size_t)s * kQ * d.plane;
-    const T* other = src + (size_t)(1 - s) * kQ * d.plane;
+    const uint32_t sub = b.o_oth - b.o_own;
+    const uint32_t hzp = (s ? zo[2] : zo[3]) + sub, hzm = (s ? zo[1] : zo[2]) + sub;
+    // rows of the +1/2 and -1/2 components for the first and the second node
+    const uint32_t hyp[2] = {s ? yo[2] : yo[1], s ? yo[3] : yo[2]}, hym[2] = {s ? yo[3] : yo[2], s ? yo[4] : yo[3]};
 
     // the two nodes' stored values stay packed (one register per population for 16-bit
     // storage) and are widened to FP32 where they are used
@@ -193,15 +212,14 @@ __device__ __forceinline__ void step_node2(const typename Codec::raw_t* __restri
         const T* base;
         if constexpr (c.shell == 5) {
             const uint32_t xz = (c.z > 0 ? hzp : hzm) + (c.x > 0 ? hxp : hxm);
-            const int ky = c.y > 0 ? kyp : kym;
-            oa = xz + yo[ky];
-            ob = xz + yo[ky + 1];
-            base = other;
+            oa = xz + (c.y > 0 ? hyp[0] : hym[0]);
+            ob = xz + (c.y > 0 ? hyp[1] : hym[1]);
+            base = b.oth;
         } else {
             const uint32_t xz = zo[c.z / 2 + 2] + xs[c.x / 2 + 2];
             oa = xz + yo[2 - c.y / 2];
             ob = xz + yo[3 - c.y / 2];
-            base = same;
+            base = b.own;
         }
         const T* p = base + (size_t)I * plane;
         pv[I] = Codec::pack2(Ld::load(p + oa), Ld::load(p + ob));
@@ -211,25 +229,151 @@ __device__ __forceinline__ void step_node2(const typename Codec::raw_t* __restri
     const NodeState<F2> st = node_state<C2>(K, vget);
     if (!state_ok(st)) atomicOr(err, 1);
 
-    T* outa = dst + (size_t)s * kQ * d.plane + ((uint32_t)z * nxy + (uint32_t)y * nx + (uint32_t)x);
-    collide<C2, PROJECT>(st, K, F2(tb * (float)Codec::kScale), F2(1.f - tb), vget,
-                                     [&](auto I, F2 val) {
-                                         T* p = outa + (size_t)I * plane;
-                                         p[0] = Codec::to_raw(val.v.x);
-                                         p[nx] = Codec::to_raw(val.v.y);
-                                     });
+    T* outa = dst_base<T, WIDE>(dst, d, s) + (b.o_own + (uint32_t)z * nxy + (uint32_t)y * nx + (uint32_t)x);
+    collide<C2, PROJECT>(st, K, F2(tb * (float)Codec::kScale), F2(1.f - tb), vget, [&](auto I, F2 val) {
+        T* p = outa + (size_t)I * plane;
+        p[0] = Codec::to_raw(val.v.x);
+        p[nx] = Codec::to_raw(val.v.y);
+    });
 }
 
-// Two x-adjacent nodes per thread (16-bit storage): nodes (s, z, y, x) and
-// (s, z, y, x + 1), x even, packed FP32x2 arithmetic.  Each plane is read as
-// aligned pairs of 16-bit values: one 32-bit load when the plane's x shift is
-// even, two loads and a byte permute when it is odd; the two results of a
-// plane are written with one 32-bit store.
+// Two rows per thread (FP32 arithmetic, any storage except FP64; ny even).
+template <class Codec, bool PROJECT, int MINB, bool WIDE>
+__global__ void __launch_bounds__(kStepThreads, MINB) k_step2(const typename Codec::raw_t* __restrict__ src,
+                                                              typename Codec::raw_t* __restrict__ dst, Dims d,
+                                                              EntryGrid g, StepConsts<float2> K, float tb,
+                                                              int* __restrict__ err) {
+    int s, z, y, x;
+    const bool active = entry_node<kRows>(d, g, s, z, y, x);
+    pdl_begin();
+    if (active) step_node2<Codec, PROJECT, LoadNC, WIDE>(src, dst, d, K, tb, err, s, z, y, x);
+}
+
+// Two x-adjacent nodes (s, z, y, x) and (s, z, y, x + 1), x even, per thread (16-bit storage, nx
+// even), packed FP32x2 arithmetic.  Each plane is read as aligned pairs of 16-bit values: one 32-bit
+// load when the plane's x shift is even, two loads and a byte permute when it is odd; the two
+// results of a plane are written with one 32-bit store.
 //
-// A block covers one chunk of x for `rpb` consecutive rows (s, z, y), y
-// fastest, and each thread loads a row's 41 pairs at the start of that row
-// (MODE below says how the next row is brought closer meanwhile).  Requires
-// nx even and nx * ny * nz < 2^32.
+// Bound by the latency of its dependent arithmetic at the warps that fit: 128 registers (4 blocks, 16
+// warps per SM, 24 bytes of spills); 33.5 GMLUPS on 256^3 with FP16 storage, 81% of the copy bandwidth
+// (a block per row chunk with the next row prefetched into L2: 32.2; 168 registers, 12 warps: 29.4).
+// SR: BF16 storage with the stochastic store of lb_common.cuh, step key sr_key (one word per
+// population and x pair).
+template <class Codec, bool PROJECT, bool WIDE, bool SR = false>
+__global__ void __launch_bounds__(kStepThreads, 4) k_step2x(const typename Codec::raw_t* __restrict__ src,
+                                                            typename Codec::raw_t* __restrict__ dst, Dims d,
+                                                            EntryGrid g, StepConsts<float2> K, float tb,
+                                                            int* __restrict__ err, uint32_t sr_key) {
+    using T = typename Codec::raw_t;
+    using P = typename Codec::pair_t;
+    using C2 = Codec2<Codec>;
+    int s, z, y, x;
+    const bool active = entry_node<kPair>(d, g, s, z, y, x);
+    pdl_begin();
+    if (!active) return;
+    const uint32_t nx = (uint32_t)d.nx, nxy = nx * (uint32_t)d.ny, plane = (uint32_t)d.plane;
+    const SubBases<T, WIDE> b(src, d, s);
+    uint32_t yo[5], zo[5];
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+        yo[k] = (uint32_t)wrap(y - (k - 2), d.ny) * nx;
+        zo[k] = (uint32_t)wrap(z - (k - 2), d.nz) * nxy + b.o_own;
+    }
+    const uint32_t sub = b.o_oth - b.o_own;
+    const uint32_t hyp = s ? yo[2] : yo[3], hym = s ? yo[1] : yo[2];
+    const uint32_t hzp = (s ? zo[2] : zo[3]) + sub, hzm = (s ? zo[1] : zo[2]) + sub;
+    // aligned pair starts: x - 2, x, x + 2 (periodic; nx even keeps them even)
+    const uint32_t xm = (uint32_t)wrap(x - 2, d.nx), x0 = (uint32_t)x, xq = (uint32_t)wrap(x + 2, d.nx);
+    // half links along x: A's +1/2 component straddles the pairs x - 2 and x, B's -1/2 one the pairs x
+    // and x + 2; the other two are the pair x itself (both pairs of the permute at x, a whole taken)
+    const uint32_t hlo = s ? x0 : xm, hhi = s ? xq : x0;
+    const uint32_t sel_p = s ? 0x7654u : 0x5432u, sel_m = s ? 0x5432u : 0x3210u;
+
+    P pv[kQ];
+    static_for<kQ>([&](auto I) {
+        constexpr Vel c = vel(I);
+        const T* base = (c.shell == 5 ? b.oth : b.own) + (size_t)I * plane;
+        auto ld = [&](uint32_t off) { return LoadNC::load(reinterpret_cast<const P*>(base + off)); };
+        if constexpr (c.shell == 5) {
+            const uint32_t row = (c.z > 0 ? hzp : hzm) + (c.y > 0 ? hyp : hym);
+            const P lo = ld(row + (c.x > 0 ? hlo : x0)), hi = ld(row + (c.x > 0 ? x0 : hhi));
+            uint32_t wl, wh;
+            memcpy(&wl, &lo, 4);
+            memcpy(&wh, &hi, 4);
+            const uint32_t w = __byte_perm(wl, wh, c.x > 0 ? sel_p : sel_m);
+            memcpy(&pv[I], &w, 4);
+        } else {
+            const uint32_t row = zo[c.z / 2 + 2] + yo[c.y / 2 + 2];
+            if constexpr (c.x == 4)
+                pv[I] = ld(row + xm);
+            else if constexpr (c.x == 2)
+                pv[I] = Codec::straddle(ld(row + xm), ld(row + x0));
+            else if constexpr (c.x == 0)
+                pv[I] = ld(row + x0);
+            else if constexpr (c.x == -2)
+                pv[I] = Codec::straddle(ld(row + x0), ld(row + xq));
+            else
+                pv[I] = ld(row + xq);
+        }
+    });
+    auto vget = [&](auto I) { return F2(Codec::unpack2(pv[I])); };
+    const NodeState<F2> st = node_state<C2>(K, vget);
+    if (!state_ok(st)) atomicOr(err, 1);
+    // The values stay packed from here to their relaxation: without the barrier the compiler keeps
+    // the 82 widened numbers of the sums alive and spills more.
+    static_for<kQ>([&](auto I) {
+        uint32_t w;
+        memcpy(&w, &pv[I], sizeof w);
+        asm volatile("" : "+r"(w));
+        memcpy(&pv[I], &w, sizeof w);
+    });
+    const uint32_t qn = (uint32_t)z * nxy + (uint32_t)y * nx + x0;
+    T* out = dst_base<T, WIDE>(dst, d, s) + (b.o_own + qn);
+    uint32_t s0 = 0;
+    if constexpr (SR) s0 = pcg_hash(sr_key ^ (((s ? plane : 0u) + qn) >> 1));
+    collide<C2, PROJECT>(st, K, F2(tb * (float)Codec::kScale), F2(1.f - tb), vget, [&](auto I, F2 val) {
+        P* o = reinterpret_cast<P*>(out + (size_t)I * plane);
+        if constexpr (SR)
+            *o = sr_bf16x2(val.v, sr_word<decltype(I)::value>(s0));
+        else
+            *o = Codec::to_raw2(val.v);
+    });
+}
+
+// Entries that leave an SM fewer than this many warps run one node per thread instead (the same bits):
+// latency counts there, not work per thread (33 x 18 x 20 FP32: 2.7 against 3.4 us a step; FP16 pairs
+// already win at 28^3, 3.7 against 3.9, FP32 rows from 40^3, 6.3 against 6.9).
+constexpr int64_t kSms = 152;
+template <int KIND>
+inline bool few_entries(const Dims& d) {
+    const int64_t warps = KIND == kPair ? 4 : 8;
+    return d.plane < kSms * warps * 32;  // entries of two nodes: as many as cells
+}
+
+// Launches `kern` over the KIND entries of the grid with the programmatic attribute (pdl_begin).  Blocks of
+// 128 threads, smaller ones where those would leave fewer than eight per SM, down to a warp, so that the
+// last wave is short.
+template <int KIND, class T, class... A>
+inline cudaError_t launch_entries(void (*kern)(const T*, T*, Dims, EntryGrid, A...), const void* src, void* dst,
+                                  const Dims& d, cudaStream_t st, const SameType<A>&... args) {
+    if (d.plane >= ((int64_t)1 << 30)) return cudaErrorInvalidValue;  // 32-bit entries (such a state exceeds the memory)
+    const EntryGrid g = entry_grid<KIND>(d);
+    constexpr uint32_t kEnough = (uint32_t)kSms * 8u;
+    const uint32_t th = g.entries >= kEnough * 128u ? 128u : g.entries >= kEnough * 64u ? 64u : 32u;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((g.entries + th - 1) / th);
+    cfg.blockDim = dim3(th);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<const T*>(src), static_cast<T*>(dst), d, g, args...);
+}
+
+// Row addresses of the nonideal fluid's x-pair passes: the pair of upwind values of one population for
+// the nodes x, x + 1 of a row (s, z, y) that the whole block shares.
 template <class Codec>
 struct RowAddr2x {
     using T = typename Codec::raw_t;
@@ -311,100 +455,6 @@ __device__ __forceinline__ void prefetch_row_l2(const typename Codec::raw_t* src
     const uintptr_t b1 = ((uintptr_t)(row + hi)) & ~(uintptr_t)15;
     if (b1 > b0)
         asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(b0), "r"((uint32_t)(b1 - b0)) : "memory");
-}
-
-// How a block of the x-pair kernel gets a row's upwind values:
-// MODE 0: direct loads at the start of the row.
-// MODE 2: as MODE 0, plus an L2 bulk prefetch of the next row's source rows
-//         (one per population, by threads 0..40; a block of only 32 threads,
-//         on a narrow grid, prefetches its first 32 populations) at the start
-//         of the current row, so that the next row's loads hit in L2.
-// SR: BF16 storage with the stochastic store of lb_common.cuh, step key sr_key (one word per
-// population and x pair).
-template <class Codec, bool PROJECT, int MINB, int MODE, bool SR = false>
-__global__ void __launch_bounds__(kStepThreads, MINB) k_step2x(const typename Codec::raw_t* __restrict__ src,
-                                                         typename Codec::raw_t* __restrict__ dst, Dims d,
-                                                         StepConsts<float2> K, float tb, int* __restrict__ err,
-                                                         int chunks, int rpb, uint32_t sr_key) {
-    using T = typename Codec::raw_t;
-    using P = typename Codec::pair_t;
-    using C2 = Codec2<Codec>;
-    const uint32_t t = blockIdx.x;
-    const uint32_t grp = t / (uint32_t)chunks;
-    const int chunk = (int)(t - grp * (uint32_t)chunks);
-    const int x = 2 * (chunk * (int)blockDim.x + (int)threadIdx.x);
-    const int xa = 2 * chunk * (int)blockDim.x, xb = min(xa + 2 * (int)blockDim.x, d.nx);
-    const uint32_t r0 = grp * (uint32_t)rpb;
-    const uint32_t r1 = min(r0 + (uint32_t)rpb, (uint32_t)d.rows);
-    int y = (int)(r0 % (uint32_t)d.ny);
-    const uint32_t zr = r0 / (uint32_t)d.ny;
-    int z = (int)(zr % (uint32_t)d.nz);
-    int s = (int)(zr / (uint32_t)d.nz);
-    const bool active = x < d.nx;
-    if (!active && (MODE != 2 || threadIdx.x >= kQ)) return;  // threads < 41 issue prefetches
-    const uint32_t nx = (uint32_t)d.nx, nxy = (uint32_t)d.nx * (uint32_t)d.ny;
-    const uint32_t plane = (uint32_t)d.plane;
-
-    // aligned pair starts: x - 2, x, x + 2 (periodic; nx even keeps them even)
-    const uint32_t xm = (uint32_t)wrap(x - 2, d.nx), x0 = (uint32_t)x, xq = (uint32_t)wrap(x + 2, d.nx);
-
-    P pv[kQ];
-    auto vget = [&](auto I) { return F2(Codec::unpack2(pv[I])); };
-
-    for (uint32_t r = r0; r < r1; ++r) {
-        // the next row, in (s, z, y) order
-        int yn = y + 1, zn = z, sn = s;
-        if (yn == d.ny) {
-            yn = 0;
-            if (++zn == d.nz) {
-                zn = 0;
-                ++sn;
-            }
-        }
-        const bool more = r + 1 < r1;
-        if constexpr (MODE == 2) {
-            if (more && threadIdx.x < kQ) prefetch_row_l2<Codec>(src, d, (int)threadIdx.x, sn, zn, yn, xa, xb);
-            if (!active) {
-                s = sn;
-                z = zn;
-                y = yn;
-                continue;
-            }
-        }
-        {
-            RowAddr2x<Codec> a;
-            a.set(src, d, s, z, y);
-            static_for<kQ>([&](auto I) { pv[I] = load_pair2x<Codec, I>(a, plane, xm, x0, xq); });
-        }
-
-        const NodeState<F2> st = node_state<C2>(K, vget);
-        if (!state_ok(st)) atomicOr(err, 1);
-        // The values stay packed from here to their relaxation: without the barrier the compiler keeps
-        // the 82 widened numbers of the sums alive and spills at 128 registers.
-        static_for<kQ>([&](auto I) {
-            uint32_t w;
-            memcpy(&w, &pv[I], sizeof w);
-            asm volatile("" : "+r"(w));
-            memcpy(&pv[I], &w, sizeof w);
-        });
-
-        P* outp = reinterpret_cast<P*>(dst + (size_t)s * kQ * d.plane + ((uint32_t)z * nxy + (uint32_t)y * nx + x0));
-        if constexpr (SR) {
-            const uint32_t q = (uint32_t)s * plane + (uint32_t)z * nxy + (uint32_t)y * nx + x0;
-            const uint32_t s0 = pcg_hash(sr_key ^ (q >> 1));
-            collide<C2, PROJECT>(st, K, F2(tb * (float)Codec::kScale), F2(1.f - tb), vget,
-                                             [&](auto I, F2 val) {
-                                                 outp[(size_t)I * (plane / 2)] =
-                                                     sr_bf16x2(val.v, sr_word<decltype(I)::value>(s0));
-                                             });
-        } else {
-            collide<C2, PROJECT>(st, K, F2(tb * (float)Codec::kScale), F2(1.f - tb), vget,
-                                             [&](auto I, F2 val) { outp[(size_t)I * (plane / 2)] = Codec::to_raw2(val.v); });
-        }
-        s = sn;
-        z = zn;
-        y = yn;
-    }
 }
 
 // Populations = equilibrium of the given float64 fields, for nodes

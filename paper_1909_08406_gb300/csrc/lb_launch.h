@@ -138,9 +138,6 @@ cudaError_t launch_nonideal_step(int prec, const void* src, void* dst, const Dim
                                  double twobeta, int kind, const double eos[4], double* work, int* err,
                                  cudaStream_t st);
 
-inline dim3 step_grid(const Dims& d, int threads) {
-    return dim3((unsigned)d.rows, (unsigned)((d.nx + threads - 1) / threads), 1);
-}
 inline int step_threads(const Dims& d) {
     return d.nx >= 128 ? 128 : ((d.nx + 31) / 32) * 32;
 }

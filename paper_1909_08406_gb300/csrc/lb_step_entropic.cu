@@ -9,17 +9,10 @@ namespace gblb {
 
 cudaError_t launch_step_entropic(int prec, int eq, const void* src, void* dst, const Dims& d, const LaunchConsts& c,
                                  double twobeta, int* err, cudaStream_t st) {
-    const int th = step_threads(d);
     auto run = [&](auto codec) {
         using C = decltype(codec);
-        using T = typename C::raw_t;
-        if (eq == 3)
-            k_step<C, 3><<<step_grid(d, th), th, 0, st>>>(static_cast<const T*>(src), static_cast<T*>(dst), d, c.kf,
-                                                          (float)twobeta, err);
-        else
-            k_step<C, 2><<<step_grid(d, th), th, 0, st>>>(static_cast<const T*>(src), static_cast<T*>(dst), d, c.kf,
-                                                          (float)twobeta, err);
-        return cudaGetLastError();
+        return launch_entries<kNode>(eq == 3 ? k_step<C, 3, true> : k_step<C, 2, true>, src, dst, d, st, c.kf,
+                                     (float)twobeta, err, 0u);
     };
     switch (prec) {
         case kF32: return run(CodecF32{});

@@ -1,7 +1,9 @@
 // FP32-arithmetic step kernels (FP32, FP16 and BF16 storage).  Variants:
 //   kKernelDirect1   k_step:        one node per thread, direct global loads
-//   kKernelDirect2   k_step2<.,.,4>: two rows per thread, packed FP32x2 math, 4 CTAs/SM
-//   kKernelDirect2R  k_step2<.,.,3>: the same, register budget for 3 CTAs/SM
+//   kKernelDirect2   k_step2<.,.,3>: two rows per thread, packed FP32x2 math
+//   kKernelDirect2R  k_step2<.,.,4>: the same, register budget for 4 CTAs/SM
+//   kKernelDirect2X, kKernelDirect2XL
+//                    k_step2x: two x-adjacent nodes per thread, 16-bit storage
 //   kKernelStaged    k_step_tma:    rows fetched by TMA bulk copies into a
 //                                   shared-memory ring
 //   kKernelWarpSpec  k_step_ws:     the same staging with a dedicated producer
@@ -15,44 +17,30 @@
 
 namespace gblb {
 
-template <class Codec, bool P>
+template <class Codec, bool P, bool SR = false>
 static cudaError_t run_direct1(const void* src, void* dst, const Dims& d, const LaunchConsts& c, double twobeta,
-                               int* err, cudaStream_t st) {
-    using T = typename Codec::raw_t;
-    const int th = step_threads(d);
-    k_step<Codec, P><<<step_grid(d, th), th, 0, st>>>(static_cast<const T*>(src), static_cast<T*>(dst), d, (step_consts<Codec, 0>(c)),
-                                                      (float)twobeta, err);
-    return cudaGetLastError();
+                               int* err, cudaStream_t st, uint32_t sr_key = 0) {
+    return launch_entries<kNode>(wide_offsets(d) ? k_step<Codec, P, true, SR> : k_step<Codec, P, false, SR>, src, dst,
+                                 d, st, step_consts<Codec, P>(c), (float)twobeta, err, sr_key);
 }
 
 template <class Codec, bool P, int MINB>
 static cudaError_t run_direct2(const void* src, void* dst, const Dims& d, const LaunchConsts& c, double twobeta,
                                int* err, cudaStream_t st) {
-    using T = typename Codec::raw_t;
-    const int th = step_threads(d);
-    const int chunks = (d.nx + th - 1) / th;
-    const int64_t blocks = d.rows / 2 * chunks;
-    k_step2<Codec, P, MINB><<<(unsigned)blocks, th, 0, st>>>(static_cast<const T*>(src), static_cast<T*>(dst), d,
-                                                             pair_consts<Codec>(c), (float)twobeta, err, chunks);
-    return cudaGetLastError();
+    if (few_entries<kRows>(d)) return run_direct1<Codec, P>(src, dst, d, c, twobeta, err, st);
+    return launch_entries<kRows>(wide_offsets(d) ? k_step2<Codec, P, MINB, true> : k_step2<Codec, P, MINB, false>,
+                                 src, dst, d, st, pair_consts<Codec>(c), (float)twobeta, err);
 }
 
-template <class Codec, bool P, int MINB, int MODE, bool SR = false>
+template <class Codec, bool P, bool SR = false>
 static cudaError_t run_direct2x(const void* src, void* dst, const Dims& d, const LaunchConsts& c, double twobeta,
-                                int* err, cudaStream_t st, int rpb, uint32_t sr_key = 0) {
-    using T = typename Codec::raw_t;
-    if constexpr (sizeof(T) != 2) {
-        return cudaErrorInvalidValue;
-    } else {
-        const int half = d.nx / 2;
-        const int th = half >= 128 ? 128 : ((half + 31) / 32) * 32;
-        const int chunks = (half + th - 1) / th;
-        const int64_t blocks = ((d.rows + rpb - 1) / rpb) * chunks;
-        auto kern = k_step2x<Codec, P, MINB, MODE, SR>;
-        kern<<<(unsigned)blocks, th, 0, st>>>(static_cast<const T*>(src), static_cast<T*>(dst), d, pair_consts<Codec>(c),
-                                                 (float)twobeta, err, chunks, rpb, sr_key);
-        return cudaGetLastError();
+                                int* err, cudaStream_t st, uint32_t sr_key = 0) {
+    if constexpr (sizeof(typename Codec::raw_t) == 2) {
+        if (few_entries<kPair>(d)) return run_direct1<Codec, P, SR>(src, dst, d, c, twobeta, err, st, sr_key);
+        return launch_entries<kPair>(wide_offsets(d) ? k_step2x<Codec, P, true, SR> : k_step2x<Codec, P, false, SR>,
+                                     src, dst, d, st, pair_consts<Codec>(c), (float)twobeta, err, sr_key);
     }
+    return cudaErrorInvalidValue;
 }
 
 // Per-instance launch data: dynamic shared memory opt-in and the persistent grid size.
@@ -185,9 +173,8 @@ static cudaError_t step_codec(int prec, int kernel, const void* src, void* dst, 
                 return run_tma<Codec, P, typename TmaShape<Codec, 256>::Cfg>(src, dst, d, c, twobeta, err, st);
             return run_tma<Codec, P, typename TmaShape<Codec, 128>::Cfg>(src, dst, d, c, twobeta, err, st);
         case kKernelWarpSpec: return run_ws<Codec, P, typename WsShape<Codec>::Cfg>(src, dst, d, c, twobeta, err, st);
-        case kKernelDirect2X: return run_direct2x<Codec, P, 4, 0>(src, dst, d, c, twobeta, err, st, 1);
-        case kKernelDirect2XL: return run_direct2x<Codec, P, 4, 2>(src, dst, d, c, twobeta, err, st, 2);
-
+        case kKernelDirect2X:
+        case kKernelDirect2XL: return run_direct2x<Codec, P>(src, dst, d, c, twobeta, err, st);
         case kKernelDirect2: return run_direct2<Codec, P, 4>(src, dst, d, c, twobeta, err, st);
         case kKernelDirect2R: return run_direct2<Codec, P, 3>(src, dst, d, c, twobeta, err, st);
         default: return run_direct1<Codec, P>(src, dst, d, c, twobeta, err, st);
@@ -214,13 +201,9 @@ cudaError_t launch_step_f32(int prec, bool project, int kernel, const void* src,
 // the x-pair kernel where it applies, else one node per thread.
 cudaError_t launch_step_sr(const void* src, void* dst, const Dims& d, const LaunchConsts& c, double twobeta, int* err,
                            cudaStream_t st, uint32_t sr_key) {
-    using T = CodecBF16::raw_t;
     if (resolve_kernel(kBF16, d, kKernelDirect2XL) == kKernelDirect2XL)
-        return run_direct2x<CodecBF16, true, 4, 2, true>(src, dst, d, c, twobeta, err, st, 2, sr_key);
-    const int th = step_threads(d);
-    k_step_sr<CodecBF16><<<step_grid(d, th), th, 0, st>>>(static_cast<const T*>(src), static_cast<T*>(dst), d,
-                                                         c.sf[0], (float)twobeta, err, sr_key);
-    return cudaGetLastError();
+        return run_direct2x<CodecBF16, true, true>(src, dst, d, c, twobeta, err, st, sr_key);
+    return run_direct1<CodecBF16, true, true>(src, dst, d, c, twobeta, err, st, sr_key);
 }
 
 }  // namespace gblb

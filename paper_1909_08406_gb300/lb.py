@@ -34,7 +34,7 @@ KERNEL_NAMES = {0: "k_step (direct, 1 node/thread)", 1: "k_step2 (direct, 2 rows
                 2: "k_step2 (direct, 2 rows/thread, FP32x2, 3 CTAs/SM)", 3: "k_step_tma (TMA-staged)",
                 4: "k_step_ws (TMA-staged, warp-specialised, FP32x2)",
                 5: "k_step2x (direct, 2 x-adjacent nodes/thread, FP32x2, paired 16-bit access)",
-                6: "k_step2x (x pairs, 2 rows/block, next row prefetched into L2)"}
+                6: "k_step2x (direct, 2 x-adjacent nodes/thread, FP32x2, paired 16-bit access)"}
 
 
 class LbError(RuntimeError):
