@@ -10,9 +10,16 @@ namespace gblb {
 
 constexpr int kStepThreads = 128;
 
-// Load paths: the read-only (non-coherent) path for kernels whose inputs no
-// thread of the same launch writes, and L2-coherent loads for persistent
-// kernels that read, after a grid barrier, what other CTAs wrote.
+// Load paths: the read-only (non-coherent) path for kernels whose inputs are complete before their
+// launch, ordinary loads for kernels that start before the kernel that writes their inputs has ended
+// (pdl_begin: a non-coherent load may be moved across the wait), and L2-coherent loads for
+// persistent kernels that read, after a grid barrier, what other CTAs wrote.
+struct LoadCA {
+    template <class T>
+    static __device__ __forceinline__ T load(const T* p) {
+        return __ldca(p);
+    }
+};
 struct LoadNC {
     template <class T>
     static __device__ __forceinline__ T load(const T* p) {
@@ -25,13 +32,13 @@ struct LoadCG {
         return __ldcg(p);
     }
 };
+
 template <class T>
 struct SameTypeOf {
     using type = T;
 };
 template <class T>
 using SameType = typename SameTypeOf<T>::type;  // a parameter that takes no part in deduction
-
 
 // Entries of the direct step kernels.  Thread p takes entry p of the grid's x-fastest order, so only
 // the last block has idle threads whatever nx is (a block per row chunk left 22% of them idle at
@@ -163,15 +170,20 @@ __device__ __forceinline__ void step_node(const typename Codec::raw_t* __restric
 }
 
 // One node per thread.  EQ: equilibrium kind (see step_relax).
+// FP32 arithmetic fits 80 registers (6 blocks per SM), FP64 128 (4).
+template <class Codec, int EQ>
+constexpr int step_min_blocks() {
+    return EQ >= 2 ? 1 : sizeof(typename Codec::R) == 8 ? 4 : 6;
+}
 template <class Codec, int EQ, bool WIDE, bool SR = false>
-__global__ void __launch_bounds__(kStepThreads, sizeof(typename Codec::R) == 8 && EQ < 2 ? 4 : 1) k_step(const typename Codec::raw_t* __restrict__ src,
+__global__ void __launch_bounds__(kStepThreads, step_min_blocks<Codec, EQ>()) k_step(const typename Codec::raw_t* __restrict__ src,
                                                        typename Codec::raw_t* __restrict__ dst, Dims d, EntryGrid g,
                                                        StepK<typename Codec::R, EQ> K, typename Codec::R tb,
                                                        int* __restrict__ err, uint32_t sr_key) {
     int s, z, y, x;
     const bool active = entry_node<kNode>(d, g, s, z, y, x);
     pdl_begin();
-    if (active) step_node<Codec, EQ, LoadNC, SR, WIDE>(src, dst, d, K, tb, err, s, z, y, x, sr_key);
+    if (active) step_node<Codec, EQ, LoadCA, SR, WIDE>(src, dst, d, K, tb, err, s, z, y, x, sr_key);
 }
 
 // Nodes (s, z, y, x) and (s, z, y + 1, x) (y even), packed FP32x2 arithmetic.
@@ -246,7 +258,7 @@ __global__ void __launch_bounds__(kStepThreads, MINB) k_step2(const typename Cod
     int s, z, y, x;
     const bool active = entry_node<kRows>(d, g, s, z, y, x);
     pdl_begin();
-    if (active) step_node2<Codec, PROJECT, LoadNC, WIDE>(src, dst, d, K, tb, err, s, z, y, x);
+    if (active) step_node2<Codec, PROJECT, LoadCA, WIDE>(src, dst, d, K, tb, err, s, z, y, x);
 }
 
 // Two x-adjacent nodes (s, z, y, x) and (s, z, y, x + 1), x even, per thread (16-bit storage, nx
@@ -293,7 +305,7 @@ __global__ void __launch_bounds__(kStepThreads, 4) k_step2x(const typename Codec
     static_for<kQ>([&](auto I) {
         constexpr Vel c = vel(I);
         const T* base = (c.shell == 5 ? b.oth : b.own) + (size_t)I * plane;
-        auto ld = [&](uint32_t off) { return LoadNC::load(reinterpret_cast<const P*>(base + off)); };
+        auto ld = [&](uint32_t off) { return LoadCA::load(reinterpret_cast<const P*>(base + off)); };
         if constexpr (c.shell == 5) {
             const uint32_t row = (c.z > 0 ? hzp : hzm) + (c.y > 0 ? hyp : hym);
             const P lo = ld(row + (c.x > 0 ? hlo : x0)), hi = ld(row + (c.x > 0 ? x0 : hhi));
