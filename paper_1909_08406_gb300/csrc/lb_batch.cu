@@ -335,7 +335,7 @@ static cudaError_t launch_batch_step(lb_batch* b, int parity, cudaStream_t st) {
                 return cudaGetLastError();
             }
         }
-        const StepConsts<typename C::R>& one = step_consts<C, 1>(lc);
+        const StepConsts<typename C::R> one = step_consts<C, 1>(lc);
         if (b->project)
             k_batch_step<C, true, false><<<grid, block, 0, st>>>(P.d_sims, b->n, parity, one, P.tx,
                                                                  log2i(P.tx), P.ry, b->d_err);
@@ -352,7 +352,8 @@ static cudaError_t launch_persistent(lb_batch* b, int64_t nsteps, int parity, cu
         using C = decltype(codec);
         const void* kern = b->project ? (const void*)k_batch_persistent<C, true, false>
                                       : (const void*)k_batch_persistent<C, false, false>;
-        const void* K = &step_consts<C, 1>(lc);
+        const StepConsts<typename C::R> one = step_consts<C, 1>(lc);
+        const void* K = &one;
         if constexpr (std::is_same<typename C::R, float>::value) {
             if (b->pp.two_rows) {
                 kern = b->project ? (const void*)k_batch_persistent<C, true, true>

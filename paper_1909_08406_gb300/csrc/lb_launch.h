@@ -32,9 +32,9 @@ inline const Consts<typename Codec::R>& consts_of(const LaunchConsts& c) {
 }
 // Constants of the series step (EQ < 2) or of the entropic one.
 template <class Codec, int EQ>
-inline const StepK<typename Codec::R, EQ>& step_consts(const LaunchConsts& c) {
+inline StepK<typename Codec::R, EQ> step_consts(const LaunchConsts& c) {
     if constexpr (EQ >= 2)
-        return consts_of<Codec>(c);
+        return {step_consts<Codec, 0>(c), consts_of<Codec>(c)};
     else if constexpr (sizeof(typename Codec::R) == 8)
         return c.sd;
     else

@@ -11,8 +11,8 @@ cudaError_t launch_step_entropic(int prec, int eq, const void* src, void* dst, c
                                  double twobeta, int* err, cudaStream_t st) {
     auto run = [&](auto codec) {
         using C = decltype(codec);
-        return launch_entries<kNode>(eq == 3 ? k_step<C, 3, true> : k_step<C, 2, true>, src, dst, d, st, c.kf,
-                                     (float)twobeta, err, 0u);
+        return launch_entries<kNode>(eq == 3 ? k_step<C, 3, true> : k_step<C, 2, true>, src, dst, d, st,
+                                     step_consts<C, 2>(c), (float)twobeta, err, 0u);
     };
     switch (prec) {
         case kF32: return run(CodecF32{});
