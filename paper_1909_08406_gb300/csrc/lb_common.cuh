@@ -458,23 +458,25 @@ __device__ __forceinline__ NodeState<typename Codec::R> node_state(const StepCon
 // direction in two shells (sc-1 and sc-2, bcc-1 and bcc-1/2) share a and a^2: with a = k a_1 the factors
 // k and k^2 go into the shell constants.  The projection v = dj / (rho theta) is odd in u along each
 // axis: v_a = -up_a (K0 + K1 up_a^2).  About 300 operations a node, against 520 for the direct form.
-// RELAX false: sink receives tb h^eq_i (f^eq_i for FP64), no relaxation.
-template <class Codec, bool PROJECT, bool RELAX = true, class VGet, class Sink>
+// RELAX false: sink receives tb h^eq_i (f^eq_i for FP64), no relaxation.  ISO: theta = theta_0 (st.eta is
+// not read), where every cubic in eta is its constant term.
+template <class Codec, bool PROJECT, bool RELAX = true, bool ISO = false, class VGet, class Sink>
 __device__ __forceinline__ void collide(const NodeState<typename Codec::R>& st,
                                         const StepConsts<typename Codec::KS>& K, typename Codec::R tb,
                                         typename Codec::R omb, VGet&& vget, Sink&& sink) {
     using R = typename Codec::R;
     constexpr bool kF = Codec::stores_f;
-    const R eta = st.eta;
-    const R it1 = recip(R(1) + eta);           // theta_0 / theta
-    const R it = it1 * R(K.inv_theta0);        // 1 / theta
+    const R eta = ISO ? R(0) : st.eta;
+    const R it1 = ISO ? R(1) : recip(R(1) + eta);                            // theta_0 / theta
+    const R it = ISO ? R(K.inv_theta0) : it1 * R(K.inv_theta0);              // 1 / theta
     const R usq = fma(st.ux, st.ux, fma(st.uy, st.uy, st.uz * st.uz));
     const R g = usq * it;
     const R r2 = it1 * it1;
     auto cubic = [&](const typename Codec::KS(&c)[4]) {
+        if constexpr (ISO) return R(c[0]);
         return fma(eta, fma(eta, fma(eta, R(c[3]), R(c[2])), R(c[1])), R(c[0]));
     };
-    const R M2 = mul(cubic(K.m2), r2);
+    const R M2 = ISO ? cubic(K.m2) : mul(cubic(K.m2), r2);
     const R A1 = (R(2.5) * M2) * recip(fma(R(2.5), M2, R(1)));
     // A2 = 5 A1 (1 - M2) - (3 + M2' - 5 M2)
     const R A2 = fma(fma(R(-5), M2, R(5)), A1, fma(R(5), M2, fma(-cubic(K.m2p), r2, R(-3))));
@@ -501,6 +503,9 @@ __device__ __forceinline__ void collide(const NodeState<typename Codec::R>& st,
         if constexpr (kF) {
             P = tbr * cubic(K.rp[s]);
             B = P * fma(nga, R(K.c2[s]), one_cg);
+        } else if constexpr (ISO) {
+            P = tbr;
+            B = fma(P, fma(nga, R(K.c2[s]), cg), tbd);
         } else {
             const R rm1 = eta * fma(eta, fma(eta, R(K.rp[s][3]), R(K.rp[s][2])), R(K.rp[s][1]));
             const R tr = fma(tbr, rm1, tbd);  // tb (rho R_s - 1)

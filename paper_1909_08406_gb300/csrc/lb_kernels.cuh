@@ -58,7 +58,8 @@ inline EntryGrid entry_grid(const Dims& d) {
     return EntryGrid{2u * wx * wy * (uint32_t)d.nz, make_fastdiv(wx), make_fastdiv(wy)};
 }
 
-template <int KIND>
+// ZSY: rows in (z, s, y) order, so that the two sub-lattices of a plane are visited together.
+template <int KIND, bool ZSY = false>
 __device__ __forceinline__ bool entry_node(const Dims& d, const EntryGrid& g, int& s, int& z, int& y, int& x) {
     const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= g.entries) return false;
@@ -67,8 +68,13 @@ __device__ __forceinline__ bool entry_node(const Dims& d, const EntryGrid& g, in
     const uint32_t row = fdiv(p, g.fx), zs = fdiv(row, g.fy);
     x = (int)(p - row * wx) * (KIND == kPair ? 2 : 1);
     y = (int)(row - zs * wy) * (KIND == kRows ? 2 : 1);
-    s = zs >= (uint32_t)d.nz;
-    z = (int)zs - (s ? d.nz : 0);
+    if constexpr (ZSY) {
+        z = (int)(zs >> 1);
+        s = (int)(zs & 1u);
+    } else {
+        s = zs >= (uint32_t)d.nz;
+        z = (int)zs - (s ? d.nz : 0);
+    }
     return true;
 }
 
@@ -105,19 +111,10 @@ __device__ __forceinline__ void pdl_begin() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
-// Fused pull update (Sec. II) of one node (s, z, y, x): gather f*_i(x - c_i, t)
-// for all 41 velocities, compute the moments, the equilibrium and the BGK
-// relaxation, and write the 41 post-collision values.  Integer links stay on
-// the sub-lattice (shifts 0, +-1, +-2 cells); the bcc-1/2 links come from the
-// other sub-lattice: for A (s = 0) a component +1/2 reads cell r - 1 and -1/2
-// reads cell r; for B (s = 1) +1/2 reads cell r and -1/2 reads cell r + 1.
-// SR: BF16 storage with the stochastic store of lb_common.cuh, step key sr_key.
-template <class Codec, int EQ, class Ld = LoadNC, bool SR = false, bool WIDE = true>
-__device__ __forceinline__ void step_node(const typename Codec::raw_t* __restrict__ src,
-                                          typename Codec::raw_t* __restrict__ dst, const Dims& d,
-                                          const StepK<typename Codec::R, EQ>& K, typename Codec::R tb,
-                                          int* __restrict__ err, int s, int z, int y, int x, uint32_t sr_key = 0) {
-    using R = typename Codec::R;
+// The gather of one node: v[i] = f*_i(x - c_i, t) in the codec's working value.
+template <class Codec, class Ld, bool WIDE>
+__device__ __forceinline__ void pull_node(const typename Codec::raw_t* src, const Dims& d, int s, int z, int y, int x,
+                                          typename Codec::R (&v)[kQ]) {
     using T = typename Codec::raw_t;
     const uint32_t nx = (uint32_t)d.nx, nxy = nx * (uint32_t)d.ny, plane = (uint32_t)d.plane;
     const SubBases<T, WIDE> b(src, d, s);
@@ -136,7 +133,6 @@ __device__ __forceinline__ void step_node(const typename Codec::raw_t* __restric
     const uint32_t sub = b.o_oth - b.o_own;
     const uint32_t hzp = (s ? zo[2] : zo[3]) + sub, hzm = (s ? zo[1] : zo[2]) + sub;
 
-    R v[kQ];
     static_for<kQ>([&](auto I) {
         constexpr Vel c = vel(I);
         if constexpr (c.shell == 5) {
@@ -147,12 +143,31 @@ __device__ __forceinline__ void step_node(const typename Codec::raw_t* __restric
             v[I] = Codec::value(Ld::load(b.own + (size_t)I * plane + off));
         }
     });
+}
+
+// Fused pull update (Sec. II) of one node (s, z, y, x): gather f*_i(x - c_i, t)
+// for all 41 velocities, compute the moments, the equilibrium and the BGK
+// relaxation, and write the 41 post-collision values.  Integer links stay on
+// the sub-lattice (shifts 0, +-1, +-2 cells); the bcc-1/2 links come from the
+// other sub-lattice: for A (s = 0) a component +1/2 reads cell r - 1 and -1/2
+// reads cell r; for B (s = 1) +1/2 reads cell r and -1/2 reads cell r + 1.
+// SR: BF16 storage with the stochastic store of lb_common.cuh, step key sr_key.
+template <class Codec, int EQ, class Ld = LoadNC, bool SR = false, bool WIDE = true>
+__device__ __forceinline__ void step_node(const typename Codec::raw_t* __restrict__ src,
+                                          typename Codec::raw_t* __restrict__ dst, const Dims& d,
+                                          const StepK<typename Codec::R, EQ>& K, typename Codec::R tb,
+                                          int* __restrict__ err, int s, int z, int y, int x, uint32_t sr_key = 0) {
+    using R = typename Codec::R;
+    using T = typename Codec::raw_t;
+    const uint32_t nx = (uint32_t)d.nx, nxy = nx * (uint32_t)d.ny, plane = (uint32_t)d.plane;
+    R v[kQ];
+    pull_node<Codec, Ld, WIDE>(src, d, s, z, y, x, v);
 
     const NodeState<R> st = step_state<Codec, EQ>(K, v);
     bool ok = state_ok(st);
 
     const uint32_t qn = (uint32_t)z * nxy + (uint32_t)y * nx + (uint32_t)x;
-    T* out = dst_base<T, WIDE>(dst, d, s) + (b.o_own + qn);
+    T* out = dst_base<T, WIDE>(dst, d, s) + (SubBases<T, WIDE>(src, d, s).o_own + qn);
     if constexpr (SR) {
         const uint32_t q = (s ? plane : 0u) + qn;
         const uint32_t s0 = pcg_hash(sr_key ^ (q >> 1));
@@ -261,28 +276,14 @@ __global__ void __launch_bounds__(kStepThreads, MINB) k_step2(const typename Cod
     if (active) step_node2<Codec, PROJECT, LoadCA, WIDE>(src, dst, d, K, tb, err, s, z, y, x);
 }
 
-// Two x-adjacent nodes (s, z, y, x) and (s, z, y, x + 1), x even, per thread (16-bit storage, nx
-// even), packed FP32x2 arithmetic.  Each plane is read as aligned pairs of 16-bit values: one 32-bit
-// load when the plane's x shift is even, two loads and a byte permute when it is odd; the two
-// results of a plane are written with one 32-bit store.
-//
-// Bound by the latency of its dependent arithmetic at the warps that fit: 128 registers (4 blocks, 16
-// warps per SM, 24 bytes of spills); 33.5 GMLUPS on 256^3 with FP16 storage, 81% of the copy bandwidth
-// (a block per row chunk with the next row prefetched into L2: 32.2; 168 registers, 12 warps: 29.4).
-// SR: BF16 storage with the stochastic store of lb_common.cuh, step key sr_key (one word per
-// population and x pair).
-template <class Codec, bool PROJECT, bool WIDE, bool SR = false>
-__global__ void __launch_bounds__(kStepThreads, 4) k_step2x(const typename Codec::raw_t* __restrict__ src,
-                                                            typename Codec::raw_t* __restrict__ dst, Dims d,
-                                                            EntryGrid g, StepConsts<float2> K, float tb,
-                                                            int* __restrict__ err, uint32_t sr_key) {
+// The gather of the x pair (s, z, y, x), (s, z, y, x + 1), x even, nx even, 16-bit storage.  Each plane is
+// read as aligned pairs of 16-bit values: one 32-bit load when the plane's x shift is even, two loads
+// and a byte permute when it is odd.
+template <class Codec, bool WIDE>
+__device__ __forceinline__ void pull_pair(const typename Codec::raw_t* src, const Dims& d, int s, int z, int y, int x,
+                                          typename Codec::pair_t (&pv)[kQ]) {
     using T = typename Codec::raw_t;
     using P = typename Codec::pair_t;
-    using C2 = Codec2<Codec>;
-    int s, z, y, x;
-    const bool active = entry_node<kPair>(d, g, s, z, y, x);
-    pdl_begin();
-    if (!active) return;
     const uint32_t nx = (uint32_t)d.nx, nxy = nx * (uint32_t)d.ny, plane = (uint32_t)d.plane;
     const SubBases<T, WIDE> b(src, d, s);
     uint32_t yo[5], zo[5];
@@ -301,7 +302,6 @@ __global__ void __launch_bounds__(kStepThreads, 4) k_step2x(const typename Codec
     const uint32_t hlo = s ? x0 : xm, hhi = s ? xq : x0;
     const uint32_t sel_p = s ? 0x7654u : 0x5432u, sel_m = s ? 0x5432u : 0x3210u;
 
-    P pv[kQ];
     static_for<kQ>([&](auto I) {
         constexpr Vel c = vel(I);
         const T* base = (c.shell == 5 ? b.oth : b.own) + (size_t)I * plane;
@@ -328,19 +328,49 @@ __global__ void __launch_bounds__(kStepThreads, 4) k_step2x(const typename Codec
                 pv[I] = ld(row + xq);
         }
     });
-    auto vget = [&](auto I) { return F2(Codec::unpack2(pv[I])); };
-    const NodeState<F2> st = node_state<C2>(K, vget);
-    if (!state_ok(st)) atomicOr(err, 1);
-    // The values stay packed from here to their relaxation: without the barrier the compiler keeps
-    // the 82 widened numbers of the sums alive and spills more.
+}
+
+// The values stay packed from here to their use: without the barrier the compiler keeps the 82 widened
+// numbers of the moment sums alive and spills more.
+template <class Codec>
+__device__ __forceinline__ void keep_packed(typename Codec::pair_t (&pv)[kQ]) {
     static_for<kQ>([&](auto I) {
         uint32_t w;
         memcpy(&w, &pv[I], sizeof w);
         asm volatile("" : "+r"(w));
         memcpy(&pv[I], &w, sizeof w);
     });
-    const uint32_t qn = (uint32_t)z * nxy + (uint32_t)y * nx + x0;
-    T* out = dst_base<T, WIDE>(dst, d, s) + (b.o_own + qn);
+}
+
+// Two x-adjacent nodes (s, z, y, x) and (s, z, y, x + 1), x even, per thread (16-bit storage, nx
+// even), packed FP32x2 arithmetic; the two results of a plane are written with one 32-bit store.
+//
+// Bound by the latency of its dependent arithmetic at the warps that fit: 128 registers (4 blocks, 16
+// warps per SM, 24 bytes of spills); 33.5 GMLUPS on 256^3 with FP16 storage, 81% of the copy bandwidth
+// (a block per row chunk with the next row prefetched into L2: 32.2; 168 registers, 12 warps: 29.4).
+// SR: BF16 storage with the stochastic store of lb_common.cuh, step key sr_key (one word per
+// population and x pair).
+template <class Codec, bool PROJECT, bool WIDE, bool SR = false>
+__global__ void __launch_bounds__(kStepThreads, 4) k_step2x(const typename Codec::raw_t* __restrict__ src,
+                                                            typename Codec::raw_t* __restrict__ dst, Dims d,
+                                                            EntryGrid g, StepConsts<float2> K, float tb,
+                                                            int* __restrict__ err, uint32_t sr_key) {
+    using T = typename Codec::raw_t;
+    using P = typename Codec::pair_t;
+    using C2 = Codec2<Codec>;
+    int s, z, y, x;
+    const bool active = entry_node<kPair>(d, g, s, z, y, x);
+    pdl_begin();
+    if (!active) return;
+    P pv[kQ];
+    pull_pair<Codec, WIDE>(src, d, s, z, y, x, pv);
+    auto vget = [&](auto I) { return F2(Codec::unpack2(pv[I])); };
+    const NodeState<F2> st = node_state<C2>(K, vget);
+    if (!state_ok(st)) atomicOr(err, 1);
+    keep_packed<Codec>(pv);
+    const uint32_t plane = (uint32_t)d.plane;
+    const uint32_t qn = ((uint32_t)z * (uint32_t)d.ny + (uint32_t)y) * (uint32_t)d.nx + (uint32_t)x;
+    T* out = dst_base<T, WIDE>(dst, d, s) + (SubBases<T, WIDE>(src, d, s).o_own + qn);
     uint32_t s0 = 0;
     if constexpr (SR) s0 = pcg_hash(sr_key ^ (((s ? plane : 0u) + qn) >> 1));
     collide<C2, PROJECT>(st, K, F2(tb * (float)Codec::kScale), F2(1.f - tb), vget, [&](auto I, F2 val) {
@@ -362,18 +392,15 @@ inline bool few_entries(const Dims& d) {
     return d.plane < kSms * warps * 32;  // entries of two nodes: as many as cells
 }
 
-// Launches `kern` over the KIND entries of the grid with the programmatic attribute (pdl_begin).  Blocks of
+// Launches `kern`, one thread per entry, with the programmatic attribute (pdl_begin).  Blocks of
 // 128 threads, smaller ones where those would leave fewer than eight per SM, down to a warp, so that the
 // last wave is short.
-template <int KIND, class T, class... A>
-inline cudaError_t launch_entries(void (*kern)(const T*, T*, Dims, EntryGrid, A...), const void* src, void* dst,
-                                  const Dims& d, cudaStream_t st, const SameType<A>&... args) {
-    if (d.plane >= ((int64_t)1 << 30)) return cudaErrorInvalidValue;  // 32-bit entries (such a state exceeds the memory)
-    const EntryGrid g = entry_grid<KIND>(d);
+template <class... A>
+inline cudaError_t launch_linear(void (*kern)(A...), uint32_t entries, cudaStream_t st, const SameType<A>&... args) {
     constexpr uint32_t kEnough = (uint32_t)kSms * 8u;
-    const uint32_t th = g.entries >= kEnough * 128u ? 128u : g.entries >= kEnough * 64u ? 64u : 32u;
+    const uint32_t th = entries >= kEnough * 128u ? 128u : entries >= kEnough * 64u ? 64u : 32u;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((g.entries + th - 1) / th);
+    cfg.gridDim = dim3((entries + th - 1) / th);
     cfg.blockDim = dim3(th);
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
@@ -381,92 +408,15 @@ inline cudaError_t launch_entries(void (*kern)(const T*, T*, Dims, EntryGrid, A.
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, static_cast<const T*>(src), static_cast<T*>(dst), d, g, args...);
+    return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
-// Row addresses of the nonideal fluid's x-pair passes: the pair of upwind values of one population for
-// the nodes x, x + 1 of a row (s, z, y) that the whole block shares.
-template <class Codec>
-struct RowAddr2x {
-    using T = typename Codec::raw_t;
-    const T* same;   // population 0 of the node's own sub-lattice
-    const T* other;  // population 0 of the other sub-lattice
-    uint32_t yo[5], zo[5];
-    uint32_t hyp, hym, hzp, hzm;
-    int s;
-    __device__ __forceinline__ void set(const T* src, const Dims& d, int s_, int z, int y) {
-        s = s_;
-        const uint32_t nx = (uint32_t)d.nx, nxy = (uint32_t)d.nx * (uint32_t)d.ny;
-#pragma unroll
-        for (int k = 0; k < 5; ++k) {
-            yo[k] = (uint32_t)wrap(y - (k - 2), d.ny) * nx;
-            zo[k] = (uint32_t)wrap(z - (k - 2), d.nz) * nxy;
-        }
-        // half links: delta = 1 - s for a +1/2 component, -s for -1/2
-        hyp = s ? yo[2] : yo[3];
-        hym = s ? yo[1] : yo[2];
-        hzp = s ? zo[2] : zo[3];
-        hzm = s ? zo[1] : zo[2];
-        same = src + (size_t)s * kQ * d.plane;
-        other = src + (size_t)(1 - s) * kQ * d.plane;
-    }
-};
-
-// The pair of upwind values of population I for the nodes x, x + 1 of the row
-// described by `a` (source x - delta for a shift delta in {-2, ..., 2}).
-template <class Codec, int I>
-__device__ __forceinline__ typename Codec::pair_t load_pair2x(const RowAddr2x<Codec>& a, uint32_t plane,
-                                                              uint32_t xm, uint32_t x0, uint32_t xq) {
-    using T = typename Codec::raw_t;
-    using P = typename Codec::pair_t;
-    constexpr Vel c = vel(I);
-    auto ld = [&](const T* p, uint32_t off) { return LoadNC::load(reinterpret_cast<const P*>(p + off)); };
-    auto pair_at = [&](const T* p, int dx) -> P {
-        switch (dx) {
-            case 2: return ld(p, xm);
-            case 1: return Codec::straddle(ld(p, xm), ld(p, x0));
-            case 0: return ld(p, x0);
-            case -1: return Codec::straddle(ld(p, x0), ld(p, xq));
-            default: return ld(p, xq);
-        }
-    };
-    if constexpr (c.shell == 5) {
-        const T* p = a.other + (size_t)I * plane + ((c.z > 0 ? a.hzp : a.hzm) + (c.y > 0 ? a.hyp : a.hym));
-        if constexpr (c.x > 0)
-            return a.s ? pair_at(p, 0) : pair_at(p, 1);
-        else
-            return a.s ? pair_at(p, -1) : pair_at(p, 0);
-    } else {
-        const T* p = a.same + (size_t)I * plane + (a.zo[c.z / 2 + 2] + a.yo[c.y / 2 + 2]);
-        return pair_at(p, c.x / 2);
-    }
-}
-
-// Prefetch into L2 the part of population I's source row that the nodes
-// [xa, xb) of the row (s, z, y) will read (x - 2 .. x + 2, not wrapped),
-// trimmed inward to whole 16-byte units of that row.
-template <class Codec>
-__device__ __forceinline__ void prefetch_row_l2(const typename Codec::raw_t* src, const Dims& d, int I, int s, int z,
-                                                int y, int xa, int xb) {
-    using T = typename Codec::raw_t;
-    const Vel c = c_vel.v[I];
-    int sp, dz, dy;
-    if (c.shell == 5) {  // half link: delta = 1 - s for +1/2, -s for -1/2; other sub-lattice
-        sp = 1 - s;
-        dz = c.z > 0 ? 1 - s : -s;
-        dy = c.y > 0 ? 1 - s : -s;
-    } else {
-        sp = s;
-        dz = c.z / 2;
-        dy = c.y / 2;
-    }
-    const int zz = wrap(z - dz, d.nz), yy = wrap(y - dy, d.ny);
-    const int lo = max(xa - 2, 0), hi = min(xb + 2, d.nx);
-    const T* row = src + ((size_t)sp * kQ + I) * d.plane + ((size_t)zz * d.ny + yy) * d.nx;
-    const uintptr_t b0 = ((uintptr_t)(row + lo) + 15) & ~(uintptr_t)15;
-    const uintptr_t b1 = ((uintptr_t)(row + hi)) & ~(uintptr_t)15;
-    if (b1 > b0)
-        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(b0), "r"((uint32_t)(b1 - b0)) : "memory");
+template <int KIND, class T, class... A>
+inline cudaError_t launch_entries(void (*kern)(const T*, T*, Dims, EntryGrid, A...), const void* src, void* dst,
+                                  const Dims& d, cudaStream_t st, const SameType<A>&... args) {
+    if (d.plane >= ((int64_t)1 << 30)) return cudaErrorInvalidValue;  // 32-bit entries (such a state exceeds the memory)
+    const EntryGrid g = entry_grid<KIND>(d);
+    return launch_linear(kern, g.entries, st, static_cast<const T*>(src), static_cast<T*>(dst), d, g, args...);
 }
 
 // Populations = equilibrium of the given float64 fields, for nodes

@@ -98,22 +98,9 @@ __device__ __forceinline__ F quad_at(const NiQuad<F>& r, int v, int c) {
 __device__ __forceinline__ uint32_t wrap_up(int a, int n) { return (uint32_t)(a == n ? 0 : a); }
 __device__ __forceinline__ uint32_t wrap_dn(int a, int n) { return (uint32_t)(a < 0 ? n - 1 : a); }
 
-// Node of this thread: blocks cover (row, x chunk) pairs, rows running (z, s, y) with y fastest, so
-// that the two sub-lattices of a plane are visited together (the stencil passes read the other
-// sub-lattice's fields, which then come from L2).  The coordinates come from 32-bit divisions of
-// the block index (2 ny nz < 2^31, checked at init); q is the node's field index
-// ((s nz + z) ny + y) nx + x.
-__device__ __forceinline__ bool ni_node(const Dims& d, int chunks, int64_t& q, int& s, int& z, int& y, int& x) {
-    const uint32_t b = blockIdx.x;
-    const uint32_t row = b / (uint32_t)chunks;
-    x = (int)(b - row * (uint32_t)chunks) * kNiThreads + (int)threadIdx.x;
-    if (x >= d.nx) return false;
-    const uint32_t zs = row / (uint32_t)d.ny;
-    y = (int)(row - zs * (uint32_t)d.ny);
-    z = (int)(zs >> 1);
-    s = (int)(zs & 1u);
-    q = (((int64_t)s * d.nz + z) * d.ny + y) * d.nx + x;
-    return true;
+// Field index of node (s, z, y, x): ((s nz + z) ny + y) nx + x, below 2^32 (checked when the mode is enabled).
+__device__ __forceinline__ uint32_t ni_index(const Dims& d, int s, int z, int y, int x) {
+    return (((uint32_t)s * (uint32_t)d.nz + (uint32_t)z) * (uint32_t)d.ny + (uint32_t)y) * (uint32_t)d.nx + (uint32_t)x;
 }
 
 // Field indices of the 14 moving stencil neighbours of node (s, z, y, x), in the order of
@@ -137,53 +124,23 @@ __device__ __forceinline__ void ni_neighbors(const Dims& d, int s, int z, int y,
     for (int j = 0; j < 8; ++j) m[6 + j] = oth + Z[(j >> 2) & 1] + Y[(j >> 1) & 1] + X[j & 1];
 }
 
-// The pull gather of step_node: v[i] = f_i(x - c_i) in the codec's working value.
 template <class Codec>
-__device__ __forceinline__ void ni_gather(const typename Codec::raw_t* __restrict__ src, const Dims& d, int s, int z,
-                                          int y, int x, typename Codec::R (&v)[kQ]) {
-    using T = typename Codec::raw_t;
-    const int64_t nxy = (int64_t)d.nx * d.ny;
-    int xs[5];
-    int64_t yo[5], zo[5];
-#pragma unroll
-    for (int k = 0; k < 5; ++k) {
-        xs[k] = wrap(x - (k - 2), d.nx);
-        yo[k] = (int64_t)wrap(y - (k - 2), d.ny) * d.nx;
-        zo[k] = (int64_t)wrap(z - (k - 2), d.nz) * nxy;
-    }
-    const int hxp = s ? xs[2] : xs[3], hxm = s ? xs[1] : xs[2];
-    const int64_t hyp = s ? yo[2] : yo[3], hym = s ? yo[1] : yo[2];
-    const int64_t hzp = s ? zo[2] : zo[3], hzm = s ? zo[1] : zo[2];
-    const T* same = src + (int64_t)s * kQ * d.plane;
-    const T* other = src + (int64_t)(1 - s) * kQ * d.plane;
-    static_for<kQ>([&](auto I) {
-        constexpr Vel c = vel(I);
-        if constexpr (c.shell == 5) {
-            const int64_t off = (c.z > 0 ? hzp : hzm) + (c.y > 0 ? hyp : hym) + (c.x > 0 ? hxp : hxm);
-            v[I] = Codec::value(other[(int64_t)I * d.plane + off]);
-        } else {
-            const int64_t off = zo[c.z / 2 + 2] + yo[c.y / 2 + 2] + xs[c.x / 2 + 2];
-            v[I] = Codec::value(same[(int64_t)I * d.plane + off]);
-        }
-    });
-}
-
-template <class Codec>
-__global__ void __launch_bounds__(kNiThreads) k_ni_density(const typename Codec::raw_t* __restrict__ src, Dims d,
-                                                           int chunks, Consts<typename Codec::R> K, NiEosT<typename Codec::R> e,
+__global__ void __launch_bounds__(kNiThreads) k_ni_density(const typename Codec::raw_t* src, Dims d, EntryGrid g,
+                                                           Consts<typename Codec::R> K, NiEosT<typename Codec::R> e,
                                                            NiFields<typename Codec::R> fl) {
     using R = typename Codec::R;
-    int64_t q;
     int s, z, y, x;
-    if (!ni_node(d, chunks, q, s, z, y, x)) return;
+    const bool active = entry_node<kNode>(d, g, s, z, y, x);
+    pdl_begin();
+    if (!active) return;
     R v[kQ];
-    ni_gather<Codec>(src, d, s, z, y, x, v);
+    pull_node<Codec, LoadCA, true>(src, d, s, z, y, x, v);
     R dr = 0;  // rho - 1 = sum_i (f_i - w_i)
     static_for<kQ>([&](auto I) { dr += Codec::dev(v[I], K.w[vel(I).shell] * R(1.0 / Codec::kScale)); });
     const R r = R(1) + dr;
     R mu, Fe;
     ni_eos<R>(r, e, mu, Fe);
-    const uint32_t qq = (uint32_t)q;
+    const uint32_t qq = ni_index(d, s, z, y, x);
     fl.RF[ni_pair_at(qq, 0)] = r;
     fl.RF[ni_pair_at(qq, 1)] = Fe;
     fl.MU[qq] = mu;
@@ -228,11 +185,12 @@ __device__ __forceinline__ void ni_fields_node(F r0, F F0, const F (&rn)[kStenci
 }
 
 template <class F>
-__global__ void __launch_bounds__(kNiThreads) k_ni_fields(Dims d, int chunks, NiFields<F> fl) {
-    int64_t q64;
+__global__ void __launch_bounds__(kNiThreads) k_ni_fields(Dims d, EntryGrid gr, NiFields<F> fl) {
     int s, z, y, x;
-    if (!ni_node(d, chunks, q64, s, z, y, x)) return;
-    const uint32_t q = (uint32_t)q64;
+    const bool active = entry_node<kNode, true>(d, gr, s, z, y, x);
+    pdl_begin();
+    if (!active) return;
+    const uint32_t q = ni_index(d, s, z, y, x);
     uint32_t nb[kStencil];
     ni_neighbors(d, s, z, y, x, nb);
     F rn[kStencil], Fn[kStencil];
@@ -313,11 +271,12 @@ __device__ __forceinline__ void ni_force_finish(const NiEosT<F>& e, const NiForc
 // g^nid of every node into G (a pass of its own: folded into the step, the stencil sums raise the
 // step's register count and the fused step ran slower than the two passes).
 template <class F>
-__global__ void __launch_bounds__(kNiThreads) k_ni_force(Dims d, int chunks, NiEosT<F> e, NiFields<F> fl) {
-    int64_t q64;
+__global__ void __launch_bounds__(kNiThreads) k_ni_force(Dims d, EntryGrid gr, NiEosT<F> e, NiFields<F> fl) {
     int s, z, y, x;
-    if (!ni_node(d, chunks, q64, s, z, y, x)) return;
-    const uint32_t q = (uint32_t)q64;
+    const bool active = entry_node<kNode, true>(d, gr, s, z, y, x);
+    pdl_begin();
+    if (!active) return;
+    const uint32_t q = ni_index(d, s, z, y, x);
     uint32_t nb[kStencil];
     ni_neighbors(d, s, z, y, x, nb);
     NiForceSums<F> a;
@@ -336,21 +295,8 @@ __global__ void __launch_bounds__(kNiThreads) k_ni_force(Dims d, int chunks, NiE
     for (int b = 0; b < 3; ++b) fl.G[b * n + q] = g[b];
 }
 
-// Two x-adjacent nodes (x even, nx even) per thread in the stencil passes, rows in the (z, s, y)
-// order of ni_node; q is the even node's field index, q >> 1 the pair's.
-__device__ __forceinline__ bool ni_pair_zsy(const Dims& d, int chunks, uint32_t& q, int& s, int& z, int& y, int& x) {
-    const uint32_t b = blockIdx.x;
-    const uint32_t row = b / (uint32_t)chunks;
-    x = 2 * ((int)(b - row * (uint32_t)chunks) * (int)blockDim.x + (int)threadIdx.x);
-    if (x >= d.nx) return false;
-    const uint32_t zs = row / (uint32_t)d.ny;
-    y = (int)(row - zs * (uint32_t)d.ny);
-    z = (int)(zs >> 1);
-    s = (int)(zs & 1u);
-    q = (((uint32_t)s * (uint32_t)d.nz + (uint32_t)z) * (uint32_t)d.ny + (uint32_t)y) * (uint32_t)d.nx + (uint32_t)x;
-    return true;
-}
-
+// Two x-adjacent nodes (x even, nx even) per thread in the stencil passes; q is the even node's field
+// index, q >> 1 the pair's.
 // The stencil neighbours of the pair (x, x + 1) on sub-lattice S lie in 15 pairs (pair indices):
 //   0-2    the own row's pairs at x - 2, x, x + 2 (wrapped)
 //   3-6    the rows +y, -y, +z, -z at x
@@ -430,10 +376,12 @@ __device__ __forceinline__ void ni_fields_pair(const Dims& d, const NiFields<F>&
 
 // k_ni_fields for an x pair.
 template <class F>
-__global__ void __launch_bounds__(kNiThreads) k_ni_fields2x(Dims d, int chunks, NiFields<F> fl) {
-    uint32_t q;
+__global__ void __launch_bounds__(kNiThreads) k_ni_fields2x(Dims d, EntryGrid gr, NiFields<F> fl) {
     int s, z, y, x;
-    if (!ni_pair_zsy(d, chunks, q, s, z, y, x)) return;
+    const bool active = entry_node<kPair, true>(d, gr, s, z, y, x);
+    pdl_begin();
+    if (!active) return;
+    const uint32_t q = ni_index(d, s, z, y, x);
     if (s)
         ni_fields_pair<F, 1>(d, fl, z, y, x, q);
     else
@@ -485,149 +433,119 @@ __device__ __forceinline__ void ni_force_pair(const Dims& d, const NiEosT<F>& e,
 // k_ni_force for an x pair.  80 registers (6 blocks per SM), without spills: 2.86 against 2.92 ms
 // for the 256^3 step at 128 registers (4 blocks).
 template <class F>
-__global__ void __launch_bounds__(kNiThreads, 6) k_ni_force2x(Dims d, int chunks, NiEosT<F> e, NiFields<F> fl) {
-    uint32_t q;
+__global__ void __launch_bounds__(kNiThreads, 6) k_ni_force2x(Dims d, EntryGrid gr, NiEosT<F> e, NiFields<F> fl) {
     int s, z, y, x;
-    if (!ni_pair_zsy(d, chunks, q, s, z, y, x)) return;
+    const bool active = entry_node<kPair, true>(d, gr, s, z, y, x);
+    pdl_begin();
+    if (!active) return;
+    const uint32_t q = ni_index(d, s, z, y, x);
     if (s)
         ni_force_pair<F, 1>(d, e, fl, z, y, x, q);
     else
         ni_force_pair<F, 0>(d, e, fl, z, y, x, q);
 }
 
-// The pull step with the forced BGK collision; g^nid from G.
-template <class Codec>
-__global__ void __launch_bounds__(kNiThreads) k_ni_step(const typename Codec::raw_t* __restrict__ src,
-                                                        typename Codec::raw_t* __restrict__ dst, Dims d, int chunks,
-                                                        StepConsts<typename Codec::R> K, typename Codec::R tb,
-                                                        typename Codec::R inv_theta0,
-                                                        const typename Codec::R* __restrict__ G,
-                                                        int* __restrict__ err) {
+// The forced relaxation of a node as collide's sink: with G_i = (1 - beta) g.(c_i - u) / theta0 the new
+// value is (1 - 2 beta) v + f^eq_i (2 beta + G_i) for FP64, and for the deviation codecs, whose f^eq_i / w_i
+// is 1 + h^eq_i, (1 - 2 beta) v + h^eq_i (2 beta + G_i) + kScale G_i.  H = (1 - beta) g / theta0, hu = H.u; the
+// direction's H.c is formed for the +c of a pair and used for both.
+template <class Codec, class VGet, class Out>
+struct NiForcedSink {
     using R = typename Codec::R;
-    using T = typename Codec::raw_t;
-    int64_t q;
-    int s, z, y, x;
-    if (!ni_node(d, chunks, q, s, z, y, x)) return;
-    const int64_t n = 2 * d.plane;
-    const R gf[3] = {G[q], G[n + q], G[2 * n + q]};
-    R v[kQ];
-    ni_gather<Codec>(src, d, s, z, y, x, v);
-    const NodeSums<R> m = node_sums<Codec>(K, [&](auto I) { return v[I]; });
+    R hx, hy, hz, hu, tb, omb;
+    VGet vget;
+    Out out;
+    R hc;
+    template <class I>
+    __device__ __forceinline__ void operator()(I i, R veq) {
+        constexpr Vel c = vel(I::value);
+        R G;
+        if constexpr (c.shell == 0) {
+            G = -hu;
+        } else if constexpr (I::value % 2 == 1) {
+            hc = R(0);
+            bool first = true;
+            auto term = [&](auto C2, R h) {
+                constexpr int k = decltype(C2)::value;
+                if constexpr (k != 0) {
+                    hc = first ? R(0.5 * k) * h : fma(R(0.5 * k), h, hc);
+                    first = false;
+                }
+            };
+            term(std::integral_constant<int, c.x>{}, hx);
+            term(std::integral_constant<int, c.y>{}, hy);
+            term(std::integral_constant<int, c.z>{}, hz);
+            G = hc - hu;
+        } else {
+            G = -hc - hu;
+        }
+        const R v = vget(i);
+        if constexpr (Codec::stores_f)
+            out(i, fma(veq, tb + G, omb * v));
+        else
+            out(i, fma(veq, tb + G, fma(omb, v, R(Codec::kScale) * G)));
+    }
+};
+
+// State of the forced step: u = j / rho + g / 2 (the temperature is theta_0 throughout).
+template <class R>
+__device__ __forceinline__ NodeState<R> ni_state(const NodeSums<R>& m, R gx, R gy, R gz) {
     NodeState<R> st;
     st.drho = m.drho;
     st.rho = R(1) + m.drho;
-    const R gx = gf[0], gy = gf[1], gz = gf[2];
-    const R inv_rho = R(1) / st.rho;
-    st.ux = m.jx * inv_rho + R(0.5) * gx;
-    st.uy = m.jy * inv_rho + R(0.5) * gy;
-    st.uz = m.jz * inv_rho + R(0.5) * gz;
-    st.eta = R(0);  // isothermal: the equilibrium at theta_0
-    const bool ok = state_ok(st);
-    // f^eq in the working representation: f (FP64 codec) or scale * h^eq (deviation codecs)
-    R veq[kQ];
-    collide<Codec, true, false>(st, K, R(Codec::kScale), R(0), [](auto) { return R(0); },
-                                [&](auto I, R val) { veq[I] = val; });
-    T* out = dst + (int64_t)s * kQ * d.plane + ((int64_t)z * d.ny + y) * d.nx + x;
-    const R half_f = R(1) - R(0.5) * tb;  // 1 - beta
-    static_for<kQ>([&](auto I) {
-        constexpr Vel c = vel(I);
-        const R gc = gx * (R(0.5 * c.x) - st.ux) + gy * (R(0.5 * c.y) - st.uy) + gz * (R(0.5 * c.z) - st.uz);
-        R val;
-        if constexpr (Codec::stores_f) {
-            const R F = gc * inv_theta0 * veq[I];
-            val = v[I] + tb * (veq[I] - v[I]) + half_f * F;
-        } else {
-            // F_i / w_i = gc / theta0 (1 + h^eq), in units of the stored scale
-            const R F = gc * inv_theta0 * (R(Codec::kScale) + veq[I]);
-            val = v[I] + tb * (veq[I] - v[I]) + half_f * F;
-        }
-        out[(int64_t)I * d.plane] = Codec::to_raw(val);
-    });
-    if (!ok) atomicOr(err, 1);
+    const R inv_rho = recip(st.rho);
+    st.ux = fma(R(0.5), gx, m.jx * inv_rho);
+    st.uy = fma(R(0.5), gy, m.jy * inv_rho);
+    st.uz = fma(R(0.5), gz, m.jz * inv_rho);
+    st.eta = R(0);
+    return st;
 }
 
-// Two x-adjacent nodes per thread (16-bit storage, nx even): the x-pair gather of k_step2x and
-// packed FP32x2 arithmetic; x is the thread's even node.  ni_pair: one row per block, blocks over
-// (row, chunk of x pairs), rows (s, z, y); q the field index of the even node.
-__device__ __forceinline__ bool ni_pair(const Dims& d, int chunks, uint32_t& q, int& s, int& z, int& y, int& x) {
-    const uint32_t b = blockIdx.x;
-    const uint32_t row = b / (uint32_t)chunks;
-    x = 2 * ((int)(b - row * (uint32_t)chunks) * (int)blockDim.x + (int)threadIdx.x);
-    if (x >= d.nx) return false;
-    const uint32_t zr = row / (uint32_t)d.ny;
-    y = (int)(row - zr * (uint32_t)d.ny);
-    s = (int)(zr / (uint32_t)d.nz);
-    z = (int)(zr - (uint32_t)s * (uint32_t)d.nz);
-    q = row * (uint32_t)d.nx + (uint32_t)x;
-    return true;
+template <class Codec, class VGet, class KS, class Out>
+__device__ __forceinline__ void ni_collide(const NodeState<typename Codec::R>& st, const StepConsts<KS>& K,
+                                           typename Codec::R tb, typename Codec::R gx, typename Codec::R gy,
+                                           typename Codec::R gz, VGet vget, Out out) {
+    using R = typename Codec::R;
+    const R k = (R(1) - R(0.5) * tb) * R(K.inv_theta0);  // (1 - beta) / theta0
+    const R hx = gx * k, hy = gy * k, hz = gz * k;
+    NiForcedSink<Codec, VGet, Out> sink{hx, hy, hz, fma(hx, st.ux, fma(hy, st.uy, hz * st.uz)), tb, R(1) - tb,
+                                        vget, out, R(0)};
+    collide<Codec, true, false, true>(st, K, R(Codec::kScale), R(0), vget, sink);
 }
 
+// The pull step with the forced BGK collision; g^nid from G.
 template <class Codec>
-__device__ __forceinline__ void ni_gather2x(const typename Codec::raw_t* __restrict__ src, const Dims& d, int s, int z,
-                                            int y, int x, typename Codec::pair_t (&pv)[kQ]) {
-    const uint32_t xm = (uint32_t)wrap(x - 2, d.nx), x0 = (uint32_t)x, xq = (uint32_t)wrap(x + 2, d.nx);
-    RowAddr2x<Codec> a;
-    a.set(src, d, s, z, y);
-    static_for<kQ>([&](auto I) { pv[I] = load_pair2x<Codec, I>(a, (uint32_t)d.plane, xm, x0, xq); });
-}
-
-// The rows of a block of the x-pair forced step: `rpb` consecutive rows (s, z, y) for one chunk
-// of x pairs, as in the energy-conserving x-pair kernel's L2 mode.  At the start of a row, threads
-// 0..40 each prefetch into L2 the next row's source row of their population, and threads 41 ..
-// call extra(j = thread - 41, next row, xa, xb) for other spans to prefetch; body(q, s, z, y, x)
-// then does the thread's pair of the row (q its field index, x even).
-template <class Codec, class Extra, class Body>
-__device__ __forceinline__ void ni_row_walk(const typename Codec::raw_t* __restrict__ src, const Dims& d, int chunks,
-                                            int rpb, Extra extra, Body body) {
-    const uint32_t grp = blockIdx.x / (uint32_t)chunks;
-    const int chunk = (int)(blockIdx.x - grp * (uint32_t)chunks);
-    const int x = 2 * (chunk * (int)blockDim.x + (int)threadIdx.x);
-    const int xa = 2 * chunk * (int)blockDim.x, xb = min(xa + 2 * (int)blockDim.x, d.nx);
-    const uint32_t r0 = grp * (uint32_t)rpb, r1 = min(r0 + (uint32_t)rpb, (uint32_t)d.rows);
-    int y = (int)(r0 % (uint32_t)d.ny);
-    const uint32_t zr = r0 / (uint32_t)d.ny;
-    int z = (int)(zr % (uint32_t)d.nz), s = (int)(zr / (uint32_t)d.nz);
-    const bool active = x < d.nx;
-    for (uint32_t r = r0; r < r1; ++r) {
-        int yn = y + 1, zn = z, sn = s;
-        if (yn == d.ny) {
-            yn = 0;
-            if (++zn == d.nz) {
-                zn = 0;
-                ++sn;
-            }
-        }
-        if (r + 1 < r1) {
-            if (threadIdx.x < kQ)
-                prefetch_row_l2<Codec>(src, d, (int)threadIdx.x, sn, zn, yn, xa, xb);
-            else
-                extra((int)threadIdx.x - kQ, r + 1, xa, xb);
-        }
-        if (active) body(r * (uint32_t)d.nx + (uint32_t)x, s, z, y, x);
-        s = sn;
-        z = zn;
-        y = yn;
-    }
-}
-
-// L2 prefetch of the whole 16-byte units inside [p0, p1).
-__device__ __forceinline__ void prefetch_span_l2(const void* p0, const void* p1) {
-    const uintptr_t b0 = ((uintptr_t)p0 + 15) & ~(uintptr_t)15, b1 = (uintptr_t)p1 & ~(uintptr_t)15;
-    if (b1 > b0)
-        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(b0), "r"((uint32_t)(b1 - b0)) : "memory");
-}
-
-// k_ni_density for an x pair (one row per block: the L2 prefetch of the next row, which helps the
-// step, measured slower here, 0.617 against 0.538 ms at 256^3).
-template <class Codec>
-__global__ void __launch_bounds__(kStepThreads) k_ni_density2x(const typename Codec::raw_t* __restrict__ src, Dims d,
-                                                               int chunks, Consts<float> K, NiEosT<float> e,
-                                                               NiFields<float> fl) {
-    uint32_t q;
+__global__ void __launch_bounds__(kNiThreads) k_ni_step(const typename Codec::raw_t* src, typename Codec::raw_t* dst,
+                                                        Dims d, EntryGrid g, StepConsts<typename Codec::R> K,
+                                                        typename Codec::R tb, const typename Codec::R* G, int* err) {
+    using R = typename Codec::R;
     int s, z, y, x;
-    if (!ni_pair(d, chunks, q, s, z, y, x)) return;
+    const bool active = entry_node<kNode>(d, g, s, z, y, x);
+    pdl_begin();
+    if (!active) return;
+    const uint32_t q = ni_index(d, s, z, y, x);
+    const size_t n = 2 * (size_t)d.plane;
+    const R gx = LoadCA::load(G + q), gy = LoadCA::load(G + n + q), gz = LoadCA::load(G + 2 * n + q);
+    R v[kQ];
+    pull_node<Codec, LoadCA, true>(src, d, s, z, y, x, v);
+    auto vget = [&](auto I) { return v[I]; };
+    const NodeState<R> st = ni_state(node_sums<Codec>(K, vget), gx, gy, gz);
+    if (!state_ok(st)) atomicOr(err, 1);
+    typename Codec::raw_t* o = dst + (size_t)s * (kQ - 1) * d.plane + q;
+    ni_collide<Codec>(st, K, tb, gx, gy, gz, vget, [&](auto I, R val) { o[(size_t)I * d.plane] = Codec::to_raw(val); });
+}
+
+// k_ni_density for an x pair (16-bit storage, nx even).
+template <class Codec, bool WIDE>
+__global__ void __launch_bounds__(kStepThreads) k_ni_density2x(const typename Codec::raw_t* src, Dims d, EntryGrid g,
+                                                               Consts<float> K, NiEosT<float> e, NiFields<float> fl) {
+    int s, z, y, x;
+    const bool active = entry_node<kPair>(d, g, s, z, y, x);
+    pdl_begin();
+    if (!active) return;
+    const uint32_t q = ni_index(d, s, z, y, x);
     typename Codec::pair_t pv[kQ];
-    ni_gather2x<Codec>(src, d, s, z, y, x, pv);
+    pull_pair<Codec, WIDE>(src, d, s, z, y, x, pv);
     constexpr float inv_scale = (float)(1.0 / Codec::kScale);
     F2 dr(0.f);  // rho - 1 = sum_i (f_i - w_i), in the population order of k_ni_density
     static_for<kQ>([&](auto I) { dr += F2(Codec::unpack2(pv[I])) * F2(K.w[vel(I).shell] * inv_scale); });
@@ -635,60 +553,35 @@ __global__ void __launch_bounds__(kStepThreads) k_ni_density2x(const typename Co
     float mu0, F0, mu1, F1;
     ni_eos<float>(r.v.x, e, mu0, F0);
     ni_eos<float>(r.v.y, e, mu1, F1);
-    *reinterpret_cast<float4*>(fl.RF + 2 * q) = make_float4(r.v.x, r.v.y, F0, F1);
+    *reinterpret_cast<float4*>(fl.RF + 2 * (size_t)q) = make_float4(r.v.x, r.v.y, F0, F1);
     *reinterpret_cast<float2*>(fl.MU + q) = make_float2(mu0, mu1);
 }
 
-// k_ni_step for an x pair: the forcing is applied as each population's equilibrium is formed.
-template <class Codec>
-__global__ void __launch_bounds__(kStepThreads, 3) k_ni_step2x(const typename Codec::raw_t* __restrict__ src,
-                                                               typename Codec::raw_t* __restrict__ dst, Dims d,
-                                                               int chunks, int rpb, StepConsts<float2> K, float tb,
-                                                               float inv_theta0, const float* __restrict__ G,
-                                                               int* __restrict__ err) {
+// k_ni_step for an x pair (16-bit storage, nx even).  Bound by the latency of its arithmetic: 4 blocks per SM
+// (128 registers, 76 bytes of spills) take the 160 x 200 x 200 step from 1.04 to 0.99 ms against 3.
+template <class Codec, bool WIDE>
+__global__ void __launch_bounds__(kStepThreads, 4) k_ni_step2x(const typename Codec::raw_t* src,
+                                                               typename Codec::raw_t* dst, Dims d, EntryGrid g,
+                                                               StepConsts<float2> K, float tb, const float* G, int* err) {
     using P = typename Codec::pair_t;
     using C2 = Codec2<Codec>;
+    int s, z, y, x;
+    const bool active = entry_node<kPair>(d, g, s, z, y, x);
+    pdl_begin();
+    if (!active) return;
+    const uint32_t q = ni_index(d, s, z, y, x);
     const size_t n = 2 * (size_t)d.plane;
-    // threads 41..43 prefetch the next row's span of g_x, g_y, g_z
-    auto g_rows = [&](int j, uint32_t row, int xa, int xb) {
-        if (j < 3) {
-            const float* g = G + (size_t)j * n + (size_t)row * (uint32_t)d.nx;
-            prefetch_span_l2(g + xa, g + xb);
-        }
-    };
-    ni_row_walk<Codec>(src, d, chunks, rpb, g_rows, [&](uint32_t q, int s, int z, int y, int x) {
     P pv[kQ];
-    ni_gather2x<Codec>(src, d, s, z, y, x, pv);
+    pull_pair<Codec, WIDE>(src, d, s, z, y, x, pv);
     auto vget = [&](auto I) { return F2(Codec::unpack2(pv[I])); };
-    const F2 gx(*reinterpret_cast<const float2*>(G + q)), gy(*reinterpret_cast<const float2*>(G + n + q)),
-        gz(*reinterpret_cast<const float2*>(G + 2 * n + q));
-    const NodeSums<F2> m = node_sums<C2>(K, vget);
-    NodeState<F2> st;
-    st.drho = m.drho;
-    st.rho = F2(1.f) + m.drho;
-    const F2 inv_rho = recip(st.rho);
-    st.ux = fma(F2(0.5f), gx, m.jx * inv_rho);
-    st.uy = fma(F2(0.5f), gy, m.jy * inv_rho);
-    st.uz = fma(F2(0.5f), gz, m.jz * inv_rho);
-    st.eta = F2(0.f);  // isothermal: the equilibrium at theta_0
+    auto ld = [&](size_t off) { return F2(LoadCA::load(reinterpret_cast<const float2*>(G + off + q))); };
+    const F2 gx = ld(0), gy = ld(n), gz = ld(2 * n);
+    const NodeState<F2> st = ni_state(node_sums<C2>(K, vget), gx, gy, gz);
     if (!state_ok(st)) atomicOr(err, 1);
-    // F_i / w_i = g.(c_i - u) / theta0 (1 + h^eq_i), in units of the stored scale
-    const F2 it(inv_theta0);
-    const F2 hx = gx * it, hy = gy * it, hz = gz * it;
-    const F2 hu = hx * st.ux + hy * st.uy + hz * st.uz;
-    const F2 tbv(tb), half_f(1.f - 0.5f * tb), scale((float)Codec::kScale);
-    P* outp = reinterpret_cast<P*>(dst + (size_t)s * kQ * d.plane + (q - (uint32_t)s * (uint32_t)d.plane));
-    const size_t pstride = (size_t)d.plane / 2;
-    collide<C2, true, false>(st, K, scale, F2(0.f), vget, [&](auto I, F2 veq) {
-        constexpr Vel c = vel(I);
-        F2 gc = F2(0.f) - hu;
-        if constexpr (c.x != 0) gc = fma(F2(0.5f * c.x), hx, gc);
-        if constexpr (c.y != 0) gc = fma(F2(0.5f * c.y), hy, gc);
-        if constexpr (c.z != 0) gc = fma(F2(0.5f * c.z), hz, gc);
-        const F2 v = vget(I);
-        const F2 val = fma(half_f, gc * (scale + veq), fma(tbv, veq - v, v));
-        outp[(size_t)I * pstride] = Codec::to_raw2(val.v);
-    });
+    keep_packed<Codec>(pv);
+    typename Codec::raw_t* o = dst + (size_t)s * (kQ - 1) * d.plane + q;
+    ni_collide<C2>(st, K, F2(tb), gx, gy, gz, vget, [&](auto I, F2 val) {
+        *reinterpret_cast<P*>(o + (size_t)I * d.plane) = Codec::to_raw2(val.v);
     });
 }
 
@@ -713,8 +606,7 @@ cudaError_t launch_nonideal_step(int prec, const void* src, void* dst, const Dim
                                  double twobeta, int kind, const double eos[4], double* work, int* err,
                                  cudaStream_t st) {
     const int64_t n = 2 * d.plane;
-    const int chunks = (d.nx + kNiThreads - 1) / kNiThreads;
-    const unsigned blocks = (unsigned)(d.rows * chunks);
+    if (d.plane >= ((int64_t)1 << 30)) return cudaErrorInvalidValue;  // 32-bit entries
     if (kind < kVdW || kind > kCarnahanStarling) return cudaErrorInvalidValue;
     const NiEos e64{eos[0], eos[1], c.theta0, eos[2], eos[3], kind};
     return ni_codec(prec, [&](auto codec) {
@@ -734,42 +626,41 @@ cudaError_t launch_nonideal_step(int prec, const void* src, void* dst, const Dim
         fl.G = fl.D + n;
         const auto* in = static_cast<const typename C::raw_t*>(src);
         auto* out = static_cast<typename C::raw_t*>(dst);
-        // 16-bit storage with nx even: the gathering passes on x pairs
+        // x pairs with nx even: the gathering passes with 16-bit storage, the stencil passes with FP32 fields
+        const bool even = d.nx % 2 == 0, wide = wide_offsets(d);
+        const EntryGrid gn = entry_grid<kNode>(d), gp = entry_grid<kPair>(d);
         constexpr bool kPairs = sizeof(typename C::raw_t) == 2;
-        const bool pairs = kPairs && d.nx % 2 == 0;
-        const int half = d.nx / 2;
-        const int th2 = half >= 128 ? 128 : ((half + 31) / 32) * 32;
-        const int chunks2 = (half + th2 - 1) / th2;
-        constexpr int kRpb = 2;  // rows per block of the forced step (the next one prefetched)
-        const unsigned blocks2 = (unsigned)(((d.rows + kRpb - 1) / kRpb) * chunks2);
+        cudaError_t err_ = cudaSuccess;
+        auto ok = [&](cudaError_t e_) { return (err_ = e_) == cudaSuccess; };
+        bool gathered = false;
         if constexpr (kPairs) {
-            if (pairs) k_ni_density2x<C><<<(unsigned)(d.rows * chunks2), th2, 0, st>>>(in, d, chunks2, *K, e, fl);
-        }
-        if (!pairs) k_ni_density<C><<<blocks, kNiThreads, 0, st>>>(in, d, chunks, *K, e, fl);
-        // FP32 fields with nx even: the stencil passes on x pairs, in 128-thread blocks
-        bool pair_fields = false;
-        if constexpr (sizeof(R) == 4) {
-            if (d.nx % 2 == 0) {
-                const int chunks_f = (half + kNiThreads - 1) / kNiThreads;
-                const unsigned blocks_f = (unsigned)(d.rows * chunks_f);
-                k_ni_fields2x<R><<<blocks_f, kNiThreads, 0, st>>>(d, chunks_f, fl);
-                k_ni_force2x<R><<<blocks_f, kNiThreads, 0, st>>>(d, chunks_f, e, fl);
-                pair_fields = true;
+            if (even) {
+                if (!ok(launch_linear(wide ? k_ni_density2x<C, true> : k_ni_density2x<C, false>, gp.entries, st, in, d, gp,
+                                      *K, e, fl)))
+                    return err_;
+                gathered = true;
             }
         }
-        if (!pair_fields) {
-            k_ni_fields<R><<<blocks, kNiThreads, 0, st>>>(d, chunks, fl);
-            k_ni_force<R><<<blocks, kNiThreads, 0, st>>>(d, chunks, e, fl);
+        if (!gathered && !ok(launch_linear(k_ni_density<C>, gn.entries, st, in, d, gn, *K, e, fl))) return err_;
+        bool fields = false;
+        if constexpr (sizeof(R) == 4) {
+            if (even) {
+                if (!ok(launch_linear(k_ni_fields2x<R>, gp.entries, st, d, gp, fl)) ||
+                    !ok(launch_linear(k_ni_force2x<R>, gp.entries, st, d, gp, e, fl)))
+                    return err_;
+                fields = true;
+            }
         }
+        if (!fields && (!ok(launch_linear(k_ni_fields<R>, gn.entries, st, d, gn, fl)) ||
+                        !ok(launch_linear(k_ni_force<R>, gn.entries, st, d, gn, e, fl))))
+            return err_;
         if constexpr (kPairs) {
-            if (pairs)
-                k_ni_step2x<C><<<blocks2, th2, 0, st>>>(in, out, d, chunks2, kRpb, pair_consts<C>(c), (float)twobeta,
-                                                         (float)(1.0 / c.theta0), fl.G, err);
+            if (even)
+                return launch_linear(wide ? k_ni_step2x<C, true> : k_ni_step2x<C, false>, gp.entries, st, in, out, d, gp,
+                                     pair_consts<C>(c), (float)twobeta, (const float*)fl.G, err);
         }
-        if (!pairs)
-            k_ni_step<C><<<blocks, kNiThreads, 0, st>>>(in, out, d, chunks, (step_consts<C, 1>(c)), (R)twobeta, (R)(1.0 / c.theta0), fl.G,
-                                                         err);
-        return cudaGetLastError();
+        return launch_linear(k_ni_step<C>, gn.entries, st, in, out, d, gn, (step_consts<C, 1>(c)), (R)twobeta,
+                             (const R*)fl.G, err);
     });
 }
 
