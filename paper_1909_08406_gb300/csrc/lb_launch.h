@@ -138,8 +138,4 @@ cudaError_t launch_nonideal_step(int prec, const void* src, void* dst, const Dim
                                  double twobeta, int kind, const double eos[4], double* work, int* err,
                                  cudaStream_t st);
 
-inline int step_threads(const Dims& d) {
-    return d.nx >= 128 ? 128 : ((d.nx + 31) / 32) * 32;
-}
-
 }  // namespace gblb
