@@ -71,6 +71,12 @@ int sg_set_conv_impl(int impl);
  * cleared), or -3 for a CUDA error. */
 int sg_status(void *stream);
 
+/* sg_conv3d_fwd on x in the df-layout of a volume (sg_relabel; s its shape, s.xper = 64 / df), with y
+ * and add in the volume's dt-layout (df, dt in {1, 2, 4, 8}); z_out stays in x's layout.  The relabelling
+ * is in the epilogue's addresses.  -1 also for extents that are not multiples of the spacing. */
+int sg_conv3d_fwd_to(sg_shape s, int cin, int cout, const void *x, const void *w, const float *bias, int act,
+                     int res_in, const void *add, float *z_out, void *y, int df, int dt, void *stream);
+
 /* Input-gradient form of the convolution: y = conv(x, w) + add, with y and
  * add (may be NULL) FP32 [voxels][cout]. */
 int sg_conv3d_fwd_f32(sg_shape s, int cin, int cout, const void *x, const void *w, const float *add, float *y,

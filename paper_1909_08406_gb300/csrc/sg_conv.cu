@@ -56,7 +56,19 @@ struct Epi {
     int add_f32;
     float* z_out;
     int y_f32;
+    // y and add in another d-layout (2^lt) than x and z_out (2^lf); nzt, nyt its volume
+    int lf = 0, lt = 0, nzt = 0, nyt = 0;
 };
+
+// Voxel index in the 2^lt-layout of the voxel (b, z, y, x) of the 2^lf-layout (k_relabel has the formula).
+__device__ __forceinline__ int64_t relabelled_voxel(const Epi& e, int b, int z, int y, int x) {
+    const int mf = (1 << e.lf) - 1, mt = (1 << e.lt) - 1;
+    const int xn = ((x & ((kW >> e.lf) - 1)) << e.lf) | (x >> (6 - e.lf));
+    const int yn = (y << e.lf) | (b & mf), zn = (z << e.lf) | ((b >> e.lf) & mf);
+    const int bt = ((((b >> (2 * e.lf)) << e.lt) | (zn & mt)) << e.lt) | (yn & mt);
+    const int xt = ((xn & mt) << (6 - e.lt)) | (xn >> e.lt);
+    return (((int64_t)bt * e.nzt + (zn >> e.lt)) * e.nyt + (yn >> e.lt)) * kW + xt;
+}
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -174,6 +186,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_conv_fwd(sg_shape s, const b
         for (int h = 0; h < 2; ++h) {
             const int xx = x0 + g + 8 * h;
             const int64_t v = (((int64_t)b * s.nz + z) * s.ny + (y0 + yl)) * kW + xx;
+            const int64_t vo = epi.lf == epi.lt ? v : relabelled_voxel(epi, b, z, y0 + yl, xx);
             float z0 = acc[nt][2 * h] + b0, z1 = acc[nt][2 * h + 1] + b1;
             if (epi.z_out) *reinterpret_cast<float2*>(epi.z_out + v * COUT + co) = make_float2(z0, z1);
             float o0 = epi.act == SG_ACT_GELU ? gelu(z0) : z0;
@@ -186,20 +199,20 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_conv_fwd(sg_shape s, const b
             }
             if (epi.add) {
                 if (epi.add_f32) {
-                    const float2 r = *reinterpret_cast<const float2*>(static_cast<const float*>(epi.add) + v * COUT + co);
+                    const float2 r = *reinterpret_cast<const float2*>(static_cast<const float*>(epi.add) + vo * COUT + co);
                     o0 += r.x;
                     o1 += r.y;
                 } else {
                     const __nv_bfloat162 r =
-                        *reinterpret_cast<const __nv_bfloat162*>(static_cast<const bf16*>(epi.add) + v * COUT + co);
+                        *reinterpret_cast<const __nv_bfloat162*>(static_cast<const bf16*>(epi.add) + vo * COUT + co);
                     o0 += __bfloat162float(r.x);
                     o1 += __bfloat162float(r.y);
                 }
             }
             if (epi.y_f32)
-                *reinterpret_cast<float2*>(static_cast<float*>(y) + v * COUT + co) = make_float2(o0, o1);
+                *reinterpret_cast<float2*>(static_cast<float*>(y) + vo * COUT + co) = make_float2(o0, o1);
             else
-                *reinterpret_cast<__nv_bfloat162*>(static_cast<bf16*>(y) + v * COUT + co) = __floats2bfloat162_rn(o0, o1);
+                *reinterpret_cast<__nv_bfloat162*>(static_cast<bf16*>(y) + vo * COUT + co) = __floats2bfloat162_rn(o0, o1);
         }
     }
 }
@@ -293,14 +306,42 @@ __global__ void __launch_bounds__(kWgThreads) k_conv_wgrad(sg_shape s, const bf1
     }
 }
 
+constexpr int kBiasBlocks = 512;  // blocks of the bias-gradient partial sums
+
+// db[co] = sum over blocks of the partials, one warp per channel, fixed order: lane l adds the
+// partials l, l + 32, ... (all loads issued before the additions), then a shuffle tree.
+__device__ __forceinline__ void bias_finish(int co, int lane, int blocks, int cout, const float* __restrict__ partial,
+                                            float* __restrict__ db) {
+    constexpr int kMaxPer = kBiasBlocks / 32;
+    float v[kMaxPer];
+#pragma unroll
+    for (int j = 0; j < kMaxPer; ++j) {
+        const int b = lane + 32 * j;
+        v[j] = b < blocks ? partial[(int64_t)b * cout + co] : 0.f;
+    }
+    float sum = 0.f;
+#pragma unroll
+    for (int j = 0; j < kMaxPer; ++j) sum += v[j];
+#pragma unroll
+    for (int w = 16; w > 0; w >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, w);
+    if (lane == 0) db[co] = sum;
+}
+
 // dw[co][tap][ci] = sum_p partials[p][tap][co][ci] (deterministic).  A block takes 32 consecutive
 // partial entries (one per lane, coalesced); warp w adds the parts of the w-th of 8 equal ranges
-// in order, then the 8 range sums are added in the order w = 0 .. 7.
+// in order, then the 8 range sums are added in the order w = 0 .. 7.  The blocks after those of
+// the weights finish the bias gradient, one warp per channel.
 __global__ void __launch_bounds__(256) k_wgrad_reduce(int cin, int cout, int parts, const float* __restrict__ partials,
-                                                      float* __restrict__ dw) {
+                                                      float* __restrict__ dw, int bias_parts,
+                                                      const float* __restrict__ bias_part, float* __restrict__ db) {
     __shared__ float sh[8][32];
-    const int n = 27 * cin * cout;
+    const int n = 27 * cin * cout, weight_blocks = (n + 31) / 32;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    if ((int)blockIdx.x >= weight_blocks) {
+        const int co = ((int)blockIdx.x - weight_blocks) * 8 + w;
+        if (co < cout) bias_finish(co, lane, bias_parts, cout, bias_part, db);
+        return;
+    }
     const int off = (int)blockIdx.x * 32 + lane;  // tap * cout * cin + co * cin + ci
     float sum = 0.f;
     if (off < n) {
@@ -319,8 +360,6 @@ __global__ void __launch_bounds__(256) k_wgrad_reduce(int cin, int cout, int par
         dw[((int64_t)co * 27 + tap) * cin + ci] = t;
     }
 }
-
-constexpr int kBiasBlocks = 512;  // blocks of the bias-gradient partial sums
 
 // Partial sums of db[co] = sum_v dz[v][co] over a contiguous range of voxels per block: thread t
 // reads 16-byte chunks t, t + 256, ... of the range (8 channels each; with cout / 8 chunks per
@@ -356,32 +395,27 @@ __global__ void __launch_bounds__(256) k_bias_partials(int64_t voxels, int cout,
         for (int k = 0; k < 8; ++k) partial[(int64_t)blockIdx.x * cout + 8 * threadIdx.x + k] = sh[threadIdx.x][k];
 }
 
-// db[co] = sum over blocks of the partials, one warp per channel, fixed order: lane l adds the
-// partials l, l + 32, ... (all loads issued before the additions), then a shuffle tree.
-__global__ void k_bias_finish(int blocks, int cout, const float* __restrict__ partial, float* __restrict__ db) {
-    const int co = (int)(threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (co >= cout) return;
-    constexpr int kMaxPer = kBiasBlocks / 32;
-    float v[kMaxPer];
-#pragma unroll
-    for (int j = 0; j < kMaxPer; ++j) {
-        const int b = lane + 32 * j;
-        v[j] = b < blocks ? partial[(int64_t)b * cout + co] : 0.f;
-    }
-    float sum = 0.f;
-#pragma unroll
-    for (int j = 0; j < kMaxPer; ++j) sum += v[j];
-#pragma unroll
-    for (int w = 16; w > 0; w >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, w);
-    if (lane == 0) db[co] = sum;
-}
-
-__global__ void k_act_bwd(int64_t n, int act, const float* __restrict__ dy, const float* __restrict__ z,
-                          bf16* __restrict__ dz) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// V elements per thread: four with aligned pointers (16-byte loads, one 8-byte store), else one.  The
+// 33.5 M gradients of a 32-channel layer at batch 4: 60 us (HBM floor 50), one by one 108.
+template <int V>
+__global__ void __launch_bounds__(256) k_act_bwd(int64_t n, int act, const float* __restrict__ dy,
+                                                 const float* __restrict__ z, bf16* __restrict__ dz) {
+    const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * V;
     if (i >= n) return;
-    const float g = act == SG_ACT_GELU ? dy[i] * gelu_grad(z[i]) : dy[i];
-    dz[i] = __float2bfloat16_rn(g);
+    if (V == 1 || i + V > n) {
+        for (int64_t j = i; j < n && j < i + V; ++j)
+            dz[j] = __float2bfloat16_rn(act == SG_ACT_GELU ? dy[j] * gelu_grad(z[j]) : dy[j]);
+        return;
+    }
+    float g[4];
+    const float4 d4 = __ldg(reinterpret_cast<const float4*>(dy + i));
+    g[0] = d4.x, g[1] = d4.y, g[2] = d4.z, g[3] = d4.w;
+    if (act == SG_ACT_GELU) {
+        const float4 z4 = __ldg(reinterpret_cast<const float4*>(z + i));
+        g[0] *= gelu_grad(z4.x), g[1] *= gelu_grad(z4.y), g[2] *= gelu_grad(z4.z), g[3] *= gelu_grad(z4.w);
+    }
+    __nv_bfloat162 o[2] = {__floats2bfloat162_rn(g[0], g[1]), __floats2bfloat162_rn(g[2], g[3])};
+    *reinterpret_cast<uint2*>(dz + i) = *reinterpret_cast<const uint2*>(o);
 }
 
 __global__ void k_transpose_w(int cin, int cout, const bf16* __restrict__ w, bf16* __restrict__ wt) {
@@ -753,8 +787,7 @@ __device__ __forceinline__ void tc_ld3(uint32_t ta, uint32_t tb, uint32_t tc, fl
     for (int j = 0; j < 8; ++j) fa[j] = __uint_as_float(a[j]), fb[j] = __uint_as_float(b[j]), fc[j] = __uint_as_float(c[j]);
 }
 
-// NW 32-bit words from p (16-byte aligned), and their addition to EC values: FP32 words (NW = EC)
-// or pairs of bf16 (NW = EC / 2).
+// EC bf16 values from p (16-byte aligned) as words, and their addition to EC FP32 values.
 template <int NW>
 __device__ __forceinline__ void ld_words(const uint4* p, uint32_t (&dst)[NW]) {
 #pragma unroll
@@ -763,22 +796,45 @@ __device__ __forceinline__ void ld_words(const uint4* p, uint32_t (&dst)[NW]) {
         dst[4 * h] = raw.x, dst[4 * h + 1] = raw.y, dst[4 * h + 2] = raw.z, dst[4 * h + 3] = raw.w;
     }
 }
-template <int EC, int NW>
-__device__ __forceinline__ void add_words(float (&o)[EC], const uint32_t (&src)[NW]) {
-    if constexpr (NW == EC) {
+template <int EC>
+__device__ __forceinline__ void add_words(float (&o)[EC], const uint32_t (&src)[EC / 2]) {
 #pragma unroll
-        for (int e = 0; e < EC; ++e) o[e] += __uint_as_float(src[e]);
-    } else {
+    for (int e = 0; e < EC / 2; ++e) {
+        const __nv_bfloat162 h2 = *reinterpret_cast<const __nv_bfloat162*>(&src[e]);
+        o[2 * e] += __bfloat162float(h2.x);
+        o[2 * e + 1] += __bfloat162float(h2.y);
+    }
+}
+
+// Transposes blocks of four values among groups of NB lanes: afterwards block j of a lane is what lane
+// (lane & ~(NB - 1)) + j had as its block lane & (NB - 1), so that the NB lanes of a group hold one
+// voxel's 16 NB contiguous bytes per block.
+template <int NB>
+__device__ __forceinline__ void transpose_blocks(float (&v)[4 * NB], int lane) {
 #pragma unroll
-        for (int e = 0; e < EC / 2; ++e) {
-            const __nv_bfloat162 h2 = *reinterpret_cast<const __nv_bfloat162*>(&src[e]);
-            o[2 * e] += __bfloat162float(h2.x);
-            o[2 * e + 1] += __bfloat162float(h2.y);
+    for (int st = 1; st < NB; st <<= 1) {
+        const bool up = lane & st;
+#pragma unroll
+        for (int b = 0; b < NB; ++b) {
+            if (b & st) continue;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const float got = __shfl_xor_sync(0xffffffffu, up ? v[4 * b + e] : v[4 * (b + st) + e], st);
+                if (up)
+                    v[4 * b + e] = got;
+                else
+                    v[4 * (b + st) + e] = got;
+            }
         }
     }
 }
 
-// WIDE: the values loaded ahead are FP32 (an FP32 added tensor and no residual input).
+// WIDE: the input-gradient form, y FP32, with an FP32 added tensor or none (and neither bias, activation
+// nor residual).  The added values are read and the results written a voxel's contiguous bytes at a time
+// (transpose_blocks): lane by lane, the four 16-byte accesses of a voxel miss each other in the L1 left
+// beside the shared memory, which is smaller than the lines in use (32 -> 32 at batch 4: 77 us against 165
+// with an added tensor, 59 against 89 without).  The bf16 form, bound by the instructions of its epilogue
+// (16 error functions a lane), gains nothing from it (111 us transposed, 98 lane by lane).
 template <int CIN, int COUT, bool WIDE>
 __global__ void __launch_bounds__(640, 1)
     k_conv_fwd_tcx(const __grid_constant__ CUtensorMap xrows, const __grid_constant__ CUtensorMap xrow, sg_shape s,
@@ -803,12 +859,20 @@ __global__ void __launch_bounds__(640, 1)
     // weights: B[g = 3 (dz+1) + (dy+1)][k8][n = 3-tap column dxi * cout + co][8 channels]
     //          <- w[co][tap = 3 g + dxi][k8 * 8 ..]
     unsigned char* Bw = smem + C::A_BYTES;
-    for (int i = tid; i < 27 * C::K8 * COUT; i += C::THREADS) {
-        const int co = i % COUT, r = i / COUT;
-        const int k8 = r % C::K8, tap = r / C::K8;
+    // read in their own order (contiguous), all of a thread's loads in flight
+    constexpr int kChunks = 27 * C::K8 * COUT, kPer = (kChunks + C::THREADS - 1) / C::THREADS;
+    uint4 wv[kPer];
+#pragma unroll
+    for (int j = 0; j < kPer; ++j)
+        if (tid + j * C::THREADS < kChunks) wv[j] = __ldg(reinterpret_cast<const uint4*>(w) + tid + j * C::THREADS);
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {
+        const int i = tid + j * C::THREADS;
+        if (i >= kChunks) break;
+        const int k8 = i % C::K8, r = i / C::K8;
+        const int tap = r % 27, co = r / 27;
         const int g = tap / 3, dxi = tap % 3;
-        *reinterpret_cast<uint4*>(Bw + (size_t)((g * C::K8 + k8) * C::N + dxi * COUT + co) * 16) =
-            *reinterpret_cast<const uint4*>(w + ((size_t)co * 27 + tap) * CIN + k8 * 8);
+        *reinterpret_cast<uint4*>(Bw + (size_t)((g * C::K8 + k8) * C::N + dxi * COUT + co) * 16) = wv[j];
     }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_holder)),
@@ -946,21 +1010,27 @@ __global__ void __launch_bounds__(640, 1)
         const int pair = half * 2 + yl, pw = quarter & 1;  // the two quarters of a row form a pair
         const bool seg = s.xper < kW;  // rows of independent periodic segments (within a quarter)
         // the residual input (or, without one, the added values) of a tile is loaded one tile of
-        // this group ahead: EC bf16 values in EC / 2 words, or EC FP32 values in EC words
+        // this group ahead
         const bool res = epi.res_in && CIN == COUT;
-        const bool pre_add = !res && epi.add;
+        const bool pre_add = !WIDE && !res && epi.add;
         const bool bias4 = bias && ((uintptr_t)bias & 15) == 0;
-        constexpr int XW = WIDE ? EC : EC / 2;  // 32-bit words loaded ahead
+        constexpr int XW = EC / 2;  // 32-bit words loaded ahead
         uint32_t nxt[XW];
         auto voxel_of = [&](const Run& R, int k) {
             return (((int64_t)R.b * s.nz + (R.z0 + k)) * s.ny + (R.y0 + yl)) * kW + xx;
         };
-        // EC bf16 values (EC / 2 words) or EC FP32 values (EC words) of voxel v: the residual input
-        // or the added tensor
-        auto extra_ptr = [&](int64_t v, bool is_res, bool f32) {
-            return is_res ? reinterpret_cast<const uint4*>(x + v * CIN + c_lo)
-                          : (f32 ? reinterpret_cast<const uint4*>(static_cast<const float*>(epi.add) + v * COUT + c_lo)
-                                 : reinterpret_cast<const uint4*>(static_cast<const bf16*>(epi.add) + v * COUT + c_lo));
+        auto out_voxel = [&](const Run& R, int k, int64_t v) {
+            return epi.lf == epi.lt ? v : relabelled_voxel(epi, R.b, R.z0 + k, R.y0 + yl, xx);
+        };
+        // what a tile loads ahead: the residual input's voxel or, in y's layout, the added tensor's
+        auto ahead = [&](const Run& R, int k) {
+            const int64_t v = voxel_of(R, k);
+            return res ? v : out_voxel(R, k, v);
+        };
+        // EC bf16 values (EC / 2 words) of voxel v: the residual input or the added tensor
+        auto extra_ptr = [&](int64_t v, bool is_res) {
+            return reinterpret_cast<const uint4*>(is_res ? x + v * CIN + c_lo
+                                                         : static_cast<const bf16*>(epi.add) + v * COUT + c_lo);
         };
         // the tiles of this group in order
         int64_t t = t0;
@@ -976,16 +1046,28 @@ __global__ void __launch_bounds__(640, 1)
             }
         };
         advance(grp);
-        if (t < t1 && (res || pre_add)) ld_words(extra_ptr(voxel_of(R, k), res, WIDE), nxt);
+        if (t < t1 && (res || pre_add)) ld_words(extra_ptr(ahead(R, k), res), nxt);
         uint32_t tt = (uint32_t)grp, use = 0;
         bool ok = true;
         while (t < t1 && ok) {
-            const int64_t v = voxel_of(R, k);
+            const int64_t v = voxel_of(R, k), vo = out_voxel(R, k, v);
             uint32_t cur[XW];
 #pragma unroll
             for (int i = 0; i < XW; ++i) cur[i] = nxt[i];
             advance(C::EPI_GROUPS);
-            if (t < t1 && (res || pre_add)) ld_words(extra_ptr(voxel_of(R, k), res, WIDE), nxt);
+            if (t < t1 && (res || pre_add)) ld_words(extra_ptr(ahead(R, k), res), nxt);
+
+            // WIDE: block j of the added values and of the results, EC / 4 lanes to a voxel
+            constexpr int NB = EC / 4;
+            const int64_t wide_at = (v - (lane & (NB - 1))) * COUT + c_lo + 4 * (lane & (NB - 1));
+            float4 wadd[WIDE ? NB : 1];
+            if constexpr (WIDE) {
+#pragma unroll
+                for (int j = 0; j < NB; ++j)
+                    wadd[j] = epi.add ? __ldg(reinterpret_cast<const float4*>(static_cast<const float*>(epi.add) + wide_at +
+                                                                              j * COUT))
+                                      : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
 
             const int acc = (int)(tt % C::NACC);
             const uint32_t au = tt / C::NACC;
@@ -1044,6 +1126,18 @@ __global__ void __launch_bounds__(640, 1)
 #pragma unroll
                 for (int e = 0; e < EC; ++e) zc[e] += xch[grp][pair][pw ^ 1][par][1][e];
             }
+            if constexpr (WIDE) {
+                transpose_blocks<NB>(zc, lane);
+                float* yo = static_cast<float*>(y) + wide_at;
+#pragma unroll
+                for (int j = 0; j < NB; ++j)
+                    *reinterpret_cast<float4*>(yo + j * COUT) =
+                        make_float4(zc[4 * j] + wadd[j].x, zc[4 * j + 1] + wadd[j].y, zc[4 * j + 2] + wadd[j].z,
+                                    zc[4 * j + 3] + wadd[j].w);
+                tt += C::EPI_GROUPS;
+                ++use;
+                continue;
+            }
             if (bias4) {
 #pragma unroll
                 for (int e = 0; e < EC / 4; ++e) {
@@ -1065,29 +1159,17 @@ __global__ void __launch_bounds__(640, 1)
             }
             if (res || pre_add) add_words(zc, cur);
             if (res && epi.add) {  // both a residual and an added tensor: the added one read here
-                if (epi.add_f32) {
-                    uint32_t ex[EC];
-                    ld_words(extra_ptr(v, false, true), ex);
-                    add_words(zc, ex);
-                } else {
-                    uint32_t ex[EC / 2];
-                    ld_words(extra_ptr(v, false, false), ex);
-                    add_words(zc, ex);
-                }
+                uint32_t ex[EC / 2];
+                ld_words(extra_ptr(vo, false), ex);
+                add_words(zc, ex);
             }
-            if (epi.y_f32) {
-                float4* yo = reinterpret_cast<float4*>(static_cast<float*>(y) + v * COUT + c_lo);
+            uint4 pk[EC / 8];
+            __nv_bfloat162* pp = reinterpret_cast<__nv_bfloat162*>(pk);
 #pragma unroll
-                for (int e = 0; e < EC / 4; ++e) yo[e] = make_float4(zc[4 * e], zc[4 * e + 1], zc[4 * e + 2], zc[4 * e + 3]);
-            } else {
-                uint4 pk[EC / 8];
-                __nv_bfloat162* pp = reinterpret_cast<__nv_bfloat162*>(pk);
+            for (int e = 0; e < EC / 2; ++e) pp[e] = __floats2bfloat162_rn(zc[2 * e], zc[2 * e + 1]);
+            uint4* yo = reinterpret_cast<uint4*>(static_cast<bf16*>(y) + vo * COUT + c_lo);
 #pragma unroll
-                for (int e = 0; e < EC / 2; ++e) pp[e] = __floats2bfloat162_rn(zc[2 * e], zc[2 * e + 1]);
-                uint4* yo = reinterpret_cast<uint4*>(static_cast<bf16*>(y) + v * COUT + c_lo);
-#pragma unroll
-                for (int h = 0; h < EC / 8; ++h) yo[h] = pk[h];
-            }
+            for (int h = 0; h < EC / 8; ++h) yo[h] = pk[h];
             tt += C::EPI_GROUPS;
             ++use;
         }
@@ -1496,7 +1578,7 @@ static int launch_fwd_tcx(sg_shape s, const void* x, const void* w, const float*
     const int64_t tiles = (int64_t)s.batch * (s.ny / 2) * s.nz;
     const int grid = (int)(tiles < grid_max ? tiles : grid_max);
     const long long wait_limit = 2000000000LL;  // ~1 s of SM clock per wait
-    const bool wide = !(epi.res_in && CIN == COUT) && epi.add && epi.add_f32;
+    const bool wide = epi.y_f32;  // sg_conv3d_fwd_f32: no bias, activation or residual, an FP32 added tensor
     auto kern = wide ? k_conv_fwd_tcx<CIN, COUT, true> : k_conv_fwd_tcx<CIN, COUT, false>;
     kern<<<grid, C::THREADS, C::SMEM, st>>>(rows, row, s, static_cast<const bf16*>(x), static_cast<const bf16*>(w),
                                             bias, epi, y, wait_limit);
@@ -1617,8 +1699,8 @@ static int launch_wgrad(sg_shape s, const void* x, const void* dz, float* dw, fl
         }
     }
     const int n = 27 * CIN * COUT;
-    k_wgrad_reduce<<<(n + 31) / 32, 256, 0, st>>>(CIN, COUT, parts, partials, dw);
-    if (db) k_bias_finish<<<1, 32 * COUT, 0, st>>>(bias_parts, COUT, bias_part, db);
+    k_wgrad_reduce<<<(n + 31) / 32 + (db ? (COUT + 7) / 8 : 0), 256, 0, st>>>(CIN, COUT, parts, partials, dw, bias_parts,
+                                                                           bias_part, db);
     return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
 
@@ -1639,6 +1721,25 @@ int sg_conv3d_fwd(sg_shape s, int cin, int cout, const void* x, const void* w, c
                   int res_in, const void* add, float* z_out, void* y, void* stream) {
     Epi e{act, res_in, add, 0, z_out, 0};
     if (!x || !w || !y || !shape_ok(s) || (res_in && cin != cout)) return -1;
+    cudaStream_t st = (cudaStream_t)stream;
+    if (cin == 16 && cout == 32) return launch_fwd<16, 32>(s, x, w, bias, e, y, st);
+    if (cin == 32 && cout == 32) return launch_fwd<32, 32>(s, x, w, bias, e, y, st);
+    if (cin == 32 && cout == 16) return launch_fwd<32, 16>(s, x, w, bias, e, y, st);
+    if (cin == 16 && cout == 16) return launch_fwd<16, 16>(s, x, w, bias, e, y, st);
+    return -1;
+}
+
+int sg_conv3d_fwd_to(sg_shape s, int cin, int cout, const void* x, const void* w, const float* bias, int act,
+                     int res_in, const void* add, float* z_out, void* y, int df, int dt, void* stream) {
+    auto log2_of = [](int d) { return d == 1 ? 0 : d == 2 ? 1 : d == 4 ? 2 : d == 8 ? 3 : -1; };
+    Epi e{act, res_in, add, 0, z_out, 0};
+    e.lf = log2_of(df);
+    e.lt = log2_of(dt);
+    if (!x || !w || !y || e.lf < 0 || e.lt < 0 || !shape_ok(s) || s.xper != kW / df || s.batch % (df * df) ||
+        (s.nz * df) % dt || (s.ny * df) % dt || (res_in && cin != cout) || x == y || (add && add == y))
+        return -1;
+    e.nzt = s.nz * df / dt;
+    e.nyt = s.ny * df / dt;
     cudaStream_t st = (cudaStream_t)stream;
     if (cin == 16 && cout == 32) return launch_fwd<16, 32>(s, x, w, bias, e, y, st);
     if (cin == 32 && cout == 32) return launch_fwd<32, 32>(s, x, w, bias, e, y, st);
@@ -1682,7 +1783,13 @@ int sg_status(void* stream) {
 int sg_act_backward(int64_t n, int act, const float* dy, const float* z, void* dz, void* stream) {
     if (n < 0 || !dy || !dz || (act == SG_ACT_GELU && !z)) return -1;
     if (n == 0) return 0;
-    k_act_bwd<<<(unsigned)((n + 255) / 256), 256, 0, (cudaStream_t)stream>>>(n, act, dy, z, static_cast<bf16*>(dz));
+    auto aligned = [](const void* p, int to) { return (reinterpret_cast<uintptr_t>(p) & (uintptr_t)(to - 1)) == 0; };
+    if (aligned(dy, 16) && (act != SG_ACT_GELU || aligned(z, 16)) && aligned(dz, 8))
+        k_act_bwd<4><<<(unsigned)((n + 1023) / 1024), 256, 0, (cudaStream_t)stream>>>(n, act, dy, z,
+                                                                                     static_cast<bf16*>(dz));
+    else
+        k_act_bwd<1><<<(unsigned)((n + 255) / 256), 256, 0, (cudaStream_t)stream>>>(n, act, dy, z,
+                                                                                   static_cast<bf16*>(dz));
     return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
 

@@ -32,6 +32,8 @@ def _L():
         vp, i64, f32p = ctypes.c_void_p, ctypes.c_int64, ctypes.c_void_p
         sig = {
             "sg_conv3d_fwd": [SgShape, ctypes.c_int, ctypes.c_int, vp, vp, vp, ctypes.c_int, ctypes.c_int, vp, vp, vp, vp],
+            "sg_conv3d_fwd_to": [SgShape, ctypes.c_int, ctypes.c_int, vp, vp, vp, ctypes.c_int, ctypes.c_int, vp, vp,
+                                 vp, ctypes.c_int, ctypes.c_int, vp],
             "sg_conv3d_fwd_f32": [SgShape, ctypes.c_int, ctypes.c_int, vp, vp, vp, vp, vp],
             "sg_act_backward": [i64, ctypes.c_int, vp, vp, vp, vp],
             "sg_transpose_weights": [ctypes.c_int, ctypes.c_int, vp, vp, vp],
@@ -112,6 +114,16 @@ def conv3d_fwd(x, w, bias=None, act=ACT_NONE, res_in=False, add=None, z_out=None
         y = torch.empty(x.shape[:-1] + (cout,), dtype=torch.bfloat16, device=x.device)
     _ok(_L().sg_conv3d_fwd(s, cin, cout, _p(x), _p(w), _p(bias), act, int(res_in), _p(add), _p(z_out), _p(y),
                            _stream()), "sg_conv3d_fwd")
+    return y
+
+
+def conv3d_fwd_to(x, w, bias, act, res_in, natural, df, dt, add=None, z_out=None):
+    """conv3d_fwd on x in the df-layout of a volume of shape `natural`; the result (and add) in its
+    dt-layout, z_out in x's."""
+    cout, _, cin = w.shape
+    y = torch.empty(relabelled_shape(natural, dt)[:-1] + (cout,), dtype=torch.bfloat16, device=x.device)
+    _ok(_L().sg_conv3d_fwd_to(shape_of(x, 64 // df), cin, cout, _p(x), _p(w), _p(bias), act, int(res_in), _p(add),
+                              _p(z_out), _p(y), df, dt, _stream()), "sg_conv3d_fwd_to")
     return y
 
 

@@ -67,23 +67,19 @@ class Surrogate:
     def forward(self, x, train=False):
         """x: [B][nz][ny][64][16] BF16 -> prediction (BF16, same shape).  Keeps, for the backward
         pass, each layer's input (cache) and FP32 pre-activation (zs) in that layer's d-layout."""
-        nat = tuple(x.shape[:-1])
-        h, cur = x, 1
+        nat = tuple(x.shape)
+        h = x if self.dil[0] == 1 else sg.relabel(x, 1, self.dil[0], nat)
         self.cache, self.zs = [], []
         for k, (ci, co, act, res) in enumerate(LAYERS):
             d = self.dil[k]
-            if d != cur:
-                h = sg.relabel(h, cur, d, nat + (h.shape[-1],))
-                cur = d
             last = k == len(LAYERS) - 1
-            add = None
-            if last:
-                add = x if d == 1 else sg.relabel(x, 1, d, nat + (x.shape[-1],))
             z = torch.empty(h.shape[:-1] + (co,), dtype=torch.float32, device=x.device) if train else None
             self.cache.append(h)
-            h = sg.conv3d_fwd(h, self.w16[k], self.b32[k], act=act, res_in=res, add=add, z_out=z, xper=64 // d)
+            # each layer writes its output in the next one's layout, the last one in x's
+            h = sg.conv3d_fwd_to(h, self.w16[k], self.b32[k], act, res, nat, d, 1 if last else self.dil[k + 1],
+                                 add=x if last else None, z_out=z)
             self.zs.append(z)
-        return h if cur == 1 else sg.relabel(h, cur, 1, nat + (h.shape[-1],))
+        return h
 
     def backward(self, dpred, scratch_w, trace=None):
         """Gradients of all weights and biases from dL/dpred (FP32, [..][16], natural layout).  If
