@@ -676,6 +676,13 @@ __device__ __forceinline__ uint64_t umma_desc_sw32(uint32_t saddr) {
            (6ull << 61);
 }
 
+// Shared-memory descriptor of a 64-byte-swizzled K-major operand: 8-row atoms of 512 B (SBO), layout
+// type 4; a 16-channel slice of the 32-channel rows is a start address 32 bytes further on.
+__device__ __forceinline__ uint64_t umma_desc_sw64(uint32_t saddr) {
+    return (uint64_t)((saddr & 0x3FFFF) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)(512 >> 4) << 32) | (1ull << 46) |
+           (4ull << 61);
+}
+
 __device__ __forceinline__ void tp_arrive(uint32_t bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
@@ -714,8 +721,9 @@ __device__ __forceinline__ void tp_tma5(uint32_t dst, const CUtensorMap* map, in
 // Work: the tiles, numbered z fastest within a column (batch item, row pair),
 // are split into one contiguous range per CTA.  A run of consecutive z within
 // a column streams its planes z - 1 .. z_end through a ring of NSLOT plane
-// slots (each plane: all channel slices, 4 rows x 64 voxels, 32-byte-swizzled
-// K-major as TMA writes it), so tile k uses the slots of planes k, k + 1, k + 2.
+// slots (each plane: 4 rows x 64 voxels x all channels, K-major in the swizzle of
+// the voxel's 32 or 64 bytes, as TMA writes it; with 32 channels one 64-byte-swizzled
+// box, 96.0 us for 32 -> 32 at batch 4 against 98.4 as two 32-byte-swizzled slices), so tile k uses the slots of planes k, k + 1, k + 2.
 // Warp roles:
 //   warp 0     TMA producer (one box per slice and plane, one per row where the
 //              rows wrap around the periodic y boundary)
@@ -731,8 +739,8 @@ struct TcxCfg {
     static constexpr int K8 = CIN / 8;
     static constexpr int SL = CIN / 16;                  // 16-channel K slices
     static constexpr int HY = 4;                         // halo rows of a 2-row tile
-    static constexpr int SLICEB = HY * kW * 32;          // one slice of one plane: 8 KB
-    static constexpr int PLANE = SL * SLICEB;
+    static constexpr int ROWB = kW * CIN * 2;            // one row of one plane
+    static constexpr int PLANE = HY * ROWB;              // 8 or 16 KB
     static constexpr int N = 3 * COUT;                   // dx-stacked output columns
     static constexpr int GB = K8 * N * 16;               // weights of one (dz, dy)
     static constexpr int B_BYTES = 9 * GB;
@@ -872,7 +880,11 @@ __global__ void __launch_bounds__(640, 1)
         const int k8 = i % C::K8, r = i / C::K8;
         const int tap = r % 27, co = r / 27;
         const int g = tap / 3, dxi = tap % 3;
-        *reinterpret_cast<uint4*>(Bw + (size_t)((g * C::K8 + k8) * C::N + dxi * COUT + co) * 16) = wv[j];
+        const int n = dxi * COUT + co;
+        // 32 channels: rows n of 64 bytes, 64-byte swizzle; 16 channels: 8-row core matrices
+        const size_t at = CIN == 32 ? (size_t)(g * C::GB + n * 64 + 16 * (k8 ^ ((n >> 1) & 3)))
+                                    : (size_t)((g * C::K8 + k8) * C::N + n) * 16;
+        *reinterpret_cast<uint4*>(Bw + at) = wv[j];
     }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_holder)),
@@ -928,13 +940,10 @@ __global__ void __launch_bounds__(640, 1)
                 __syncwarp();
                 const uint32_t dst = a_s + (uint32_t)(slot * C::PLANE);
                 if (y_inside) {
-                    if (lane < C::SL)
-                        tp_tma5(dst + (uint32_t)(lane * C::SLICEB), &xrows, 16 * lane, 0, R.y0 - 1, zz, R.b,
-                                bar(LT + slot));
-                } else if (lane < C::SL * C::HY) {
-                    const int j = lane / C::HY, r = lane % C::HY;
-                    tp_tma5(dst + (uint32_t)(j * C::SLICEB + r * kW * 32), &xrow, 16 * j, 0, wrapi(R.y0 + r - 1, s.ny),
-                            zz, R.b, bar(LT + slot));
+                    if (lane == 0) tp_tma5(dst, &xrows, 0, 0, R.y0 - 1, zz, R.b, bar(LT + slot));
+                } else if (lane < C::HY) {
+                    tp_tma5(dst + (uint32_t)(lane * C::ROWB), &xrow, 0, 0, wrapi(R.y0 + lane - 1, s.ny), zz, R.b,
+                            bar(LT + slot));
                 }
                 __syncwarp();
             }
@@ -974,15 +983,18 @@ __global__ void __launch_bounds__(640, 1)
                 }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t d_tmem = tmem + (uint32_t)(acc * C::ACOLS);
-                const uint64_t a_pl[3] = {umma_desc_sw32(a_s + ((q + k) % C::NSLOT) * C::PLANE),
-                                          umma_desc_sw32(a_s + ((q + k + 1) % C::NSLOT) * C::PLANE),
-                                          umma_desc_sw32(a_s + ((q + k + 2) % C::NSLOT) * C::PLANE)};
-                const uint64_t b0 = umma_desc(b_s, C::N * 16, 128);
+                auto a_desc = [&](uint32_t slot) {
+                    const uint32_t at = a_s + slot * C::PLANE;
+                    return CIN == 32 ? umma_desc_sw64(at) : umma_desc_sw32(at);
+                };
+                const uint64_t a_pl[3] = {a_desc((q + k) % C::NSLOT), a_desc((q + k + 1) % C::NSLOT),
+                                          a_desc((q + k + 2) % C::NSLOT)};
+                const uint64_t b0 = CIN == 32 ? umma_desc_sw64(b_s) : umma_desc(b_s, C::N * 16, 128);
                 static_for<C::SL>([&](auto J) {
                     static_for<9>([&](auto G) {
                         constexpr int dz = G / 3, dy = G % 3;  // each + 1
-                        constexpr uint64_t aoff = (uint64_t)((J * C::SLICEB + dy * kW * 32) >> 4);
-                        constexpr uint64_t boff = (uint64_t)(((G * C::K8 + 2 * J) * C::N * 16) >> 4);
+                        constexpr uint64_t aoff = (uint64_t)((dy * C::ROWB + J * 32) >> 4);
+                        constexpr uint64_t boff = (uint64_t)((G * C::GB + J * 32) >> 4);
                         tc_mma_elect(d_tmem, a_pl[dz] + aoff, b0 + boff, C::IDESC, (J == 0 && G == 0) ? 0u : 1u);
                     });
                 });
@@ -1559,20 +1571,21 @@ static int launch_fwd_tcx(sg_shape s, const void* x, const void* w, const float*
     }
     auto encode = tensor_map_encoder();
     if (!encode) return -3;
-    // activations x[b][z][y][x][c] as a 5D tensor (c fastest); boxes of 16 channels (32 bytes, the
-    // swizzle span) x 64 voxels x 4 rows or x 1 row, written 32-byte swizzled
+    // activations x[b][z][y][x][c] as a 5D tensor (c fastest); boxes of all channels (32 or 64 bytes, the
+    // swizzle span) x 64 voxels x 4 rows or x 1 row
     const cuuint64_t dims[5] = {(cuuint64_t)CIN, (cuuint64_t)kW, (cuuint64_t)s.ny, (cuuint64_t)s.nz, (cuuint64_t)s.batch};
     const cuuint64_t strides[4] = {(cuuint64_t)CIN * 2, (cuuint64_t)kW * CIN * 2, (cuuint64_t)s.ny * kW * CIN * 2,
                                    (cuuint64_t)s.nz * s.ny * kW * CIN * 2};
     const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
     alignas(64) CUtensorMap rows, row;
-    const cuuint32_t box_rows[5] = {16, (cuuint32_t)kW, (cuuint32_t)C::HY, 1, 1};
-    const cuuint32_t box_row[5] = {16, (cuuint32_t)kW, 1, 1, 1};
+    const cuuint32_t box_rows[5] = {CIN, (cuuint32_t)kW, (cuuint32_t)C::HY, 1, 1};
+    const cuuint32_t box_row[5] = {CIN, (cuuint32_t)kW, 1, 1, 1};
+    const CUtensorMapSwizzle swz = CIN == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B;
     if (encode(&rows, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(x), dims, strides, box_rows, estr,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, swz, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS ||
         encode(&row, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(x), dims, strides, box_row, estr,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, swz, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return -3;
     const int64_t tiles = (int64_t)s.batch * (s.ny / 2) * s.nz;
