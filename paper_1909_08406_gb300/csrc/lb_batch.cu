@@ -124,13 +124,14 @@ __device__ __forceinline__ void batch_tile2(const BatchSim* __restrict__ sims, i
                                    S.tbf, err, s, z, y, x);
 }
 
-// Resident CTAs per SM the register allocation is sized for.  One node per thread in FP32
-// arithmetic fits 80 registers without spills (6 CTAs of 128 threads, 24 warps per SM); the
-// persistent kernel's loop state needs 96 (5 CTAs); two nodes per thread (packed FP32x2) and
-// FP64 arithmetic need about 168 (3 CTAs).
+// Resident CTAs per SM the register allocation is sized for.  One node per thread in FP32 arithmetic:
+// 80 registers without spills (6 CTAs of 128 threads, 24 warps per SM).  Two nodes per thread (packed
+// FP32x2): 128 registers (4 CTAs) in the one-step kernel, 168 (3) in the persistent one, which has the
+// loop's state besides and spills at 128 (24 FP32 grids of edges 32 to 128: 19.5 against 15.9 GMLUPS; FP16
+// 24.0 against 23.4).  FP64 arithmetic: 168 (3).
 template <class Codec, bool TWO>
 constexpr int batch_min_blocks(bool persistent) {
-    return sizeof(typename Codec::R) == 8 ? 3 : TWO ? 4 : 6;
+    return sizeof(typename Codec::R) == 8 || (TWO && persistent) ? 3 : TWO ? 4 : 6;
 }
 
 // Constants of the one-node and of the packed two-node update.
