@@ -5,14 +5,16 @@
 // Per step, from the post-collision state src:
 //   k_ni_density  rho of the streamed populations, sum_i f_i(x - c_i), and
 //                 mu_nid(rho), F_nid(rho) of each node
-//   k_ni_fields   per node: grad2 rho (3), lap F_nid and the isotropic part of I_ab,
-//                 -(1/2)|grad2 rho|^2 - rho lap rho
+//   k_ni_fields   per node: grad2 rho (3) and the scalar S whose gradient holds the force's isotropic
+//                 terms,
+//                   S = -F + (1 - eta) (theta_hat / 2) lap F + kappa [-(1/2)|grad2 rho|^2 - rho lap rho]
 //   k_ni_force    g^nid of Eq. (gradientFinal) at the node, from its stencil
 //                 neighbours' fields:
 //                   rho g = -[rho grad2 mu + mu grad2 rho - eta grad2 F
 //                             - (1 - eta) grad4 F + kappa grad2_b I_ab],
 //                   grad4 = grad2 - (theta_hat / 2) grad2 lap,
-//                   I_ab = [-(1/2)|grad rho|^2 - rho lap rho] delta_ab + grad_a rho grad_b rho
+//                   I_ab = [-(1/2)|grad rho|^2 - rho lap rho] delta_ab + grad_a rho grad_b rho,
+//                 which is -[rho grad2 mu + mu grad2 rho + grad2 S + kappa grad2_b (grad_a rho grad_b rho)]
 //   k_ni_step     the pull step with the forced BGK collision of
 //                 Eq. (multiphaseEvolution), alpha = 2: u = j / rho + g / 2,
 //                 f^eq = f^eq(rho, u, theta_0), F_i = g.(c_i - u)/theta_0 f^eq_i,
@@ -65,18 +67,14 @@ constexpr int kNiThreads = 128;
 // {u(2p), u(2p + 1), v(2p), v(2p + 1)}: an x pair (x even, nx even) reads both nodes' u and v
 // in one 16-byte load, and a warp's loads of 32 pairs are contiguous.
 //   RF = {rho, F_nid}, MU[q] = mu_nid                              (density pass)
-//   A = {mu_nid, F_nid}, B = {lap F_nid, iso}, C = {grad2_x rho, grad2_y rho},
-//   D[q] = grad2_z rho                                              (field pass)
-//   G[a n + q] = g^nid_a                                            (force pass)
-// with iso = -(1/2)|grad2 rho|^2 - rho lap rho, the isotropic part of I_ab.
+//   C = {grad2_x rho, grad2_y rho}, D = {grad2_z rho, S}           (field pass)
+//   G[a n + q] = g^nid_a                                           (force pass)
 template <class F>
 struct NiFields {
     F* RF;
-    F* A;
-    F* B;
     F* C;
-    F* MU;
     F* D;
+    F* MU;
     F* G;
 };
 
@@ -148,7 +146,8 @@ __global__ void __launch_bounds__(kNiThreads) k_ni_density(const typename Codec:
 
 // Every moving stencil term of a first derivative carries w_k c_ka / 2 = +-1/36 (sc-1: 1/36 x +-1,
 // bcc-1/2: 2/36 x +-1/2), so the passes sum the neighbours' values with signs and apply the weight
-// once; grad2 X = (1 / (36 theta_hat)) sum_k sgn(c_ka) X(x + c_k) over the k with c_ka != 0.
+// once; grad2 X = (1 / (36 theta_hat)) sum_k sgn(c_ka) (X(x + c_k) - X(x)) over the k with c_ka != 0.
+// The signs sum to zero; close values subtract exactly, so the differences round less than the values.
 constexpr double kGradScale = 1.0 / (36.0 * kHatTheta);
 
 // acc += v for sign > 0, acc -= v otherwise (the sign is a compile-time constant after unrolling).
@@ -158,34 +157,35 @@ __device__ __forceinline__ void add_signed(F& acc, F v, int sign) {
 }
 
 // The field pass at one node from its rho0, F0 and its neighbours' rn, Fn (in the order of
-// stencil()): grad2 rho, lap F_nid and iso.  The Laplacian sums the neighbours' differences from
-// the node, lap X = (2 / theta_hat) sum_k w_k (X(x + c_k) - X(x)) = (1/3) [sum_sc dX + 2 sum_bcc
-// dX], each difference formed before it is added (close values subtract exactly).
+// stencil()): grad2 rho and S.  lap X = (2 / theta_hat) sum_k w_k (X(x + c_k) - X(x)) = (1/3) [sum_sc dX +
+// 2 sum_bcc dX].
 template <class F>
-__device__ __forceinline__ void ni_fields_node(F r0, F F0, const F (&rn)[kStencil], const F (&Fn)[kStencil],
-                                               F (&g)[3], F& lapF, F& iso) {
+__device__ __forceinline__ void ni_fields_node(const NiEosT<F>& e, F r0, F F0, const F (&rn)[kStencil],
+                                               const F (&Fn)[kStencil], F (&g)[3], F& S) {
     F gsum[3] = {F(0), F(0), F(0)}, lr[2] = {F(0), F(0)}, lF[2] = {F(0), F(0)};
 #pragma unroll
     for (int k = 0; k < kStencil; ++k) {
         int cx, cy, cz;
         F w;
         stencil(k, cx, cy, cz, w);
-        if (cx) add_signed(gsum[0], rn[k], cx);
-        if (cy) add_signed(gsum[1], rn[k], cy);
-        if (cz) add_signed(gsum[2], rn[k], cz);
+        const F dr = rn[k] - r0;
+        if (cx) add_signed(gsum[0], dr, cx);
+        if (cy) add_signed(gsum[1], dr, cy);
+        if (cz) add_signed(gsum[2], dr, cz);
         const int sh = k < 6 ? 0 : 1;  // sc-1 or bcc-1/2
-        lr[sh] += rn[k] - r0;
+        lr[sh] += dr;
         lF[sh] += Fn[k] - F0;
     }
     const F gs = F(kGradScale);
     for (int b = 0; b < 3; ++b) g[b] = gsum[b] * gs;
     const F lap = F(1.0 / 3.0) * (lr[0] + F(2) * lr[1]);
-    iso = F(-0.5) * (g[0] * g[0] + g[1] * g[1] + g[2] * g[2]) - r0 * lap;
-    lapF = F(1.0 / 3.0) * (lF[0] + F(2) * lF[1]);
+    const F iso = F(-0.5) * (g[0] * g[0] + g[1] * g[1] + g[2] * g[2]) - r0 * lap;
+    const F lapF = F(1.0 / 3.0) * (lF[0] + F(2) * lF[1]);
+    S = fma((F(1) - e.eta) * F(0.5 * kHatTheta), lapF, e.kappa * iso) - F0;
 }
 
 template <class F>
-__global__ void __launch_bounds__(kNiThreads) k_ni_fields(Dims d, EntryGrid gr, NiFields<F> fl) {
+__global__ void __launch_bounds__(kNiThreads) k_ni_fields(Dims d, EntryGrid gr, NiEosT<F> e, NiFields<F> fl) {
     int s, z, y, x;
     const bool active = entry_node<kNode, true>(d, gr, s, z, y, x);
     pdl_begin();
@@ -199,71 +199,62 @@ __global__ void __launch_bounds__(kNiThreads) k_ni_fields(Dims d, EntryGrid gr, 
         rn[k] = fl.RF[ni_pair_at(nb[k], 0)];
         Fn[k] = fl.RF[ni_pair_at(nb[k], 1)];
     }
-    const F F0 = fl.RF[ni_pair_at(q, 1)];
-    F g[3], lapF, iso;
-    ni_fields_node<F>(fl.RF[ni_pair_at(q, 0)], F0, rn, Fn, g, lapF, iso);
-    fl.A[ni_pair_at(q, 0)] = fl.MU[q];
-    fl.A[ni_pair_at(q, 1)] = F0;
-    fl.B[ni_pair_at(q, 0)] = lapF;
-    fl.B[ni_pair_at(q, 1)] = iso;
+    F g[3], S;
+    ni_fields_node<F>(e, fl.RF[ni_pair_at(q, 0)], fl.RF[ni_pair_at(q, 1)], rn, Fn, g, S);
     fl.C[ni_pair_at(q, 0)] = g[0];
     fl.C[ni_pair_at(q, 1)] = g[1];
-    fl.D[q] = g[2];
+    fl.D[ni_pair_at(q, 0)] = g[2];
+    fl.D[ni_pair_at(q, 1)] = S;
 }
 
 // A stencil neighbour's fields as the force pass uses them.
 template <class F>
 struct NiNb {
-    F mu, Fe, lF, iso, g[3];
+    F mu, S, g[3];
 };
 
 // One stencil neighbour's terms of the force sums, k its stencil velocity (doubled c: sc-1 +-2
-// along one axis; bcc-1/2 +-1 along each).  With sgn(c_a) = c_a / |c_a|:
-//   dmu_a, dF_a, dlF_a += sgn(c_a) mu, F, lap F                                  (c_a != 0)
-//   divI_a += sum_b sgn(c_b) I_ab = grad_a rho sum_b sgn(c_b) grad_b rho + sgn(c_a) iso;
+// along one axis; bcc-1/2 +-1 along each), o the node itself.  With sgn(c_a) = c_a / |c_a|:
+//   dmu_a, t_a += sgn(c_a) (mu - mu_0), sgn(c_a) (S - S_0)                        (c_a != 0)
+//   tau_a += sum_b sgn(c_b) grad_a rho grad_b rho;
 // each sum times 1 / (36 theta_hat) is the grad2 of Appendix A.
 template <class F>
 struct NiForceSums {
-    F dmu[3], dF[3], dlF[3], divI[3];
+    F dmu[3], dS[3], tau[3];
 };
 template <class F>
 __device__ __forceinline__ void ni_sums_zero(NiForceSums<F>& a) {
-    for (int b = 0; b < 3; ++b) a.dmu[b] = a.dF[b] = a.dlF[b] = a.divI[b] = F(0);
+    for (int b = 0; b < 3; ++b) a.dmu[b] = a.dS[b] = a.tau[b] = F(0);
 }
 template <class F>
-__device__ __forceinline__ void ni_force_term(NiForceSums<F>& a, int k, const NiNb<F>& v) {
+__device__ __forceinline__ void ni_force_term(NiForceSums<F>& a, int k, const NiNb<F>& v, F mu0, F S0) {
     int cc[3];
     F w;
     stencil(k, cc[0], cc[1], cc[2], w);
+    const F dmu = v.mu - mu0, dS = v.S - S0;
     F cg = F(0);  // sum_b sgn(c_b) grad_b rho
     bool first = true;
     for (int b = 0; b < 3; ++b) {
         if (cc[b] == 0) continue;
-        add_signed(a.dmu[b], v.mu, cc[b]);
-        add_signed(a.dF[b], v.Fe, cc[b]);
-        add_signed(a.dlF[b], v.lF, cc[b]);
+        add_signed(a.dmu[b], dmu, cc[b]);
+        add_signed(a.dS[b], dS, cc[b]);
         if (first)
             cg = cc[b] > 0 ? v.g[b] : -v.g[b];
         else
             add_signed(cg, v.g[b], cc[b]);
         first = false;
     }
-    for (int b = 0; b < 3; ++b) {
-        a.divI[b] = fma(v.g[b], cg, a.divI[b]);
-        if (cc[b]) add_signed(a.divI[b], v.iso, cc[b]);
-    }
+    for (int b = 0; b < 3; ++b) a.tau[b] = fma(v.g[b], cg, a.tau[b]);
 }
 
 // g^nid from the sums and the node's own rho, mu and grad2 rho:
-//   rho g = -[rho grad2 mu + mu grad2 rho - eta grad2 F - (1 - eta) grad4 F + kappa grad2_b I_ab].
+//   rho g = -[rho grad2 mu + mu grad2 rho + grad2 S + kappa grad2_b (grad_a rho grad_b rho)].
 template <class F>
 __device__ __forceinline__ void ni_force_finish(const NiEosT<F>& e, const NiForceSums<F>& a, F r0, F mu0,
                                                 const F (&g2r)[3], F (&g)[3]) {
     const F gs = F(kGradScale), inv_r0 = F(1) / r0;
     for (int b = 0; b < 3; ++b) {
-        const F g2mu = a.dmu[b] * gs, g2F = a.dF[b] * gs, g2lF = a.dlF[b] * gs;
-        const F g4F = g2F - F(0.5 * kHatTheta) * g2lF;
-        const F rg = -(r0 * g2mu + mu0 * g2r[b] - e.eta * g2F - (F(1) - e.eta) * g4F + e.kappa * a.divI[b] * gs);
+        const F rg = -(r0 * (a.dmu[b] * gs) + mu0 * g2r[b] + fma(e.kappa, a.tau[b], a.dS[b]) * gs);
         g[b] = rg * inv_r0;
     }
 }
@@ -279,18 +270,19 @@ __global__ void __launch_bounds__(kNiThreads) k_ni_force(Dims d, EntryGrid gr, N
     const uint32_t q = ni_index(d, s, z, y, x);
     uint32_t nb[kStencil];
     ni_neighbors(d, s, z, y, x, nb);
+    const F mu0 = fl.MU[q], S0 = fl.D[ni_pair_at(q, 1)];
     NiForceSums<F> a;
     ni_sums_zero(a);
 #pragma unroll
     for (int k = 0; k < kStencil; ++k) {
         const uint32_t m = nb[k];
-        const NiNb<F> v{fl.A[ni_pair_at(m, 0)], fl.A[ni_pair_at(m, 1)], fl.B[ni_pair_at(m, 0)],
-                        fl.B[ni_pair_at(m, 1)], {fl.C[ni_pair_at(m, 0)], fl.C[ni_pair_at(m, 1)], fl.D[m]}};
-        ni_force_term<F>(a, k, v);
+        const NiNb<F> v{fl.MU[m], fl.D[ni_pair_at(m, 1)],
+                        {fl.C[ni_pair_at(m, 0)], fl.C[ni_pair_at(m, 1)], fl.D[ni_pair_at(m, 0)]}};
+        ni_force_term<F>(a, k, v, mu0, S0);
     }
-    const F g2r[3] = {fl.C[ni_pair_at(q, 0)], fl.C[ni_pair_at(q, 1)], fl.D[q]};
+    const F g2r[3] = {fl.C[ni_pair_at(q, 0)], fl.C[ni_pair_at(q, 1)], fl.D[ni_pair_at(q, 0)]};
     F g[3];
-    ni_force_finish<F>(e, a, fl.RF[ni_pair_at(q, 0)], fl.A[ni_pair_at(q, 0)], g2r, g);
+    ni_force_finish<F>(e, a, fl.RF[ni_pair_at(q, 0)], mu0, g2r, g);
     const size_t n = 2 * (size_t)d.plane;
     for (int b = 0; b < 3; ++b) fl.G[b * n + q] = g[b];
 }
@@ -347,15 +339,14 @@ struct alignas(2 * sizeof(F)) NiDuo {
 };
 
 template <class F, int S>
-__device__ __forceinline__ void ni_fields_pair(const Dims& d, const NiFields<F>& fl, int z, int y, int x, uint32_t q) {
+__device__ __forceinline__ void ni_fields_pair(const Dims& d, const NiEosT<F>& e, const NiFields<F>& fl, int z, int y, int x, uint32_t q) {
     uint32_t p[kPairPos];
     ni_pair_positions<S>(d, z, y, x, q, p);
     const NiQuad<F>* RF = reinterpret_cast<const NiQuad<F>*>(fl.RF);
     NiQuad<F> rf[kPairPos];
 #pragma unroll
     for (int i = 0; i < kPairPos; ++i) rf[i] = RF[p[i]];
-    const NiDuo<F> mu = *reinterpret_cast<const NiDuo<F>*>(fl.MU + q);
-    F g[2][3], lapF[2], iso[2];
+    F g[2][3], S_[2];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         F rn[kStencil], Fn[kStencil];
@@ -365,27 +356,25 @@ __device__ __forceinline__ void ni_fields_pair(const Dims& d, const NiFields<F>&
             rn[k] = quad_at(rf[src >> 1], 0, src & 1);
             Fn[k] = quad_at(rf[src >> 1], 1, src & 1);
         }
-        ni_fields_node<F>(quad_at(rf[1], 0, h), quad_at(rf[1], 1, h), rn, Fn, g[h], lapF[h], iso[h]);
+        ni_fields_node<F>(e, quad_at(rf[1], 0, h), quad_at(rf[1], 1, h), rn, Fn, g[h], S_[h]);
     }
     const uint32_t pq = q >> 1;
-    reinterpret_cast<NiQuad<F>*>(fl.A)[pq] = NiQuad<F>{mu.x, mu.y, rf[1].z, rf[1].w};
-    reinterpret_cast<NiQuad<F>*>(fl.B)[pq] = NiQuad<F>{lapF[0], lapF[1], iso[0], iso[1]};
     reinterpret_cast<NiQuad<F>*>(fl.C)[pq] = NiQuad<F>{g[0][0], g[1][0], g[0][1], g[1][1]};
-    *reinterpret_cast<NiDuo<F>*>(fl.D + q) = NiDuo<F>{g[0][2], g[1][2]};
+    reinterpret_cast<NiQuad<F>*>(fl.D)[pq] = NiQuad<F>{g[0][2], g[1][2], S_[0], S_[1]};
 }
 
 // k_ni_fields for an x pair.
 template <class F>
-__global__ void __launch_bounds__(kNiThreads) k_ni_fields2x(Dims d, EntryGrid gr, NiFields<F> fl) {
+__global__ void __launch_bounds__(kNiThreads) k_ni_fields2x(Dims d, EntryGrid gr, NiEosT<F> e, NiFields<F> fl) {
     int s, z, y, x;
     const bool active = entry_node<kPair, true>(d, gr, s, z, y, x);
     pdl_begin();
     if (!active) return;
     const uint32_t q = ni_index(d, s, z, y, x);
     if (s)
-        ni_fields_pair<F, 1>(d, fl, z, y, x, q);
+        ni_fields_pair<F, 1>(d, e, fl, z, y, x, q);
     else
-        ni_fields_pair<F, 0>(d, fl, z, y, x, q);
+        ni_fields_pair<F, 0>(d, e, fl, z, y, x, q);
 }
 
 template <class F, int S>
@@ -393,18 +382,16 @@ __device__ __forceinline__ void ni_force_pair(const Dims& d, const NiEosT<F>& e,
                                               int x, uint32_t q) {
     uint32_t p[kPairPos];
     ni_pair_positions<S>(d, z, y, x, q, p);
-    const NiQuad<F>* A = reinterpret_cast<const NiQuad<F>*>(fl.A);
-    const NiQuad<F>* B = reinterpret_cast<const NiQuad<F>*>(fl.B);
     const NiQuad<F>* C = reinterpret_cast<const NiQuad<F>*>(fl.C);
-    const NiDuo<F>* D = reinterpret_cast<const NiDuo<F>*>(fl.D);
-    NiQuad<F> qa[kPairPos], qb[kPairPos], qc[kPairPos];
-    NiDuo<F> qd[kPairPos];
+    const NiQuad<F>* D = reinterpret_cast<const NiQuad<F>*>(fl.D);
+    const NiDuo<F>* MU = reinterpret_cast<const NiDuo<F>*>(fl.MU);
+    NiQuad<F> qc[kPairPos], qd[kPairPos];
+    NiDuo<F> qm[kPairPos];
 #pragma unroll
     for (int i = 0; i < kPairPos; ++i) {
-        qa[i] = A[p[i]];
-        qb[i] = B[p[i]];
         qc[i] = C[p[i]];
         qd[i] = D[p[i]];
+        qm[i] = MU[p[i]];
     }
     NiForceSums<F> a[2];
     ni_sums_zero(a[0]);
@@ -414,26 +401,28 @@ __device__ __forceinline__ void ni_force_pair(const Dims& d, const NiEosT<F>& e,
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const int src = ni_pair_src<S>(h, k), i = src >> 1, c = src & 1;
-            const NiNb<F> v{quad_at(qa[i], 0, c), quad_at(qa[i], 1, c), quad_at(qb[i], 0, c), quad_at(qb[i], 1, c),
-                            {quad_at(qc[i], 0, c), quad_at(qc[i], 1, c), c ? qd[i].y : qd[i].x}};
-            ni_force_term<F>(a[h], k, v);
+            const NiNb<F> v{c ? qm[i].y : qm[i].x, quad_at(qd[i], 1, c),
+                            {quad_at(qc[i], 0, c), quad_at(qc[i], 1, c), quad_at(qd[i], 0, c)}};
+            ni_force_term<F>(a[h], k, v, h ? qm[1].y : qm[1].x, quad_at(qd[1], 1, h));
         }
     }
     const NiQuad<F> rf = reinterpret_cast<const NiQuad<F>*>(fl.RF)[q >> 1];
     F g[2][3];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-        const F g2r[3] = {quad_at(qc[1], 0, h), quad_at(qc[1], 1, h), h ? qd[1].y : qd[1].x};
-        ni_force_finish<F>(e, a[h], quad_at(rf, 0, h), quad_at(qa[1], 0, h), g2r, g[h]);
+        const F g2r[3] = {quad_at(qc[1], 0, h), quad_at(qc[1], 1, h), quad_at(qd[1], 0, h)};
+        ni_force_finish<F>(e, a[h], quad_at(rf, 0, h), h ? qm[1].y : qm[1].x, g2r, g[h]);
     }
     const size_t n = 2 * (size_t)d.plane;
     for (int b = 0; b < 3; ++b) *reinterpret_cast<NiDuo<F>*>(fl.G + b * n + q) = NiDuo<F>{g[0][b], g[1][b]};
 }
 
-// k_ni_force for an x pair.  80 registers (6 blocks per SM), without spills: 2.86 against 2.92 ms
-// for the 256^3 step at 128 registers (4 blocks).
+// k_ni_force for an x pair.  Bound by the L1 traffic of its 15 pairs and the latency of the loads: five
+// values of a neighbour instead of seven (mu, F, lap F, iso and the gradient apart) take the 160 x 200 x 200
+// step with FP16 storage from 0.99 to 0.92 ms, FP32 from 1.30 to 1.23.  64 registers (8 blocks per SM),
+// without spills: 1.180 ms for the 256 x 256 x 128 step, against 1.186 with 80 (6 blocks).
 template <class F>
-__global__ void __launch_bounds__(kNiThreads, 6) k_ni_force2x(Dims d, EntryGrid gr, NiEosT<F> e, NiFields<F> fl) {
+__global__ void __launch_bounds__(kNiThreads, 8) k_ni_force2x(Dims d, EntryGrid gr, NiEosT<F> e, NiFields<F> fl) {
     int s, z, y, x;
     const bool active = entry_node<kPair, true>(d, gr, s, z, y, x);
     pdl_begin();
@@ -596,9 +585,9 @@ static cudaError_t ni_codec(int prec, F&& f) {
     }
 }
 
-// The field arrays RF, A, B, C (2 values per node each), MU, D (1) and G (3), in the field type.
+// The field arrays RF, C, D (2 values per node each), MU (1) and G (3), in the field type.
 size_t nonideal_doubles(const Dims& d, int prec) {
-    const size_t values = (size_t)13 * 2 * d.plane;
+    const size_t values = (size_t)10 * 2 * d.plane;
     return prec == kF64 ? values : (values + 1) / 2;
 }
 
@@ -614,16 +603,14 @@ cudaError_t launch_nonideal_step(int prec, const void* src, void* dst, const Dim
         using R = typename C::R;
         const Consts<R>* K = &consts_of<C>(c);
         const NiEosT<R> e = ni_eos_in<R>(e64);
-        // field arrays in the compute type: RF, A, B, C (2 values per node each; 16-byte aligned, n
-        // is even), then MU, D (1) and G (3)
+        // field arrays in the compute type: RF, C, D (2 values per node each; 16-byte aligned, n
+        // is even), then MU (1) and G (3)
         NiFields<R> fl;
         fl.RF = reinterpret_cast<R*>(work);
-        fl.A = fl.RF + 2 * n;
-        fl.B = fl.A + 2 * n;
-        fl.C = fl.B + 2 * n;
-        fl.MU = fl.C + 2 * n;
-        fl.D = fl.MU + n;
-        fl.G = fl.D + n;
+        fl.C = fl.RF + 2 * n;
+        fl.D = fl.C + 2 * n;
+        fl.MU = fl.D + 2 * n;
+        fl.G = fl.MU + n;
         const auto* in = static_cast<const typename C::raw_t*>(src);
         auto* out = static_cast<typename C::raw_t*>(dst);
         // x pairs with nx even: the gathering passes with 16-bit storage, the stencil passes with FP32 fields
@@ -645,13 +632,13 @@ cudaError_t launch_nonideal_step(int prec, const void* src, void* dst, const Dim
         bool fields = false;
         if constexpr (sizeof(R) == 4) {
             if (even) {
-                if (!ok(launch_linear(k_ni_fields2x<R>, gp.entries, st, d, gp, fl)) ||
+                if (!ok(launch_linear(k_ni_fields2x<R>, gp.entries, st, d, gp, e, fl)) ||
                     !ok(launch_linear(k_ni_force2x<R>, gp.entries, st, d, gp, e, fl)))
                     return err_;
                 fields = true;
             }
         }
-        if (!fields && (!ok(launch_linear(k_ni_fields<R>, gn.entries, st, d, gn, fl)) ||
+        if (!fields && (!ok(launch_linear(k_ni_fields<R>, gn.entries, st, d, gn, e, fl)) ||
                         !ok(launch_linear(k_ni_force<R>, gn.entries, st, d, gn, e, fl))))
             return err_;
         if constexpr (kPairs) {
