@@ -1,7 +1,8 @@
 // FP32-arithmetic step kernels (FP32, FP16 and BF16 storage).  Variants:
 //   kKernelDirect1   k_step:        one node per thread, direct global loads
-//   kKernelDirect2   k_step2<.,.,3>: two rows per thread, packed FP32x2 math
-//   kKernelDirect2R  k_step2<.,.,4>: the same, register budget for 4 CTAs/SM
+//   kKernelDirect2   k_step2:       two rows per thread, packed FP32x2 math, register
+//                                   budget for 4 CTAs/SM
+//   kKernelDirect2R  k_step2:       the same, register budget for 3 CTAs/SM
 //   kKernelDirect2X, kKernelDirect2XL
 //                    k_step2x: two x-adjacent nodes per thread, 16-bit storage
 //   kKernelStaged    k_step_tma:    rows fetched by TMA bulk copies into a

@@ -840,8 +840,8 @@ __device__ __forceinline__ void transpose_blocks(float (&v)[4 * NB], int lane) {
 // WIDE: the input-gradient form, y FP32, with an FP32 added tensor or none (and neither bias, activation
 // nor residual).  The added values are read and the results written a voxel's contiguous bytes at a time
 // (transpose_blocks): lane by lane, the four 16-byte accesses of a voxel miss each other in the L1 left
-// beside the shared memory, which is smaller than the lines in use (32 -> 32 at batch 4: 77 us against 165
-// with an added tensor, 59 against 89 without).  The bf16 form, bound by the instructions of its epilogue
+// beside the shared memory, which is smaller than the lines in use (32 -> 32 at batch 4: 81 us against 165
+// with an added tensor, 60 against 89 without).  The bf16 form, bound by the instructions of its epilogue
 // (16 error functions a lane), gains nothing from it (111 us transposed, 98 lane by lane).
 template <int CIN, int COUT, bool WIDE>
 __global__ void __launch_bounds__(640, 1)
