@@ -82,8 +82,8 @@ __global__ void __launch_bounds__(Cfg::THREADS, Cfg::MINB) k_step_ws(const typen
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int tiles_per_row = d.nx / TX;
     const int nyh = d.ny >> 1;
-    const int64_t ntiles = d.rows / 2 * tiles_per_row;  // row pairs x tiles
-    const int64_t my_tiles = (int64_t)blockIdx.x < ntiles ? (ntiles - 1 - blockIdx.x) / gridDim.x + 1 : 0;
+    const int ntiles = (int)(d.rows / 2 * tiles_per_row);  // row pairs x tiles
+    const int my_tiles = (int)blockIdx.x < ntiles ? (ntiles - 1 - blockIdx.x) / gridDim.x + 1 : 0;
     const uint32_t nx = (uint32_t)d.nx, nxy = (uint32_t)d.nx * (uint32_t)d.ny;
     const uint32_t plane = (uint32_t)d.plane;
 
@@ -98,18 +98,18 @@ __global__ void __launch_bounds__(Cfg::THREADS, Cfg::MINB) k_step_ws(const typen
     __syncthreads();
 
     // tile t -> (s, z, y pair, x0)
-    auto coord = [&](int64_t t, int& s, int& z, int& y, int& x0) {
-        const int64_t rp = t / tiles_per_row;
+    auto coord = [&](int t, int& s, int& z, int& y, int& x0) {
+        const int rp = t / tiles_per_row;
         x0 = (int)(t - rp * tiles_per_row) * TX;
         y = 2 * (int)(rp % nyh);
-        const int64_t zr = rp / nyh;
+        const int zr = rp / nyh;
         z = (int)(zr % d.nz);
         s = (int)(zr / d.nz);
     };
 
     if (warp == 0) {
         // ---------------- producer ----------------
-        int64_t k = 0;
+        int k = 0;
         for (; k < my_tiles; ++k) {
             const int st = (int)(k % STAGES);
             const uint32_t n = (uint32_t)(k / STAGES);
@@ -167,16 +167,15 @@ __global__ void __launch_bounds__(Cfg::THREADS, Cfg::MINB) k_step_ws(const typen
         }
         // let every issued copy land before the CTA can exit (tiles k-STAGES+1 .. k-1 at most in flight)
         if (lane == 0) {
-            const int64_t first = k > STAGES ? k - STAGES : 0;
-            for (int64_t kk = first; kk < k; ++kk)
+            const int first = k > STAGES ? k - STAGES : 0;
+            for (int kk = first; kk < k; ++kk)
                 mbar_wait_bounded(smem_u32(&full[kk % STAGES]), (uint32_t)((kk / STAGES) & 1), wait_limit);
         }
     } else {
         // ---------------- consumers ----------------
         const int xl = tid - 32;
-        constexpr float inv_scale = (float)(1.0 / Codec::kScale);
         const F2 tbs(tb * (float)Codec::kScale), omb(1.f - tb);
-        for (int64_t k = 0; k < my_tiles; ++k) {
+        for (int k = 0; k < my_tiles; ++k) {
             const int st = (int)(k % STAGES);
             if (!mbar_wait_bounded(smem_u32(&full[st]), (uint32_t)((k / STAGES) & 1), wait_limit)) {
                 if (lane == 0) {
@@ -202,6 +201,10 @@ __global__ void __launch_bounds__(Cfg::THREADS, Cfg::MINB) k_step_ws(const typen
             };
             const NodeState<F2> ns = node_state<C2>(K, vget);
             if (!state_ok(ns)) atomicOr(err, 1);
+            // formed here, not before the sums: the tile number is all that stays live through them
+            int tile = (int)(blockIdx.x + k * gridDim.x);
+            asm volatile("" : "+r"(tile));
+            coord(tile, s, z, y, x0);
             T* outa = dst + (size_t)s * kQ * d.plane + ((uint32_t)z * nxy + (uint32_t)y * nx + (uint32_t)(x0 + xl));
             collide<C2, PROJECT>(ns, K, tbs, omb, vget, [&](auto I, F2 val) {
                 T* p = outa + (size_t)I * plane;
