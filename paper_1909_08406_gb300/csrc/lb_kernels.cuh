@@ -13,11 +13,46 @@ constexpr int kStepThreads = 128;
 // Load paths: the read-only (non-coherent) path for kernels whose inputs are complete before their
 // launch, ordinary loads for kernels that start before the kernel that writes their inputs has ended
 // (pdl_begin: a non-coherent load may be moved across the wait), and L2-coherent loads for
-// persistent kernels that read, after a grid barrier, what other CTAs wrote.
+// persistent kernels that read, after a grid barrier, what other CTAs wrote.  The last two must not be
+// moved across the wait or the barrier.  The intrinsics for the 32- and 64-bit types and for the unsigned
+// integers are volatile, those for __half, __nv_bfloat16 and their pairs are not (cuda_fp16.hpp,
+// cuda_bf16.hpp): the 16-bit types are loaded as integers of their size.
+template <class T>
+struct LoadWord {
+    using type = T;
+};
+template <>
+struct LoadWord<__half> {
+    using type = unsigned short;
+};
+template <>
+struct LoadWord<__nv_bfloat16> {
+    using type = unsigned short;
+};
+template <>
+struct LoadWord<__half2> {
+    using type = unsigned int;
+};
+template <>
+struct LoadWord<__nv_bfloat162> {
+    using type = unsigned int;
+};
+template <class T, class F>
+__device__ __forceinline__ T load_as_word(const T* p, F&& load) {
+    using W = typename LoadWord<T>::type;
+    static_assert(sizeof(W) == sizeof(T), "one word per value");
+    static_assert(std::is_same<W, float>::value || std::is_same<W, float2>::value || std::is_same<W, double>::value ||
+                      std::is_same<W, unsigned short>::value || std::is_same<W, unsigned int>::value,
+                  "a type whose load intrinsic is volatile");
+    const W w = load(reinterpret_cast<const W*>(p));
+    T v;
+    memcpy(&v, &w, sizeof v);
+    return v;
+}
 struct LoadCA {
     template <class T>
     static __device__ __forceinline__ T load(const T* p) {
-        return __ldca(p);
+        return load_as_word(p, [](auto* q) { return __ldca(q); });
     }
 };
 struct LoadNC {
@@ -29,7 +64,7 @@ struct LoadNC {
 struct LoadCG {
     template <class T>
     static __device__ __forceinline__ T load(const T* p) {
-        return __ldcg(p);
+        return load_as_word(p, [](auto* q) { return __ldcg(q); });
     }
 };
 
