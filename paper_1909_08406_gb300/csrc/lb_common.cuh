@@ -213,12 +213,28 @@ __device__ __forceinline__ F2& operator+=(F2& a, F2 b) {
 using ::fma;  // keep the scalar overloads visible next to the F2 one
 __device__ __forceinline__ F2 fma(F2 a, F2 b, F2 c) { return F2(__ffma2_rn(a.v, b.v, c.v)); }
 
-// Reciprocals of the node scalars (1/rho, theta0/theta, ...).  FP64 keeps the IEEE
-// division; the FP32 paths use the hardware reciprocal approximation (within 2 ulp),
-// far below the FP32 rounding of the populations themselves.
+// Reciprocals of the node scalars (1/rho, theta0/theta, ...).  FP64 keeps the IEEE division.
+// recip: the FP32 hardware approximation (within 2 ulp), for what is evaluated once: initial states and
+// exported moments.
 __device__ __forceinline__ double recip(double x) { return 1.0 / x; }
 __device__ __forceinline__ float recip(float x) { return __fdividef(1.0f, x); }
 __device__ __forceinline__ F2 recip(F2 x) { return F2(__fdividef(1.0f, x.v.x), __fdividef(1.0f, x.v.y)); }
+// recip_step: for the time step, the approximation and one step of Newton's iteration, r + r (1 - x r).  The
+// approximation is biased near 1, where these numbers lie: mean relative error -1.1e-8 over [0.99, 1.01],
+// -1.5e-8 over [1, 1.001], which adds up linearly over the steps.  After the Newton step the mean, rms and
+// largest errors over 2^20 numbers are the rounded quotient's.  Error of h against 64 bits after 100 FP32
+// steps, 21 x 95 x 12: 5.2e-7 (2.3e-6 by the approximation); 33 x 18 x 20: 1.2e-6 (3.8e-6).  The time stays
+// within 0.6%: 512 x 512 x 256 with FP16 storage, ten steps, 44.45 ms (44.46), stochastic 150 x 110 x 90 BF16,
+// 20 steps, 2.054 ms (2.043).
+__device__ __forceinline__ double recip_step(double x) { return 1.0 / x; }
+__device__ __forceinline__ float recip_step(float x) {
+    const float r = recip(x);
+    return fmaf(r, fmaf(-x, r, 1.0f), r);
+}
+__device__ __forceinline__ F2 recip_step(F2 x) {
+    const F2 r = recip(x);
+    return fma(r, fma(-x, r, F2(1.0f)), r);
+}
 
 // A product rounded by itself (not contracted into a following addition).
 __device__ __forceinline__ double mul(double a, double b) { return a * b; }
@@ -431,7 +447,7 @@ __device__ __forceinline__ NodeState<R> state_from_sums(const NodeSums<R>& m, co
     NodeState<R> st;
     st.drho = m.drho;
     st.rho = R(1) + m.drho;
-    const R inv_rho = recip(st.rho);
+    const R inv_rho = recip_step(st.rho);
     st.ux = m.jx * inv_rho;
     st.uy = m.jy * inv_rho;
     st.uz = m.jz * inv_rho;
@@ -467,7 +483,7 @@ __device__ __forceinline__ void collide(const NodeState<typename Codec::R>& st,
     using R = typename Codec::R;
     constexpr bool kF = Codec::stores_f;
     const R eta = ISO ? R(0) : st.eta;
-    const R it1 = ISO ? R(1) : recip(R(1) + eta);                            // theta_0 / theta
+    const R it1 = ISO ? R(1) : recip_step(R(1) + eta);                       // theta_0 / theta
     const R it = ISO ? R(K.inv_theta0) : it1 * R(K.inv_theta0);              // 1 / theta
     const R usq = fma(st.ux, st.ux, fma(st.uy, st.uy, st.uz * st.uz));
     const R g = usq * it;
@@ -477,7 +493,7 @@ __device__ __forceinline__ void collide(const NodeState<typename Codec::R>& st,
         return fma(eta, fma(eta, fma(eta, R(c[3]), R(c[2])), R(c[1])), R(c[0]));
     };
     const R M2 = ISO ? cubic(K.m2) : mul(cubic(K.m2), r2);
-    const R A1 = (R(2.5) * M2) * recip(fma(R(2.5), M2, R(1)));
+    const R A1 = (R(2.5) * M2) * recip_step(fma(R(2.5), M2, R(1)));
     // A2 = 5 A1 (1 - M2) - (3 + M2' - 5 M2)
     const R A2 = fma(fma(R(-5), M2, R(5)), A1, fma(R(5), M2, fma(-cubic(K.m2p), r2, R(-3))));
     const R nga = (g * A1) * (it * R(-1.0 / 6.0));  // -g A1 / (6 theta)
