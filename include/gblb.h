@@ -240,8 +240,11 @@ lb_status lb_set_state(lb_ctx *ctx, const void *raw, int on_device);
  *   LB_KERNEL_DIRECT2XL the same kernel (it once prefetched rows into L2)
  *   LB_KERNEL_AUTO     DIRECT2XL for 16-bit storage with nx even, else DIRECT2 where
  *                      it applies, else DIRECT1 (the default)
- * The direct kernels give the same bits; a grid too small to fill the SMs with two
- * nodes per thread runs one node per thread under any of their names.
+ * The direct kernels give the same bits.  A kernel that is asked for by name and applies is
+ * the one that runs.  Where the choice is the library's, one node per thread (the kernel
+ * of DIRECT1) stands in for DIRECT2XL below 19456 cells, and for DIRECT2 below 38912 cells
+ * and, with FP32 storage, where nx is not a multiple of 32.  The stochastic store always takes
+ * DIRECT2XL's kernel with nx even.
  * A request that does not apply to the grid falls back to one that does. */
 #define LB_KERNEL_AUTO (-1)
 #define LB_KERNEL_DIRECT1 0
@@ -252,8 +255,10 @@ lb_status lb_set_state(lb_ctx *ctx, const void *raw, int on_device);
 #define LB_KERNEL_DIRECT2X 5
 #define LB_KERNEL_DIRECT2XL 6
 
-/* Kernel lb_step will run for this context (LB_KERNEL_DIRECT1 .. LB_KERNEL_DIRECT2XL;
- * with stochastic rounding on, the one that carries the stochastic store). */
+/* Kernel that lb_step resolves to for this context (LB_KERNEL_DIRECT1 .. LB_KERNEL_DIRECT2XL; with
+ * stochastic rounding on, the one that carries the stochastic store): the kernel that runs, but
+ * for the one-node stand-ins of the library's own choice described above, which keep the name of the
+ * kernel they stand in for. */
 int lb_step_variant(const lb_ctx *ctx);
 /* Request a step kernel (LB_KERNEL_*). */
 lb_status lb_set_step_kernel(lb_ctx *ctx, int kernel);

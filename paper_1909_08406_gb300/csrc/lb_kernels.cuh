@@ -417,9 +417,10 @@ __global__ void __launch_bounds__(kStepThreads, 4) k_step2x(const typename Codec
     });
 }
 
-// Entries that leave an SM fewer than this many warps run one node per thread instead (the same bits):
-// latency counts there, not work per thread (33 x 18 x 20 FP32: 2.7 against 3.4 us a step; FP16 pairs
-// already win at 28^3, 3.7 against 3.9, FP32 rows from 40^3, 6.3 against 6.9).
+// Entries that leave an SM fewer than this many warps: where the choice of the kernel is the library's, it
+// takes one node per thread there (the same bits), as latency counts, not work per thread.  Microseconds a
+// step, one node against two: FP16 pairs 2.39 to 2.69 at 12 x 6 x 6, 2.55 to 2.79 at 24 x 20 x 20, 3.52 to
+// 3.48 at 28^3, 4.68 to 3.59 at 40 x 30 x 30; FP32 rows 2.26 to 2.90, 2.48 to 2.92, 3.69 to 3.87, 4.43 to 4.18.
 constexpr int64_t kSms = 152;
 template <int KIND>
 inline bool few_entries(const Dims& d) {

@@ -28,11 +28,6 @@ static cudaError_t run_direct1(const void* src, void* dst, const Dims& d, const 
 template <class Codec, bool P, int MINB>
 static cudaError_t run_direct2(const void* src, void* dst, const Dims& d, const LaunchConsts& c, double twobeta,
                                int* err, cudaStream_t st) {
-    // FP32 rows that do not start on a 128-byte line: a warp's two row segments then touch twice as many
-    // partial lines, and one node per thread is faster (150 x 110 x 90: 142 against 160 us; at
-    // nx = 256 both run at the copy bandwidth)
-    const bool ragged = sizeof(typename Codec::raw_t) == 4 && d.nx % 32 != 0;
-    if (ragged || few_entries<kRows>(d)) return run_direct1<Codec, P>(src, dst, d, c, twobeta, err, st);
     return launch_entries<kRows>(wide_offsets(d) ? k_step2<Codec, P, MINB, true> : k_step2<Codec, P, MINB, false>,
                                  src, dst, d, st, pair_consts<Codec>(c), (float)twobeta, err);
 }
@@ -41,7 +36,6 @@ template <class Codec, bool P, bool SR = false>
 static cudaError_t run_direct2x(const void* src, void* dst, const Dims& d, const LaunchConsts& c, double twobeta,
                                 int* err, cudaStream_t st, uint32_t sr_key = 0) {
     if constexpr (sizeof(typename Codec::raw_t) == 2) {
-        if (few_entries<kPair>(d)) return run_direct1<Codec, P, SR>(src, dst, d, c, twobeta, err, st, sr_key);
         return launch_entries<kPair>(wide_offsets(d) ? k_step2x<Codec, P, true, SR> : k_step2x<Codec, P, false, SR>,
                                      src, dst, d, st, pair_consts<Codec>(c), (float)twobeta, err, sr_key);
     }
@@ -169,10 +163,24 @@ int resolve_kernel(int prec, const Dims& d, int kernel) {
     }
 }
 
+// The kernel that a step with the given request launches: a kernel asked for by name where it applies to the
+// grid, whatever the size.  Where the choice is the library's (kKernelAuto, or a request that does not
+// apply), one node per thread takes the place of two nodes per thread, with the same bits, on a grid with few
+// entries and, with FP32 storage, where the rows do not start on a 128-byte line: a warp's two row
+// segments then touch twice as many partial lines (150 x 110 x 90: 142 against 160 us; at nx = 256
+// both run at the copy bandwidth).
+static int launched_kernel(int prec, const Dims& d, int request) {
+    const int k = resolve_kernel(prec, d, request);
+    if (k == request) return k;
+    if (k == kKernelDirect2XL && few_entries<kPair>(d)) return kKernelDirect1;
+    if (k == kKernelDirect2 && (few_entries<kRows>(d) || (prec == kF32 && d.nx % 32 != 0))) return kKernelDirect1;
+    return k;
+}
+
 template <class Codec, bool P>
 static cudaError_t step_codec(int prec, int kernel, const void* src, void* dst, const Dims& d, const LaunchConsts& c,
                               double twobeta, int* err, cudaStream_t st) {
-    switch (resolve_kernel(prec, d, kernel)) {
+    switch (launched_kernel(prec, d, kernel)) {
         case kKernelStaged:
             if (tma_tile_width(prec, d) == 256)
                 return run_tma<Codec, P, typename TmaShape<Codec, 256>::Cfg>(src, dst, d, c, twobeta, err, st);
@@ -203,7 +211,7 @@ cudaError_t launch_step_f32(int prec, bool project, int kernel, const void* src,
 }
 
 // The fused step with the stochastic BF16 store (series equilibrium with the momentum projection):
-// the x-pair kernel where it applies, else one node per thread.
+// the x-pair kernel where it applies (whatever the size), else one node per thread.
 cudaError_t launch_step_sr(const void* src, void* dst, const Dims& d, const LaunchConsts& c, double twobeta, int* err,
                            cudaStream_t st, uint32_t sr_key) {
     if (resolve_kernel(kBF16, d, kKernelDirect2XL) == kKernelDirect2XL)
