@@ -653,11 +653,11 @@ __device__ __forceinline__ float scale_to_float(double d, float chi, float clo) 
     // the lower 29 bits in units of 2^(e - 1023 - 52)
     const float unit = __uint_as_float(sign | ((e - 896u - 52u) << 23));
     const float lo = __uint2float_rn(l & 0x1fffffffu) * unit;
-    const float p = hi * chi;
+    const float p = mul(hi, chi);  // rounded by itself: r holds what the rounding leaves
     float r = fmaf(hi, chi, -p);
     r = fmaf(hi, clo, r);
     r = fmaf(lo, chi, r);
-    return p + r;
+    return __fadd_rn(p, r);
 }
 
 // Raw storage <-> float64 populations for elements e in [e0, e0 + count) of the
