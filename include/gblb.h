@@ -262,7 +262,8 @@ lb_status lb_set_state(lb_ctx *ctx, const void *raw, int on_device);
 int lb_step_variant(const lb_ctx *ctx);
 /* Request a step kernel (LB_KERNEL_*). */
 lb_status lb_set_step_kernel(lb_ctx *ctx, int kernel);
-/* Autotuner: time every step kernel that applies to this grid for reps steps
+/* Autotuner: time every step kernel that applies to this grid (DIRECT2X and
+ * DIRECT2XL are one kernel, timed as DIRECT2XL) for reps steps
  * (the state is not advanced), keep the fastest, report it and its ms per step. */
 lb_status lb_tune(lb_ctx *ctx, int reps, int *kernel, double *ms_per_step);
 

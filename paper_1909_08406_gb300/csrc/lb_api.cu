@@ -368,6 +368,7 @@ lb_status lb_tune(lb_ctx* c, int reps, int* kernel_out, double* ms_out) {
     int best_k = resolve_kernel(c->prec, c->d, kKernelAuto);
     // trial steps read buf[cur] and write buf[1 - cur] without flipping: the state is unchanged
     for (int k = LB_KERNEL_DIRECT1; k <= LB_KERNEL_DIRECT2XL; ++k) {
+        if (k == kKernelDirect2X) continue;  // DIRECT2XL's kernel
         if (resolve_kernel(c->prec, c->d, k) != k) continue;
         cudaError_t e = launch_step(c->prec, c->eq, k, c->buf[c->cur], c->buf[1 - c->cur], c->d, lc, c->twobeta,
                                     c->d_err, c->stream);

@@ -33,7 +33,7 @@ LB_HALO = 2  # halo planes at each end of a padded z slab (lb_halo_pack)
 KERNEL_NAMES = {0: "k_step (direct, 1 node/thread)", 1: "k_step2 (direct, 2 rows/thread, FP32x2)",
                 2: "k_step2 (direct, 2 rows/thread, FP32x2, 3 CTAs/SM)", 3: "k_step_tma (TMA-staged)",
                 4: "k_step_ws (TMA-staged, warp-specialised, FP32x2)",
-                5: "k_step2x (direct, 2 x-adjacent nodes/thread, FP32x2, paired 16-bit access)",
+                5: "k_step2x (LB_KERNEL_DIRECT2X: the kernel of LB_KERNEL_DIRECT2XL)",
                 6: "k_step2x (direct, 2 x-adjacent nodes/thread, FP32x2, paired 16-bit access)"}
 
 
