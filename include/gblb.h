@@ -193,7 +193,7 @@ lb_status lb_halo_unpack(lb_ctx *ctx, int side, const void *buf);
  *   out          device pointer to 5 doubles (mass, momentum x/y/z, energy)
  *   cuda_stream  stream to enqueue on (NULL = legacy default stream)
  * Asynchronous: out is written by work enqueued on cuda_stream.  Its only
- * scratch is a fixed 160 KB array (4096 planes x 5 doubles) in the library's
+ * scratch is a fixed 18 KB array (456 partial sums x 5 doubles) in the library's
  * device memory, which every GPU that loads the library holds until the
  * process exits.  The first call on each device looks up that array's device
  * address (cudaGetSymbolAddress) with the device current; make that first
@@ -362,7 +362,8 @@ lb_status lb_nonideal_constants(int eos, double theta_star, double rho_c, double
  * synchronising call; the Carnahan-Starling form is checked only for
  * rho > 0 and finite moments.  An eos outside LB_EOS_* gives LB_ERR_ARG.
  * Needs the projected series equilibrium (no LB_FLAG_PAPER_LITERAL or
- * LB_FLAG_ENTROPIC; LB_ERR_ARG), fewer than 2^31 cells (LB_ERR_ARG), and
+ * LB_FLAG_ENTROPIC; LB_ERR_ARG), fewer than 2^31 cells (LB_ERR_ARG; from 2^30 cells, whose
+ * two state buffers exceed 280 GB, every step would be refused), and
  * neither walls nor stochastic rounding (LB_ERR_STATE).  Each step runs four kernels (density,
  * stencil fields, force, forced step); the work buffer holds 10 field values per node, 80 bytes
  * with FP64 storage and 40 otherwise.  A batch (lb_batch_step) refuses members with

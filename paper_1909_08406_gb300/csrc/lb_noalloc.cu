@@ -17,12 +17,14 @@
 
 namespace gblb {
 
-constexpr int kNoAllocMaxPlanes = 4096;  // 2 * nz must not exceed this
+constexpr int kNoAllocMaxPlanes = 4096;  // 2 * nz must not exceed this: the entry point's limit, from when the
+                                         // scratch held a sum per plane
+constexpr int kNoAllocSlots = 152 * 3;   // blocks of the summing kernel at most
 
 // Scratch shared by every call on a device: slot p holds the five FP64 sums of
 // block p.  Each call writes every slot it reads back, so nothing carries over
 // from an earlier call; calls that overlap on the GPU race on these slots.
-static __device__ __align__(256) double g_noalloc_partials[kNoAllocMaxPlanes * 5];
+static __device__ __align__(256) double g_noalloc_partials[kNoAllocSlots * 5];
 
 // Blocks of the summing kernel, each with one slot of the scratch: one wave on 152 SMs.
 template <class Codec>
@@ -47,7 +49,7 @@ template <class Codec>
 static void launch_noalloc_sums(const void* populations, const Dims& d, const Consts<typename Codec::R>& K,
                                 double theta0, double* partials, double* out, cudaStream_t st) {
     constexpr int nb = noalloc_blocks<Codec>();
-    static_assert(nb <= kNoAllocMaxPlanes, "one scratch slot per block");
+    static_assert(nb <= kNoAllocSlots, "one scratch slot per block");
     const auto* f = static_cast<const typename Codec::raw_t*>(populations);
     if (sum_vector_ok<Codec>(populations, d))
         k_conserved<Codec, sum_width<Codec>()><<<nb, kRedThreads, 0, st>>>(f, d, K, partials, 0, d.nz);
@@ -83,7 +85,7 @@ lb_status lb_conserved_noalloc(const void* populations, lb_grid grid, lb_precisi
     }
     if (2 * grid.nz > kNoAllocMaxPlanes) {
         g_noalloc_msg = "lb_conserved_noalloc: 2 * nz = " + std::to_string(2 * grid.nz) +
-                        " planes exceeds the fixed scratch of " + std::to_string(kNoAllocMaxPlanes) + " planes";
+                        " planes exceeds the limit of " + std::to_string(kNoAllocMaxPlanes) + " planes";
         return LB_ERR_ARG;
     }
     if ((int)precision < LB_F64 || (int)precision > LB_F32_S16B) {

@@ -170,7 +170,6 @@ __global__ void __launch_bounds__(Cfg::THREADS, Cfg::MINB) k_step_tma(const type
     if (producer)
         for (int64_t k = 0; k < STAGES - 1 && k < my_tiles; ++k) issue(k);
 
-    constexpr R inv_scale = R(1.0 / Codec::kScale);
     const R tbs = tb * R(Codec::kScale);
     const R omb = R(1) - tb;
     int64_t k = 0;
