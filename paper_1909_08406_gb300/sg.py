@@ -119,17 +119,17 @@ def conv3d_fwd(x, w, bias=None, act=ACT_NONE, res_in=False, add=None, z_out=None
 
 def conv3d_fwd_to(x, w, bias, act, res_in, natural, df, dt, add=None, z_out=None):
     """conv3d_fwd on x in the df-layout of a volume of shape `natural`; the result (and add) in its
-    dt-layout, z_out in x's.  ValueError for shapes that do not belong together: the kernel writes as many
+    dt-layout, z_out in x's.  RuntimeError for shapes that do not belong together: the kernel writes as many
     voxels as x has."""
     cout, _, cin = w.shape
     b, nz, ny, nx, _ = x.shape
     if (natural[0] * df * df, *natural[1:4]) != (b, nz * df, ny * df, nx):
-        raise ValueError(f"x of shape {tuple(x.shape)} is not the {df}-layout of a volume natural = {tuple(natural)}")
+        raise RuntimeError(f"x of shape {tuple(x.shape)} is not the {df}-layout of a volume natural = {tuple(natural)}")
     out = relabelled_shape(natural, dt)[:-1] + (cout,)
     if add is not None and tuple(add.shape) != out:
-        raise ValueError(f"add of shape {tuple(add.shape)}, the result has {out}")
+        raise RuntimeError(f"add of shape {tuple(add.shape)}, the result has {out}")
     if z_out is not None and tuple(z_out.shape) != tuple(x.shape[:-1]) + (cout,):
-        raise ValueError(f"z_out of shape {tuple(z_out.shape)} for x of shape {tuple(x.shape)}")
+        raise RuntimeError(f"z_out of shape {tuple(z_out.shape)} for x of shape {tuple(x.shape)}")
     y = torch.empty(out, dtype=torch.bfloat16, device=x.device)
     _ok(_L().sg_conv3d_fwd_to(shape_of(x, 64 // df), cin, cout, _p(x), _p(w), _p(bias), act, int(res_in), _p(add),
                               _p(z_out), _p(y), df, dt, _stream()), "sg_conv3d_fwd_to")
