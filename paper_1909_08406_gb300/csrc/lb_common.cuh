@@ -214,26 +214,31 @@ using ::fma;  // keep the scalar overloads visible next to the F2 one
 __device__ __forceinline__ F2 fma(F2 a, F2 b, F2 c) { return F2(__ffma2_rn(a.v, b.v, c.v)); }
 
 // Reciprocals of the node scalars (1/rho, theta0/theta, ...).  FP64 keeps the IEEE division.
-// recip: the FP32 hardware approximation (within 2 ulp), for what is evaluated once: initial states and
-// exported moments.
+// recip: the FP32 hardware approximation (within 2 ulp).
 __device__ __forceinline__ double recip(double x) { return 1.0 / x; }
 __device__ __forceinline__ float recip(float x) { return __fdividef(1.0f, x); }
 __device__ __forceinline__ F2 recip(F2 x) { return F2(__fdividef(1.0f, x.v.x), __fdividef(1.0f, x.v.y)); }
-// recip_step: for the time step, the approximation and one step of Newton's iteration, r + r (1 - x r).  The
-// approximation is biased near 1, where these numbers lie: mean relative error -1.1e-8 over [0.99, 1.01],
-// -1.5e-8 over [1, 1.001], which adds up linearly over the steps.  After the Newton step the mean, rms and
-// largest errors over 2^20 numbers are the rounded quotient's.  Error of h against 64 bits after 100 FP32
-// steps, 21 x 95 x 12: 5.2e-7 (2.3e-6 by the approximation); 33 x 18 x 20: 1.2e-6 (3.8e-6).  The time stays
-// within 0.6%: 512 x 512 x 256 with FP16 storage, ten steps, 44.45 ms (44.46), stochastic 150 x 110 x 90 BF16,
-// 20 steps, 2.054 ms (2.043).
-__device__ __forceinline__ double recip_step(double x) { return 1.0 / x; }
-__device__ __forceinline__ float recip_step(float x) {
+// recip_newton: the approximation and one step of Newton's iteration, r + r (1 - x r).  The approximation is
+// biased near 1, where these numbers lie: mean relative error -1.1e-8 over [0.99, 1.01], -1.5e-8 over [1, 1.001].
+// After the step the mean, rms and largest errors over 2^20 numbers are the rounded quotient's.
+__device__ __forceinline__ double recip_newton(double x) { return 1.0 / x; }
+__device__ __forceinline__ float recip_newton(float x) {
     const float r = recip(x);
     return fmaf(r, fmaf(-x, r, 1.0f), r);
 }
-__device__ __forceinline__ F2 recip_step(F2 x) {
+__device__ __forceinline__ F2 recip_newton(F2 x) {
     const F2 r = recip(x);
     return fma(r, fma(-x, r, F2(1.0f)), r);
+}
+// The reciprocals of rho and theta / theta0 in a time step with the codec's storage.  FP32 keeps the populations
+// to 2^-24, and the bias adds up over the steps: error of h against 64 bits after 100 steps, 21 x 95 x 12, 5.2e-7
+// with the Newton step, 2.3e-6 without; 33 x 18 x 20, 1.2e-6 and 3.8e-6; a 256^3 step takes 1.604 ms (1.593), a
+// 512^3 one 12.58 (12.58).  The rounding of 16-bit storage (2^-11, 2^-8) hides the bias: the errors are the
+// same with and without, and the Newton step would cost 5% of the BF16 step at 256^3 (1.119 against 1.063 ms)
+// and 2% of the stochastic one at 512^3.
+template <class Codec>
+__device__ __forceinline__ typename Codec::R recip_step(typename Codec::R x) {
+    return sizeof(typename Codec::raw_t) == 2 ? recip(x) : recip_newton(x);
 }
 
 // A product rounded by itself (not contracted into a following addition).
@@ -442,12 +447,12 @@ __device__ __forceinline__ NodeSums<typename Codec::R> node_sums(const StepConst
 }
 
 // Primitive variables from the shell sums: eta = (de / rho - u^2) / (3 theta_0).
-template <class R, class KS>
+template <class Codec, class R, class KS>
 __device__ __forceinline__ NodeState<R> state_from_sums(const NodeSums<R>& m, const StepConsts<KS>& K) {
     NodeState<R> st;
     st.drho = m.drho;
     st.rho = R(1) + m.drho;
-    const R inv_rho = recip_step(st.rho);
+    const R inv_rho = recip_step<Codec>(st.rho);
     st.ux = m.jx * inv_rho;
     st.uy = m.jy * inv_rho;
     st.uz = m.jz * inv_rho;
@@ -458,7 +463,7 @@ __device__ __forceinline__ NodeState<R> state_from_sums(const NodeSums<R>& m, co
 
 template <class Codec, class VGet>
 __device__ __forceinline__ NodeState<typename Codec::R> node_state(const StepConsts<typename Codec::KS>& K, VGet&& vget) {
-    return state_from_sums(node_sums<Codec>(K, vget), K);
+    return state_from_sums<Codec>(node_sums<Codec>(K, vget), K);
 }
 
 // Equilibrium (Eq. feqGenU3, with the optional momentum projection) and BGK relaxation of one node, in
@@ -483,7 +488,7 @@ __device__ __forceinline__ void collide(const NodeState<typename Codec::R>& st,
     using R = typename Codec::R;
     constexpr bool kF = Codec::stores_f;
     const R eta = ISO ? R(0) : st.eta;
-    const R it1 = ISO ? R(1) : recip_step(R(1) + eta);                       // theta_0 / theta
+    const R it1 = ISO ? R(1) : recip_step<Codec>(R(1) + eta);                // theta_0 / theta
     const R it = ISO ? R(K.inv_theta0) : it1 * R(K.inv_theta0);              // 1 / theta
     const R usq = fma(st.ux, st.ux, fma(st.uy, st.uy, st.uz * st.uz));
     const R g = usq * it;
@@ -493,7 +498,7 @@ __device__ __forceinline__ void collide(const NodeState<typename Codec::R>& st,
         return fma(eta, fma(eta, fma(eta, R(c[3]), R(c[2])), R(c[1])), R(c[0]));
     };
     const R M2 = ISO ? cubic(K.m2) : mul(cubic(K.m2), r2);
-    const R A1 = (R(2.5) * M2) * recip_step(fma(R(2.5), M2, R(1)));
+    const R A1 = (R(2.5) * M2) * recip(fma(R(2.5), M2, R(1)));
     // A2 = 5 A1 (1 - M2) - (3 + M2' - 5 M2)
     const R A2 = fma(fma(R(-5), M2, R(5)), A1, fma(R(5), M2, fma(-cubic(K.m2p), r2, R(-3))));
     const R nga = (g * A1) * (it * R(-1.0 / 6.0));  // -g A1 / (6 theta)

@@ -482,7 +482,7 @@ __device__ __forceinline__ NodeState<R> ni_state(const NodeSums<R>& m, R gx, R g
     NodeState<R> st;
     st.drho = m.drho;
     st.rho = R(1) + m.drho;
-    const R inv_rho = recip_step(st.rho);
+    const R inv_rho = recip_newton(st.rho);
     st.ux = fma(R(0.5), gx, m.jx * inv_rho);
     st.uy = fma(R(0.5), gy, m.jy * inv_rho);
     st.uz = fma(R(0.5), gz, m.jz * inv_rho);
@@ -547,7 +547,7 @@ __global__ void __launch_bounds__(kStepThreads) k_ni_density2x(const typename Co
 }
 
 // k_ni_step for an x pair (16-bit storage, nx even).  Bound by the latency of its arithmetic: 4 blocks per SM
-// (128 registers, 72 bytes of spills) take the 160 x 200 x 200 step from 1.04 to 0.99 ms against 3.
+// (128 registers, 76 bytes of spills) take the 160 x 200 x 200 step from 1.04 to 0.99 ms against 3.
 template <class Codec, bool WIDE>
 __global__ void __launch_bounds__(kStepThreads, 4) k_ni_step2x(const typename Codec::raw_t* src,
                                                                typename Codec::raw_t* dst, Dims d, EntryGrid g,
