@@ -243,8 +243,9 @@ lb_status lb_set_state(lb_ctx *ctx, const void *raw, int on_device);
  * The direct kernels give the same bits.  A kernel that is asked for by name and applies is
  * the one that runs.  Where the choice is the library's, one node per thread (the kernel
  * of DIRECT1) stands in for DIRECT2XL below 19456 cells, and for DIRECT2 below 38912 cells
- * and, with FP32 storage, where nx is not a multiple of 32.  The stochastic store always takes
- * DIRECT2XL's kernel with nx even.
+ * and, with FP32 storage, where nx is not a multiple of 32.  The stochastic store runs in the
+ * kernels of DIRECT2XL (nx even) and DIRECT1: in the former if it is asked for by name, else
+ * by the same choice.
  * A request that does not apply to the grid falls back to one that does. */
 #define LB_KERNEL_AUTO (-1)
 #define LB_KERNEL_DIRECT1 0

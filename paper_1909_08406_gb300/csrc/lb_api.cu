@@ -445,7 +445,7 @@ lb_status lb_step(lb_ctx* c, int64_t n) {
             CK(c, launch_nonideal_step(c->prec, c->buf[c->cur], c->buf[1 - c->cur], c->d, lc, c->twobeta,
                                        c->nonideal, c->ni_eos, c->d_ni, c->d_err, c->stream));
         else if (c->sr)
-            CK(c, launch_step_sr(c->buf[c->cur], c->buf[1 - c->cur], c->d, lc, c->twobeta, c->d_err, c->stream,
+            CK(c, launch_step_sr(c->variant, c->buf[c->cur], c->buf[1 - c->cur], c->d, lc, c->twobeta, c->d_err, c->stream,
                                  sr_step_key(c->sr_seed, c->sr_t++)));
         else if (c->walls)
             CK(c, launch_wall_step(c->prec, c->eq, c->variant, c->buf[c->cur], c->buf[1 - c->cur], c->d, lc,

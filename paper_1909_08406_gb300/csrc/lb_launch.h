@@ -74,7 +74,7 @@ cudaError_t launch_step(int prec, int eq, int variant, const void* src, void* ds
 
 // One fused step with the stochastic BF16 store (BF16 storage, series equilibrium with the
 // momentum projection, periodic grid); sr_key is the step key k_t of lb_common.cuh.
-cudaError_t launch_step_sr(const void* src, void* dst, const Dims& d, const LaunchConsts& c, double twobeta, int* err,
+cudaError_t launch_step_sr(int kernel, const void* src, void* dst, const Dims& d, const LaunchConsts& c, double twobeta, int* err,
                            cudaStream_t st, uint32_t sr_key);
 
 // Equilibrium of float64 fields for nodes [q0, q0 + count).

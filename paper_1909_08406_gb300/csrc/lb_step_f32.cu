@@ -210,11 +210,12 @@ cudaError_t launch_step_f32(int prec, bool project, int kernel, const void* src,
     }
 }
 
-// The fused step with the stochastic BF16 store (series equilibrium with the momentum projection):
-// the x-pair kernel where it applies (whatever the size), else one node per thread.
-cudaError_t launch_step_sr(const void* src, void* dst, const Dims& d, const LaunchConsts& c, double twobeta, int* err,
-                           cudaStream_t st, uint32_t sr_key) {
-    if (resolve_kernel(kBF16, d, kKernelDirect2XL) == kKernelDirect2XL)
+// The fused step with the stochastic BF16 store (series equilibrium with the momentum projection): the
+// x-pair kernel where it applies and is asked for by name or has enough entries, else one node per thread.
+cudaError_t launch_step_sr(int kernel, const void* src, void* dst, const Dims& d, const LaunchConsts& c, double twobeta,
+                           int* err, cudaStream_t st, uint32_t sr_key) {
+    const bool named = kernel == kKernelDirect2X || kernel == kKernelDirect2XL;
+    if (launched_kernel(kBF16, d, named ? kKernelDirect2XL : kKernelAuto) == kKernelDirect2XL)
         return run_direct2x<CodecBF16, true, true>(src, dst, d, c, twobeta, err, st, sr_key);
     return run_direct1<CodecBF16, true, true>(src, dst, d, c, twobeta, err, st, sr_key);
 }

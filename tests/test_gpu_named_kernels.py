@@ -77,11 +77,14 @@ def test_launched_kernel(shape, prec, kernel, want):
     assert len(names) == 1 and want in names[0], names
 
 
-@pytest.mark.parametrize("shape,want", [((16, 6, 5), PAIRS), ((13, 6, 5), ONE), ((150, 66, 5), PAIRS)])
-def test_launched_kernel_of_the_stochastic_store(shape, want):
+@pytest.mark.parametrize("shape,kernel,want", [((16, 6, 5), lb.LB_KERNEL_AUTO, ONE), ((16, 6, 5), lb.LB_KERNEL_DIRECT2XL, PAIRS),
+                                               ((16, 6, 5), lb.LB_KERNEL_DIRECT2X, PAIRS), ((13, 6, 5), lb.LB_KERNEL_DIRECT2XL, ONE),
+                                               ((150, 66, 5), lb.LB_KERNEL_AUTO, PAIRS), ((150, 66, 5), lb.LB_KERNEL_STAGED, PAIRS)])
+def test_launched_kernel_of_the_stochastic_store(shape, kernel, want):
     stream = torch.cuda.Stream()
     ctx = lb.lb_init(shape, 0.4, "bf16", stream=stream.cuda_stream)
     try:
+        lb.lb_set_step_kernel(ctx, kernel)
         lb.lb_set_stochastic_rounding(ctx, 5)
         names = _launched(ctx, stream.cuda_stream)
     finally:
@@ -89,10 +92,12 @@ def test_launched_kernel_of_the_stochastic_store(shape, want):
     assert len(names) == 1 and want in names[0], names
 
 
-def _run(shape, prec, kernel, fields, steps, flags):
+def _run(shape, prec, kernel, fields, steps, flags, seed=None):
     ctx = lb.lb_init(shape, 0.3, prec, flags=flags)
     try:
         lb.lb_set_step_kernel(ctx, kernel)
+        if seed is not None:
+            lb.lb_set_stochastic_rounding(ctx, seed)
         lb.lb_set_fields(ctx, *fields)
         lb.lb_step(ctx, steps)
         raw = torch.empty((2, 41, shape[2], shape[1], shape[0]), dtype=TORCH_DTYPE[prec], device="cuda")
@@ -113,3 +118,13 @@ def test_two_node_kernels_give_the_one_node_bits(shape, prec, flags):
     want = _run(shape, prec, lb.LB_KERNEL_DIRECT1, fields, 10, flags)
     for k in (lb.LB_KERNEL_AUTO, lb.LB_KERNEL_DIRECT2, lb.LB_KERNEL_DIRECT2R, lb.LB_KERNEL_DIRECT2X):
         assert torch.equal(_run(shape, prec, k, fields, 10, flags), want), (shape, prec, k)
+
+
+@pytest.mark.parametrize("shape", [(2, 2, 2), (16, 6, 5), (62, 4, 5), (262, 3, 2), (130, 9, 16)])
+def test_the_stochastic_pairs_give_the_one_node_bits(shape):
+    """Below the size from which the library takes x pairs: one node per thread (which
+    test_gpu_stochastic_rounding.py compares with the oracle there) against the pairs by name."""
+    fl = wl.random_fields(*shape, lb.lb_theta0(), seed=4, du=0.02, drho=0.02, dtheta=0.02)
+    fields = [fl[k].cuda() for k in ("rho", "u", "theta")]
+    want = _run(shape, "bf16", lb.LB_KERNEL_AUTO, fields, 10, 0, seed=77)
+    assert torch.equal(_run(shape, "bf16", lb.LB_KERNEL_DIRECT2XL, fields, 10, 0, seed=77), want)
