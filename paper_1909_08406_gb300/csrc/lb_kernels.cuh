@@ -381,7 +381,7 @@ __device__ __forceinline__ void keep_packed(typename Codec::pair_t (&pv)[kQ]) {
 // even), packed FP32x2 arithmetic; the two results of a plane are written with one 32-bit store.
 //
 // Bound by the latency of its dependent arithmetic at the warps that fit: 128 registers (4 blocks, 16
-// warps per SM, 24 bytes of spills); 33.5 GMLUPS on 256^3 with FP16 storage, 81% of the copy bandwidth
+// warps per SM, 24 bytes of spills); 32.9 GMLUPS on 256^3 with FP16 storage, 80% of the copy bandwidth
 // (a block per row chunk with the next row prefetched into L2: 32.2; 168 registers, 12 warps: 29.4).
 // SR: BF16 storage with the stochastic store of lb_common.cuh, step key sr_key (one word per
 // population and x pair).
